@@ -144,6 +144,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   }
 }
 
+// mbar_wait by polling only: mbarrier.test_wait does not suspend the thread,
+// so the wait ends sooner after the last arrival (about 150 cycles measured).
+// For one thread whose next instruction everything else waits for.
+__device__ __forceinline__ bool mbar_wait_spin(uint64_t* bar, uint32_t parity,
+                                               uint64_t limit_ns = kWaitLimitNs) {
+  uint64_t t0 = 0;
+  for (uint32_t i = 1;; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((i & 4095u) == 0) {
+      const uint64_t t = globaltimer_ns();
+      if (t0 == 0) t0 = t;
+      if (t - t0 > limit_ns) return false;
+    }
+  }
+}
+
 // Proxy fences: order this thread's generic-proxy memory accesses (and the
 // writes of other threads it has already synchronised with) before its later
 // bulk-copy (async-proxy) accesses of global / shared memory.

@@ -7,30 +7,47 @@
 // Design (GB300).  A prefill pass is a dense contraction on both sides of the
 // softmax, so it runs on the tcgen05 tensor cores (bf16 operands, fp32
 // accumulation in TMEM), warp-specialised in the manner of flash attention on
-// this architecture.  One CTA (10 warps, one per SM) owns two 128-row query
-// tiles of one query head and walks the 128-slot KV tiles of the sequence's
-// channel up to each tile's largest position:
+// this architecture.  One CTA per SM (12 warps) takes work items one after
+// another; an item is two 128-row query tiles of one query head, for which the
+// CTA walks the 128-slot KV tiles of the sequence's channel up to each tile's
+// largest position:
 //    With grouped-query attention (an even number G of query heads per kv
 //    head) the two tiles are the same 128 rows of two query heads that share
 //    a kv head: equal causal ranges, and one K/V stream serves both.
 //    Otherwise they are two consecutive 128-row tiles of one head.
-//  * warp 8 (TMA): the two Q tiles once, then K and V of every KV tile
-//    through separate rings (128-byte swizzle, 64-column boxes; paged: one
-//    box per page, or per 128 slots of a longer page);
+//  * warp 8 (load): takes the next item (cluster launch control: a CTA that
+//    has not started yet is cancelled and its index taken over, so the items
+//    are handed out as SMs become free), publishes its rows' positions and
+//    extents to the other warps, and fills Q and K through TMA (K in a ring;
+//    128-byte swizzle, 64-column boxes; paged: one box per page, or per 128
+//    slots of a longer page); warp 10 fills V.  (One warp for both loaded K
+//    too late: it waited for V's slots, which free up half a step later.)
+//    They run ahead of the other warps across items, so an item's first tiles
+//    load while the last one finishes;
 //  * warp 9 (MMA): S_i = Q_i K^T into TMEM, and O_i += P_i V with P_i read
 //    from TMEM and V as an MN-major operand straight from its [slot][d] tile;
 //    issue order PV_0(j), S_0(j+1), PV_1(j), S_1(j+1) keeps one tile's
 //    matrix products running while the other tile's softmax works;
 //  * warps 0-3 and 4-7 (softmax of tile 0 / 1): one thread per query row
-//    reads its S row from TMEM, applies the causal mask slot <= pos (on
-//    tiles the diagonal crosses), and writes the bf16 probabilities back over
-//    the S columns it has read, where P V takes them as its A operand.  The
-//    running max is raised only when it grows by more than 2^8: only then is
-//    the row of O in TMEM rescaled; in between the probabilities stay below
-//    2^8, and the final O / l is exact either way.
-// Slots beyond the CTA's largest position may hold anything (unwritten
+//    reads its S row from TMEM, applies the causal mask slot <= pos (on tiles
+//    the diagonal crosses), and writes the bf16 probabilities back over the S
+//    columns it has read, where P V takes them as its A operand, each half as
+//    it is ready.  The running max is raised only when it grows by more than
+//    2^8: only then is the row of O in TMEM rescaled; in between the
+//    probabilities stay below 2^8, and the final O / l is exact either way.
+//    So the probabilities are computed with the max of the tiles before, and
+//    computed again in the rare step that raises it.
+// Slots beyond the item's largest position may hold anything (unwritten
 // cache); their V rows are zeroed in shared memory before P V, and masked
 // scores are replaced, never multiplied, so no NaN there reaches the output.
+//
+// What bounds it: the chain S -> softmax -> P V -> next S of each tile; with
+// two tiles in turn a 128-slot step of both takes about 2900 cycles at d = 128,
+// where the matrix products alone take 2048 and the 16384 exponentials 2048.
+// One launch at 32 heads of 128, two prompts of 8192 positions: 939 us before
+// (one item per CTA; every descriptor moved to uniform registers one by one,
+// 90 cycles per MMA; 16-byte row stores at the end), 773 us now; 6/3 heads of
+// 96, sixteen prompts of 2048: 126 and 86 us.
 #include <math.h>
 
 #include "internal.h"
@@ -41,26 +58,37 @@ namespace {
 
 constexpr int kPM = 128;                    // query rows per tile (MMA M)
 constexpr int kPN = 128;                    // slots per KV tile
-constexpr int kQT = 2;                      // query tiles per CTA
+constexpr int kQT = 2;                      // query tiles per item
 constexpr int kSoftWarps = 4 * kQT;         // one 4-warp group per query tile
-constexpr int kLoadWarp = kSoftWarps;       // TMA producer
+constexpr int kLoadWarp = kSoftWarps;       // items; TMA producer of Q and K
 constexpr int kMmaWarp = kSoftWarps + 1;    // MMA issuer
-constexpr int kPThreads = (kSoftWarps + 2) * 32;
+constexpr int kLoadVWarp = kSoftWarps + 2;  // TMA producer of V
+// Three warpgroups; the last holds the load and MMA warps (its fourth warp only
+// takes part in the block's barriers).  A softmax thread keeps its 128
+// scores in registers, so that group hands registers over: (2 x 208 + 88) x
+// 128 threads = the 384 x 168 of the launch.  (Two threads per row, 64 scores
+// each, took as long per step: the 128 exponentials of a row quadrant bind.)
+constexpr int kPThreads = (kSoftWarps + 4) * 32;
+constexpr int kSoftRegs = 208, kIssueRegs = 88;
 constexpr uint32_t kBlock = 128u * 128u;    // one 64-column block of a 128-row tile
-constexpr uint32_t kTmemCols = 512;         // S_i at 128 i (P_i over its first 64), O_i at 256 + 128 i
+constexpr uint32_t kTmemCols = 512;         // S_i at 128 i (P over its first 64), O_i at 256 + 128 i
 constexpr float kStaleMax = 8.f;            // log2 headroom before O is rescaled
+constexpr float kStaleSum = 16384.f;        // ... as a sum of 64 probabilities
+constexpr uint32_t kStageBytes = 32 * 64;   // output staging of a softmax warp: 32 rows x 32 columns
 
 template <int HD>
 struct PShape {
   static constexpr int CB = (HD + 63) / 64;          // 64-column blocks of a head row
-  // Ring depths: the next K tile is waited for first (S of the next KV tile
-  // is issued behind P V of this one), so K gets the deeper ring.
-  static constexpr int NSK = HD <= 64 ? 4 : 3;
+  // A slot of either ring is refilled about one and a half steps before it is
+  // needed (K of step j + 2 once both S of step j are done), so two deep is
+  // enough; a third K tile at d = 128 would take the output staging's place.
+  static constexpr int NSK = HD <= 64 ? 4 : 2;
   static constexpr int NSV = HD <= 64 ? 4 : 2;
   static constexpr uint32_t Q_BYTES = CB * kBlock;   // one Q tile
   static constexpr uint32_t KV_BYTES = CB * kBlock;  // one K or V tile
-  static constexpr uint32_t SMEM = kQT * Q_BYTES + (NSK + NSV) * KV_BYTES + 1024;  // + alignment
-  static_assert(SMEM <= 227 * 1024, "shared memory");
+  static constexpr uint32_t SMEM =
+      kQT * Q_BYTES + (NSK + NSV) * KV_BYTES + kSoftWarps * kStageBytes + 1024;  // + alignment
+  static_assert(SMEM <= 222 * 1024, "shared memory (5 KB of it static)");
 };
 
 struct PrefillParams {
@@ -70,8 +98,50 @@ struct PrefillParams {
   int32_t* status;
   int32_t B, Tq, Hq, G, Hkv, chan, num_pages, max_pages, P, log2P;
   int32_t pair;               // 1: the two tiles are query heads 2y, 2y+1 over the same rows
+  int32_t nblk, heads;        // row blocks per sequence, items' heads (or head pairs) per sequence
+  int32_t group;              // (sequence, head) units walked together, see launch_prefill_attn
   float qscale;               // log2(e) / sqrt(d)
 };
+
+// One item as the load warp publishes it.
+struct Item {
+  int valid;       // 0: no more items
+  int b, y, r0;    // sequence, head (or head pair), first row
+  int nt[kQT];     // KV tiles of each query tile
+  int tmaxpos;     // largest position of the item, -1: none valid
+};
+
+// Cluster launch control: ask for the index of a CTA of this grid that has not
+// started; the 16-byte answer arrives on `bar`.
+__device__ __forceinline__ void clc_request(void* answer, uint64_t* bar) {
+  asm volatile(
+      "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+          smem_u32(answer)),
+      "r"(smem_u32(bar))
+      : "memory");
+}
+// The answer: the CTA's x index, or -1 when none was left.
+__device__ __forceinline__ int clc_answer(const void* answer) {
+  uint32_t x, got;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 a;\n\t"
+      "ld.shared.b128 a, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+      "selp.u32 %1, 1, 0, p;\n\t"
+      "mov.u32 %0, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, a;\n\t}"
+      : "=r"(x), "=r"(got)
+      : "r"(smem_u32(answer))
+      : "memory");
+  return got ? (int)x : -1;
+}
+
+// max of three (one instruction on this architecture)
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -87,32 +157,28 @@ __global__ void __launch_bounds__(kPThreads, 1)
   using SH = PShape<HD>;
   constexpr int CB = SH::CB, NSK = SH::NSK, NSV = SH::NSV;
   extern __shared__ uint8_t smem_dyn[];
-  __shared__ uint64_t qbar, kfull[NSK], kempty[NSK], vfull[NSV], vempty[NSV];
-  __shared__ uint64_t sfull[kQT], pfull[kQT], odone[kQT];
+  __shared__ __align__(16) uint8_t clc_buf[16];
+  __shared__ uint64_t clc_bar, vzero, qfull, qempty, kfull[NSK], kempty[NSK], vfull[NSV], vempty[NSV];
+  __shared__ uint64_t info_full[2], info_empty[2];
+  __shared__ uint64_t sfull[kQT], pfull[kQT][2], odone[kQT];  // pfull: first, second half of P
   __shared__ uint32_t tmem_base;
-  __shared__ int wmax[kSoftWarps];
+  __shared__ Item items[2];
+  __shared__ int spos[2][kQT * kPM];        // positions of the item's rows (-1: absent or invalid)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // query tile i: rows rb[i] .. rb[i] + 127 of query head hh[i]
-  const int b = blockIdx.z;
-  const int rows_cta = p.pair ? kPM : kQT * kPM;
-  const int nblk = (p.Tq + rows_cta - 1) / rows_cta;
-  const int r0 = (nblk - 1 - (int)blockIdx.x) * rows_cta;  // later rows (more work) first
-  int rb[kQT], hh[kQT];
-#pragma unroll
-  for (int i = 0; i < kQT; ++i) {
-    rb[i] = p.pair ? r0 : r0 + i * kPM;
-    hh[i] = p.pair ? kQT * (int)blockIdx.y + i : (int)blockIdx.y;
-  }
-  const int hkv = hh[0] / p.G;  // the same kv head for both tiles
+  const int rows_item = p.pair ? kPM : kQT * kPM;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* Qs = base;                         // [kQT] Q tiles
   uint8_t* Ks = Qs + kQT * SH::Q_BYTES;       // [NSK] K tiles
   uint8_t* Vs = Ks + NSK * SH::KV_BYTES;      // [NSV] V tiles
+  uint8_t* Os = Vs + NSV * SH::KV_BYTES;      // [kSoftWarps] output staging
 
   if (tid == 0) {
-    mbar_init(&qbar, 1);
+    mbar_init(&clc_bar, 1);
+    mbar_init(&vzero, 1);
+    mbar_init(&qfull, 1);
+    mbar_init(&qempty, 1);
     for (int s = 0; s < NSK; ++s) {
       mbar_init(&kfull[s], 1);
       mbar_init(&kempty[s], 1);
@@ -121,9 +187,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
       mbar_init(&vfull[s], 1);
       mbar_init(&vempty[s], 1);
     }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&info_full[i], 1);
+      mbar_init(&info_empty[i], 2 + kSoftWarps);
+    }
     for (int i = 0; i < kQT; ++i) {
       mbar_init(&sfull[i], 1);
-      mbar_init(&pfull[i], kPM);
+      mbar_init(&pfull[i][0], 4);
+      mbar_init(&pfull[i][1], 4);
       mbar_init(&odone[i], 1);
     }
     fence_mbar_init();
@@ -139,314 +210,482 @@ __global__ void __launch_bounds__(kPThreads, 1)
   // come from the previous grid
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-
-  // ---- positions of the softmax threads' rows; the largest of each tile
-  const int max_slots = p.max_pages * p.P;
-  int mypos = -1;  // -1: row absent or invalid, fully masked
-  const int my_tile = warp < kSoftWarps ? warp >> 2 : 0;
-  const int r = rb[my_tile] + (tid - my_tile * kPM);
-  if (warp < kSoftWarps && r < p.Tq) {
-    const int v = p.pos[(int64_t)b * p.Tq + r];
-    if (v >= 0 && v < max_slots) mypos = v;
-    else report(p.status, WM_ERR_BOUNDS);
-  }
-  if (warp < kSoftWarps) {
-    int mx = mypos;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    }
-    if (lane == 0) {
-      wmax[warp] = mx;
-    }
-  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_base;
-  int ntile[kQT], tmaxpos = -1;
-#pragma unroll
-  for (int i = 0; i < kQT; ++i) {
-    const int mx = max(max(wmax[4 * i], wmax[4 * i + 1]), max(wmax[4 * i + 2], wmax[4 * i + 3]));
-    ntile[i] = mx >= 0 ? mx / kPN + 1 : 0;  // KV tiles of query tile i
-    tmaxpos = max(tmaxpos, mx);
-  }
-  const int nmax = tmaxpos >= 0 ? tmaxpos / kPN + 1 : 0;
 
-  if (warp == kLoadWarp) {
-    // ================================================================ TMA
-    // Lane t owns box t of every KV tile (one box per page, or one per 128
-    // slots of a longer page): its page id for the next tile is fetched
-    // while the current tile is issued, so no page-table load sits on the
-    // issue path.  Lane 0 posts the expected bytes before the lanes copy.
-    if (nmax > 0) {
+  if (warp >= kSoftWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssueRegs));
+    // Lane t of a load warp owns box t of every KV tile (one box per page, or
+    // one per 128 slots of a longer page): its page id for the next tile is
+    // fetched while the current tile is issued, so no page-table load sits on
+    // the issue path.  Lane 0 posts the expected bytes before the lanes copy.
+    const int boxes = p.P >= kPN ? 1 : kPN >> p.log2P;  // <= 16 for pages of >= 8 slots
+    const int brows = p.P >= kPN ? kPN : p.P;
+    // tensor-map row of this lane's box of KV tile j (-brows: read zeros)
+    auto box_row = [&](int j, int b, int hkv, int tmaxpos, bool tell) -> int {
+      const int s = j * kPN + lane * brows;  // first slot of the box
+      const int lp = s >> p.log2P;           // logical page
+      int row = -brows;
+      if (lane < boxes && s <= tmaxpos && lp < p.max_pages) {
+        const int pg = p.page_table[(int64_t)b * p.max_pages + lp];
+        if (pg >= 0 && pg < p.num_pages)
+          row = (int)((((int64_t)p.chan * p.num_pages + pg) * p.Hkv + hkv) * p.P + (s & (p.P - 1)));
+        else if (tell)
+          report(p.status, WM_ERR_BOUNDS);
+      }
+      return row;
+    };
+    auto load_tile = [&](const CUtensorMap* tm, uint8_t* dst, int row, uint64_t* bar) {
+      if (lane == 0) mbar_arrive_expect_tx(bar, SH::KV_BYTES);
+      __syncwarp();
+      if (lane < boxes)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+          tc::tma_load_2d(dst + cb * kBlock + lane * brows * 128, tm, cb * 64, row, bar);
+    };
+    if (warp == kLoadWarp) {
+      // ============================================================== items, Q, K
+      const int max_slots = p.max_pages * p.P;
       bool ok = true;
-      if (lane == 0) {
-        mbar_arrive_expect_tx(&qbar, kQT * SH::Q_BYTES);
-        for (int i = 0; i < kQT; ++i)
-#pragma unroll
-          for (int cb = 0; cb < CB; ++cb)
-            tc::tma_load_2d(Qs + i * SH::Q_BYTES + cb * kBlock, &tmQ, hh[i] * HD + cb * 64,
-                            b * p.Tq + rb[i], &qbar);
-      }
-      const int boxes = p.P >= kPN ? 1 : kPN >> p.log2P;  // <= 16 for pages of >= 8 slots
-      const int brows = p.P >= kPN ? kPN : p.P;
-      // tensor-map row of this lane's box of KV tile j (-brows: read zeros)
-      auto box_row = [&](int j) -> int {
-        const int s = j * kPN + lane * brows;  // first slot of the box
-        const int lp = s >> p.log2P;           // logical page
-        int row = -brows;
-        if (lane < boxes && s <= tmaxpos && lp < p.max_pages) {
-          const int pg = p.page_table[(int64_t)b * p.max_pages + lp];
-          if (pg >= 0 && pg < p.num_pages)
-            row = (int)((((int64_t)p.chan * p.num_pages + pg) * p.Hkv + hkv) * p.P + (s & (p.P - 1)));
-          else
-            report(p.status, WM_ERR_BOUNDS);
+      int lin = (int)blockIdx.x;
+      uint32_t kc = 0, qc = 0;  // K tiles and items' Q loaded so far
+      for (uint32_t it = 0; ok; ++it) {
+        const int slot = it & 1;
+        if (it >= 2)
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(&info_empty[slot], ((it >> 1) - 1) & 1));
+        if (!ok) break;
+        if (lin < 0) {
+          if (lane == 0) {
+            items[slot].valid = 0;
+            mbar_arrive(&info_full[slot]);
+          }
+          break;
         }
-        return row;
-      };
-      auto load_tile = [&](const CUtensorMap* tm, uint8_t* dst, int row, uint64_t* bar) {
-        if (lane == 0) mbar_arrive_expect_tx(bar, SH::KV_BYTES);
+        // item `lin`: units of a group side by side, later rows (more work) first
+        const int units = p.B * p.heads;
+        const int g0 = lin / (p.group * p.nblk) * p.group;
+        const int rem = lin - g0 * p.nblk, gn = min(p.group, units - g0);
+        const int unit = g0 + rem % gn;
+        const int b = unit / p.heads, y = unit - b * p.heads;
+        const int r0 = (p.nblk - 1 - rem / gn) * rows_item;
+        int mx[kQT] = {-1, -1}, ps[kQT * kPM / 32];
+        bool bad = false;
+#pragma unroll
+        for (int u = 0; u < kQT * kPM / 32; ++u) {
+          const int row = u * 32 + lane;
+          ps[u] = -1;
+          if (row < rows_item && r0 + row < p.Tq) ps[u] = p.pos[(int64_t)b * p.Tq + r0 + row];
+        }
+#pragma unroll
+        for (int u = 0; u < kQT * kPM / 32; ++u) {
+          const int row = u * 32 + lane;
+          const bool there = row < rows_item && r0 + row < p.Tq;
+          const int v = there && ps[u] >= 0 && ps[u] < max_slots ? ps[u] : -1;
+          bad |= there && v < 0;
+          if (row < rows_item) spos[slot][row] = v;
+          if (u < kPM / 32) mx[0] = max(mx[0], v);
+          else mx[1] = max(mx[1], v);
+        }
+        if (bad) report(p.status, WM_ERR_BOUNDS);
+        mx[0] = __reduce_max_sync(0xFFFFFFFFu, mx[0]);
+        mx[1] = p.pair ? mx[0] : __reduce_max_sync(0xFFFFFFFFu, mx[1]);
+        const int tmaxpos = max(mx[0], mx[1]);
+        const int nmax = tmaxpos >= 0 ? tmaxpos / kPN + 1 : 0;
+        if (lane == 0) {
+          Item q;
+          q.valid = 1;
+          q.b = b;
+          q.y = y;
+          q.r0 = r0;
+#pragma unroll
+          for (int i = 0; i < kQT; ++i) q.nt[i] = mx[i] >= 0 ? mx[i] / kPN + 1 : 0;
+          q.tmaxpos = tmaxpos;
+          items[slot] = q;
+        }
         __syncwarp();
-        if (lane < boxes)
-#pragma unroll
-          for (int cb = 0; cb < CB; ++cb)
-            tc::tma_load_2d(dst + cb * kBlock + lane * brows * 128, tm, cb * 64, row, bar);
-      };
-      int row_next = box_row(0);
-      for (int j = 0; j < nmax && ok; ++j) {
-        const int row = row_next;
-        if (j + 1 < nmax) row_next = box_row(j + 1);
-        const int sk = j % NSK, sv = j % NSV;
-        if (j >= NSK) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&kempty[sk], (j / NSK - 1) & 1));
-        if (!ok) break;
-        load_tile(&tmK, Ks + sk * SH::KV_BYTES, row, &kfull[sk]);
-        if (j >= NSV) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&vempty[sv], (j / NSV - 1) & 1));
-        if (!ok) break;
-        load_tile(&tmV, Vs + sv * SH::KV_BYTES, row, &vfull[sv]);
-      }
-      if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
-    }
-  } else if (warp == kMmaWarp) {
-    // ================================================================ MMA
-    // every lane runs the schedule (all wait, all zero the last V tile's
-    // unwritten rows, wait outcomes made warp-uniform); lane 0 issues
-    const uint32_t idesc_s = tc::idesc_bf16_f32(kPM, kPN);
-    const uint32_t idesc_o = tc::idesc_bf16_f32(kPM, HD) | tc::kIdescBMajorMN;
-    auto wait_all = [&](uint64_t* bar, uint32_t parity) {
-      return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity));
-    };
-    bool ok = nmax == 0 || wait_all(&qbar, 0);
-    auto issue_s = [&](int i, int j) {  // S_i = Q_i K_j^T
-      if (lane == 0) {
-        const uint32_t q0 = smem_u32(Qs + i * SH::Q_BYTES);
-        const uint32_t k0 = smem_u32(Ks + (j % NSK) * SH::KV_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * kBlock + (kk & 3) * 32;
-          tc::mma_bf16(tmem + 128 * i, tc::sdesc_kmajor_sw128(q0 + off),
-                       tc::sdesc_kmajor_sw128(k0 + off), idesc_s, kk > 0);
+        if (lane == 0) {
+          mbar_arrive(&info_full[slot]);
+          // the next item's index, needed when this item's loads are out
+          mbar_arrive_expect_tx(&clc_bar, 16);
+          clc_request(clc_buf, &clc_bar);
         }
-        tc::mma_commit(&sfull[i]);
-      }
-    };
-    auto issue_pv = [&](int i, int j) {  // O_i += P_i V_j
-      if (lane == 0) {
-        const uint32_t v0 = smem_u32(Vs + (j % NSV) * SH::KV_BYTES);
+        __syncwarp();
+        if (nmax > 0) {
+          const int hkv = (p.pair ? kQT * y : y) / p.G;  // the same kv head for both tiles
+          int row_next = box_row(0, b, hkv, tmaxpos, true);
+          for (int j = 0; j < nmax && ok; ++j) {
+            const int row = row_next;
+            if (j + 1 < nmax) row_next = box_row(j + 1, b, hkv, tmaxpos, true);
+            const int sk = kc % NSK;
+            if (kc >= NSK) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&kempty[sk], (kc / NSK - 1) & 1));
+            if (!ok) break;
+            load_tile(&tmK, Ks + sk * SH::KV_BYTES, row, &kfull[sk]);
+            ++kc;
+            if (j == 0) {  // the Q tiles, once every S of the last item is done with theirs
+              if (qc > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&qempty, (qc - 1) & 1));
+              if (!ok) break;
+              if (lane == 0) {
+                mbar_arrive_expect_tx(&qfull, kQT * SH::Q_BYTES);
+                for (int i = 0; i < kQT; ++i) {
+                  const int hh = p.pair ? kQT * y + i : y;
+                  const int rb = p.pair ? r0 : r0 + i * kPM;
 #pragma unroll
-        for (int kk = 0; kk < kPN / 16; ++kk)
-          tc::mma_bf16_ts(tmem + 256 + 128 * i, tmem + 128 * i + 8 * kk,
-                          tc::sdesc_mnmajor_sw128(v0 + kk * 16 * 128, kBlock, 1024), idesc_o,
-                          (j | kk) != 0);
-        tc::mma_commit(&odone[i]);
-      }
-    };
-    if (ok && nmax > 0) {
-      ok = wait_all(&kfull[0], 0);
-      tc::fence_after_sync();
-      if (ok) {
-        for (int i = 0; i < kQT; ++i)
-          if (ntile[i] > 0) issue_s(i, 0);
-        if (lane == 0) tc::mma_commit(&kempty[0]);
-      }
-    }
-    for (int j = 0; j < nmax && ok; ++j) {
-      const int st = j % NSV;
-      ok = wait_all(&vfull[st], (j / NSV) & 1);
-      if (!ok) break;
-      const int s0 = j * kPN;
-      if (j == nmax - 1 && s0 + kPN - 1 > tmaxpos) {
-        // slots past the largest position may be unwritten: zero their V rows
-        uint8_t* vt = Vs + st * SH::KV_BYTES;
-        for (int row = tmaxpos - s0 + 1 + lane; row < kPN; row += 32)
-#pragma unroll
-          for (int cb = 0; cb < CB; ++cb)
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              *reinterpret_cast<uint4*>(vt + cb * kBlock + row * 128 + u * 16) =
-                  make_uint4(0, 0, 0, 0);
+                  for (int cb = 0; cb < CB; ++cb)
+                    tc::tma_load_2d(Qs + i * SH::Q_BYTES + cb * kBlock, &tmQ, hh * HD + cb * 64,
+                                    b * p.Tq + rb, &qfull);
+                }
+              }
+              __syncwarp();
+              ++qc;
+            }
+          }
+        }
+        // the answer is read (or, after a failure, waited for) before its
+        // buffer may be used again or given up
+        const bool got = __all_sync(0xFFFFFFFFu, mbar_wait(&clc_bar, it & 1));
+        ok = ok && got;
+        if (!ok) break;
+        lin = clc_answer(clc_buf);
         fence_proxy_async_shared();
         __syncwarp();
       }
-      const bool more = j + 1 < nmax;
-      if (more) {
-        ok = wait_all(&kfull[(j + 1) % NSK], ((j + 1) / NSK) & 1);
+      if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
+    } else if (warp == kLoadVWarp) {
+      // ============================================================== V
+      bool ok = true;
+      uint32_t vc = 0;  // V tiles loaded so far
+      for (uint32_t it = 0; ok; ++it) {
+        const int slot = it & 1;
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&info_full[slot], (it >> 1) & 1));
         if (!ok) break;
+        const Item q = items[slot];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&info_empty[slot]);
+        if (!q.valid) break;
+        const int nmax = q.tmaxpos >= 0 ? q.tmaxpos / kPN + 1 : 0;
+        if (nmax == 0) continue;
+        const int hkv = (p.pair ? kQT * q.y : q.y) / p.G;
+        int row_next = box_row(0, q.b, hkv, q.tmaxpos, false);  // (the K warp reports bad pages)
+        for (int j = 0; j < nmax && ok; ++j) {
+          const int row = row_next;
+          if (j + 1 < nmax) row_next = box_row(j + 1, q.b, hkv, q.tmaxpos, false);
+          const int sv = vc % NSV;
+          if (vc >= NSV) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&vempty[sv], (vc / NSV - 1) & 1));
+          if (!ok) break;
+          load_tile(&tmV, Vs + sv * SH::KV_BYTES, row, &vfull[sv]);
+          ++vc;
+          const int first = q.tmaxpos - j * kPN + 1;  // slots past the largest position
+          if (j + 1 == nmax && first < kPN) {
+            // they may be unwritten: zero their V rows before P V reads the tile
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&vfull[sv], ((vc - 1) / NSV) & 1));
+            if (!ok) break;
+            uint8_t* vt = Vs + sv * SH::KV_BYTES;
+            for (int r = first + lane; r < kPN; r += 32)
+#pragma unroll
+              for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                  *reinterpret_cast<uint4*>(vt + cb * kBlock + r * 128 + u * 16) =
+                      make_uint4(0, 0, 0, 0);
+            fence_proxy_async_shared();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&vzero);
+          }
+        }
       }
-      for (int i = 0; i < kQT && ok; ++i) {
-        if (j >= ntile[i]) continue;
-        ok = wait_all(&pfull[i], j & 1);
-        if (!ok) break;
-        tc::fence_after_sync();
-        issue_pv(i, j);
-        if (j + 1 < ntile[i]) issue_s(i, j + 1);
-      }
-      if (lane == 0) {
-        tc::mma_commit(&vempty[st]);
-        if (more) tc::mma_commit(&kempty[(j + 1) % NSK]);
+      if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
+    } else if (warp == kMmaWarp) {
+      // ============================================================== MMA
+      // One elected thread runs the schedule.  (With the whole warp in the
+      // waits, each cost about 110 cycles of an idle matrix pipe, 5 a step.)
+      if (tc::elect_one()) {
+        const uint32_t idesc_s = tc::idesc_bf16_f32(kPM, kPN);
+        const uint32_t idesc_o = tc::idesc_bf16_f32(kPM, HD) | tc::kIdescBMajorMN;
+        // Descriptors of the first tiles; a tile or k-step further on adds its byte
+        // offset / 16 to the address field (all of shared memory fits its 14 bits).
+        const uint64_t qd0 = tc::sdesc_kmajor_sw128(smem_u32(Qs));
+        const uint64_t kd0 = tc::sdesc_kmajor_sw128(smem_u32(Ks));
+        const uint64_t vd0 = tc::sdesc_mnmajor_sw128(smem_u32(Vs), kBlock, 1024);
+        auto issue_s = [&](int i, uint32_t st) {  // S_i = Q_i K^T, K in ring slot st
+          const uint64_t qd = qd0 + (uint64_t)((uint32_t)i * (SH::Q_BYTES >> 4));
+          const uint64_t kd = kd0 + (uint64_t)(st * (SH::KV_BYTES >> 4));
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk) {
+            const uint64_t off = ((kk >> 2) * kBlock + (kk & 3) * 32) >> 4;
+            tc::mma_bf16(tmem + 128 * i, qd + off, kd + off, idesc_s, kk > 0);
+          }
+          tc::mma_commit(&sfull[i]);
+        };
+        // O_i (+)= P_i V over half of the slots, V in ring slot st
+        auto issue_pv = [&](int i, uint32_t st, bool first, int half) {
+          const uint64_t vd = vd0 + (uint64_t)(st * (SH::KV_BYTES >> 4));
+#pragma unroll
+          for (int k2 = 0; k2 < kPN / 32; ++k2) {
+            const int kk = half * (kPN / 32) + k2;
+            tc::mma_bf16_ts(tmem + 256 + 128 * i, tmem + 128 * i + 8 * kk,
+                            vd + (kk * 16 * 128 >> 4), idesc_o, !first || kk != 0);
+          }
+          if (half == 1) tc::mma_commit(&odone[i]);
+        };
+        bool ok = true;
+        uint32_t kc = 0, vc = 0, qc = 0, zc = 0;  // K, V, items' Q and zeroed V tiles used so far
+        uint32_t cnt[kQT] = {0, 0};               // P tiles used so far
+        for (uint32_t it = 0; ok; ++it) {
+          const int slot = it & 1;
+          ok = mbar_wait_spin(&info_full[slot], (it >> 1) & 1);
+          if (!ok) break;
+          const int valid = items[slot].valid, tmaxpos = items[slot].tmaxpos;
+          const int nt[kQT] = {items[slot].nt[0], items[slot].nt[1]};
+          mbar_arrive(&info_empty[slot]);
+          if (!valid) break;
+          const int nmax = tmaxpos >= 0 ? tmaxpos / kPN + 1 : 0;
+          if (nmax == 0) continue;
+          ok = mbar_wait_spin(&kfull[kc % NSK], (kc / NSK) & 1) && mbar_wait_spin(&qfull, qc & 1);
+          if (!ok) break;
+          ++qc;
+          tc::fence_after_sync();
+#pragma unroll
+          for (int i = 0; i < kQT; ++i)
+            if (nt[i] > 0) issue_s(i, kc % NSK);
+          if (nmax == 1) tc::mma_commit(&qempty);
+          tc::mma_commit(&kempty[kc % NSK]);
+          ++kc;
+          for (int j = 0; j < nmax; ++j) {
+            const uint32_t st = vc % NSV;
+            ok = mbar_wait_spin(&vfull[st], (vc / NSV) & 1);
+            const bool more = j + 1 < nmax;
+            if (ok && !more && tmaxpos - j * kPN + 1 < kPN) ok = mbar_wait_spin(&vzero, zc++ & 1);
+            if (!ok) break;
+#pragma unroll
+            for (int i = 0; i < kQT; ++i) {
+              if (j >= nt[i] || !ok) continue;
+              ok = mbar_wait_spin(&pfull[i][0], cnt[i] & 1);
+              if (!ok) continue;
+              tc::fence_after_sync();
+              issue_pv(i, st, j == 0, 0);
+              ok = mbar_wait_spin(&pfull[i][1], cnt[i] & 1);
+              if (!ok) continue;
+              tc::fence_after_sync();
+              issue_pv(i, st, j == 0, 1);
+              ++cnt[i];
+              if (j + 1 < nt[i]) {
+                ok = mbar_wait_spin(&kfull[kc % NSK], (kc / NSK) & 1);  // (at once for the second tile)
+                if (!ok) continue;
+                tc::fence_after_sync();
+                issue_s(i, kc % NSK);
+              }
+            }
+            if (!ok) break;
+            tc::mma_commit(&vempty[st]);
+            if (more) tc::mma_commit(&kempty[kc % NSK]);
+            if (j + 2 == nmax) tc::mma_commit(&qempty);  // that was the item's last S
+            ++vc;
+            if (more) ++kc;
+          }
+        }
+        if (!ok) report(p.status, WM_ERR_TIMEOUT);
       }
       __syncwarp();
     }
-    if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
   } else {
     // ================================================================ softmax
-    const int i = warp >> 2;  // query tile
-    const int n = ntile[i];
-    const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t scol = 128 * i, ocol = 256 + 128 * i;
-    float m = -INFINITY, l = 0.f;  // max used for P (log2 units) and running sum
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs));
+    const int i = warp >> 2, quad = warp & 3;  // query tile, TMEM lane quadrant
+    const int row = quad * 32 + lane;
+    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+    const uint32_t scol = lane_base + 128 * i, ocol = lane_base + 256 + 128 * i;
+    uint8_t* stage = Os + warp * kStageBytes;
+    uint32_t cnt = 0;  // S tiles used so far
     bool ok = true;
-    // tcgen05.ld / st are warp-collective: every lane of the warp issues each
-    // one, and the wait outcomes are made warp-uniform before any branch
-    for (int j = 0; j < n && ok; ++j) {
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&sfull[i], j & 1));
+    for (uint32_t it = 0; ok; ++it) {
+      const int slot = it & 1;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(&info_full[slot], (it >> 1) & 1));
+      if (!ok) break;
+      const int n = items[slot].valid ? items[slot].nt[i] : -1;
+      if (n < 0) break;
+      const int mypos = spos[slot][p.pair ? row : i * kPM + row];
+      float m = -INFINITY, l = 0.f;  // max used for P (log2 units) and running sum
+      // tcgen05.ld / st are warp-collective: every lane of the warp issues each
+      // one, and the wait outcomes are made warp-uniform before any branch
+      for (int j = 0; j < n; ++j) {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&sfull[i], cnt & 1));
+        if (!ok) break;
+        ++cnt;
+        tc::fence_after_sync();
+        // Visible slots of this row in the tile: e < vis (all 128 unless the
+        // diagonal crosses the tile).  The masked path only runs there.
+        const int vis = min(max(mypos - j * kPN + 1, 0), kPN);
+        const bool whole = __all_sync(0xFFFFFFFFu, vis == kPN);
+        uint32_t v[4][32];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc::tmem_ld32(scol + 32 * c, v[c]);
+        tc::tmem_ld_wait();
+        // max of 64 scores (log2 units), two chains per 32 of them
+        auto half_max = [&](int half) {
+          float mc[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mc[c] = -INFINITY;
+          if (whole) {
+#pragma unroll
+            for (int e = 0; e < 16; e += 2)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const int cc = 2 * half + (c >> 1), o = 16 * (c & 1) + e;
+                mc[c] = max3(mc[c], __uint_as_float(v[cc][o]), __uint_as_float(v[cc][o + 1]));
+              }
+          } else {
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const int cc = 2 * half + (c >> 1), o = 16 * (c & 1) + e;
+                if (32 * cc + o < vis) mc[c] = fmaxf(mc[c], __uint_as_float(v[cc][o]));
+              }
+          }
+          // qscale > 0: the max commutes with the scale
+          return fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3])) * p.qscale;
+        };
+        // Half of P (64 slots): p = 2^(s * qscale - m) in pairs; masked slots
+        // (and rows with nothing visible yet) give 0.  w: packed pairs.
+        float2 sum2[4];
+        auto half_p = [&](int half, uint32_t (&w)[2][16]) {
+          const float2 qs2 = make_float2(p.qscale, p.qscale), nm2 = make_float2(-m, -m);
+          const bool live = m != -INFINITY;
+          const bool open = whole && __all_sync(0xFFFFFFFFu, live);
+          const int lim0 = live ? vis - 64 * half : 0;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int cc = 2 * half + c, lim = lim0 - 32 * c;
+            sum2[cc] = make_float2(0.f, 0.f);
+            if (open) {
+#pragma unroll
+              for (int e = 0; e < 32; e += 2) {
+                const float2 x = __ffma2_rn(
+                    make_float2(__uint_as_float(v[cc][e]), __uint_as_float(v[cc][e + 1])), qs2, nm2);
+                const float2 pr = make_float2(ex2(x.x), ex2(x.y));
+                sum2[cc] = __fadd2_rn(sum2[cc], pr);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
+                w[c][e / 2] = *reinterpret_cast<const uint32_t*>(&h);
+              }
+            } else {
+#pragma unroll
+              for (int e = 0; e < 32; e += 2) {
+                const float2 x = __ffma2_rn(
+                    make_float2(__uint_as_float(v[cc][e]), __uint_as_float(v[cc][e + 1])), qs2, nm2);
+                const float2 pr =
+                    make_float2(e < lim ? ex2(x.x) : 0.f, e + 1 < lim ? ex2(x.y) : 0.f);
+                sum2[cc] = __fadd2_rn(sum2[cc], pr);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
+                w[c][e / 2] = *reinterpret_cast<const uint32_t*>(&h);
+              }
+            }
+          }
+        };
+        // P goes over the S columns (all read above), slots 2c, 2c + 1 in column c
+        auto hand_over = [&](int half, const uint32_t (&w)[2][16]) {
+          tc::tmem_st16(scol + 32 * half, w[0]);
+          tc::tmem_st16(scol + 32 * half + 16, w[1]);
+          tc::tmem_st_wait();
+          tc::fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&pfull[i][half]);
+        };
+        uint32_t w[2][16];
+        if (j == 0) m = fmaxf(half_max(0), half_max(1));
+        half_p(0, w);
+        if (j > 0) {
+          // Did the row's max grow past the headroom?  The first half's sum of
+          // probabilities tells (64 of at most 2^8 each stay below 2^14, and one
+          // above 2^14 shows, infinities included), the second half's max is taken
+          // beside the exponentials.
+          const float2 s2 = __fadd2_rn(sum2[0], sum2[1]);
+          const float mt1 = half_max(1);
+          bool raise = s2.x + s2.y > kStaleSum || mt1 > m + kStaleMax || m == -INFINITY;
+          if (__any_sync(0xFFFFFFFFu, raise)) {
+            // A row's max grew past the headroom: rescale O (every lane of the
+            // warp takes part; rows that did not raise their max scale by 1)
+            // and take the probabilities again.  P V of the previous tile is
+            // in O: its MMAs were issued before the S that was waited for.
+            float scale = 1.f;
+            const float mt = fmaxf(half_max(0), mt1);
+            raise = raise && mt > m;  // (also false while nothing is visible)
+            if (raise) {
+              scale = m == -INFINITY ? 0.f : ex2(m - mt);
+              m = mt;
+            }
+            l *= scale;
+#pragma unroll 1
+            for (int c = 0; c < HD / 8; ++c) {
+              uint32_t o[8];
+              tc::tmem_ld8(ocol + 8 * c, o);
+              tc::tmem_ld_wait();
+#pragma unroll
+              for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * scale);
+              tc::tmem_st8(ocol + 8 * c, o);
+            }
+            half_p(0, w);
+          }
+        }
+        hand_over(0, w);
+        half_p(1, w);
+        hand_over(1, w);
+        const float2 sa = __fadd2_rn(sum2[0], sum2[1]), sb = __fadd2_rn(sum2[2], sum2[3]);
+        l += (sa.x + sb.x) + (sa.y + sb.y);
+      }
+      if (!ok) break;
+      // ---- the item's rows: O / l, staged through shared memory so that the
+      // stores cover whole sectors (a thread's own row at 16 bytes per
+      // store touched 32 rows at a time: 6500-8700 cycles per item)
+      if (n > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&odone[i], (cnt - 1) & 1));
       if (!ok) break;
       tc::fence_after_sync();
-      const int s0 = j * kPN;
-      // Visible slots of this row in the tile: e < vis (all 128 unless the
-      // diagonal crosses the tile).  The masked path only runs there.
-      const int vis = min(max(mypos - s0 + 1, 0), kPN);
-      // the whole S row in one TMEM read
-      uint32_t v[kPN / 32][32];
-#pragma unroll
-      for (int c = 0; c < kPN / 32; ++c) tc::tmem_ld32(lane_base + scol + 32 * c, v[c]);
-      tc::tmem_ld_wait();
-      float mx = -INFINITY;
-      if (vis == kPN) {
-#pragma unroll
-        for (int c = 0; c < kPN / 32; ++c)
-#pragma unroll
-          for (int e = 0; e < 32; ++e) mx = fmaxf(mx, __uint_as_float(v[c][e]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < kPN / 32; ++c)
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if (32 * c + e < vis) mx = fmaxf(mx, __uint_as_float(v[c][e]));
-      }
-      const float mt = mx * p.qscale;  // qscale > 0: the max commutes with the scale
-      float scale = 1.f;
-      const bool raise = (m == -INFINITY) ? (mt != -INFINITY) : (mt > m + kStaleMax);
-      if (raise) {
-        scale = (m == -INFINITY) ? 0.f : ex2(m - mt);
-        m = mt;
-      }
-      // p = 2^(s * qscale - m) in pairs; masked slots (and rows with nothing
-      // visible yet) give 0
-      const float2 qs2 = make_float2(p.qscale, p.qscale), nm2 = make_float2(-m, -m);
-      const bool live = m != -INFINITY;
-      float2 sum2 = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int c = 0; c < kPN / 32; ++c) {
-        uint32_t w[16];
-        const int lim = live ? vis - 32 * c : 0;
-        if (lim >= 32) {
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float2 x = __ffma2_rn(
-                make_float2(__uint_as_float(v[c][e]), __uint_as_float(v[c][e + 1])), qs2, nm2);
-            const float2 pr = make_float2(ex2(x.x), ex2(x.y));
-            sum2 = __fadd2_rn(sum2, pr);
-            const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
-            w[e / 2] = *reinterpret_cast<const uint32_t*>(&h);
-          }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float2 x = __ffma2_rn(
-                make_float2(__uint_as_float(v[c][e]), __uint_as_float(v[c][e + 1])), qs2, nm2);
-            const float2 pr = make_float2(e < lim ? ex2(x.x) : 0.f, e + 1 < lim ? ex2(x.y) : 0.f);
-            sum2 = __fadd2_rn(sum2, pr);
-            const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
-            w[e / 2] = *reinterpret_cast<const uint32_t*>(&h);
-          }
-        }
-        // P over the S columns (all read above): packed pairs, columns 16c .. 16c+15
-        tc::tmem_st16(lane_base + scol + 16 * c, w);
-      }
-      const float sum = sum2.x + sum2.y;
-      l = l * scale + sum;
-      if (__any_sync(0xFFFFFFFFu, raise && j > 0)) {
-        // a row's max grew past the headroom: rescale O (every lane of the
-        // warp takes part; rows that did not raise their max scale by 1)
-        // once P V of the previous tile has landed in it
-        if (!(raise && j > 0)) scale = 1.f;
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&odone[i], (j - 1) & 1));
-        if (!ok) break;
-        tc::fence_after_sync();
-#pragma unroll
-        for (int c = 0; c < HD / 32; ++c) {
-          uint32_t v[32];
-          tc::tmem_ld32(lane_base + ocol + 32 * c, v);
-          tc::tmem_ld_wait();
-          uint32_t w0[16], w1[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            w0[e] = __float_as_uint(__uint_as_float(v[e]) * scale);
-            w1[e] = __float_as_uint(__uint_as_float(v[16 + e]) * scale);
-          }
-          tc::tmem_st16(lane_base + ocol + 32 * c, w0);
-          tc::tmem_st16(lane_base + ocol + 32 * c + 16, w1);
-        }
-      }
-      tc::tmem_st_wait();
-      tc::fence_before_sync();
-      mbar_arrive(&pfull[i]);
-    }
-    if (ok && n > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&odone[i], (n - 1) & 1));
-    if (!ok) {
-      report(p.status, WM_ERR_TIMEOUT);
-    } else {
-      __nv_bfloat16* dst =
-          reinterpret_cast<__nv_bfloat16*>(p.out) + (((int64_t)b * p.Tq + r) * p.Hq + hh[i]) * HD;
       const float inv = (n > 0 && l > 0.f) ? 1.f / l : 0.f;
-      tc::fence_after_sync();
+      const int b = items[slot].b, y = items[slot].y;
+      const int rb = items[slot].r0 + (p.pair ? 0 : i * kPM) + quad * 32;  // the warp's first row
+      __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) +
+                           (((int64_t)b * p.Tq + rb) * p.Hq + (p.pair ? kQT * y + i : y)) * HD;
+      const int rr = lane >> 2, ch = lane & 3;  // row (of 8) and 16-byte chunk this lane stores
+      const int64_t pitch = (int64_t)p.Hq * HD;
+      __nv_bfloat16* drow = dst + rr * pitch + 8 * ch;
+      uint32_t o[2][32];  // one group of 32 columns on its way while the last is stored
+      tc::tmem_ld32(ocol, o[0]);
 #pragma unroll
       for (int c = 0; c < HD / 32; ++c) {
-        uint32_t v[32];
-        if (n > 0) {  // n is the same for the whole warp group
-          tc::tmem_ld32(lane_base + ocol + 32 * c, v);
-          tc::tmem_ld_wait();
-        }
-        if (r >= p.Tq) continue;
+        tc::tmem_ld_wait();
+        if (c + 1 < HD / 32) tc::tmem_ld32(ocol + 32 * (c + 1), o[(c + 1) & 1]);
 #pragma unroll
         for (int e = 0; e < 32; e += 8) {
-          float f[8];
+          uint32_t u[4];
 #pragma unroll
-          for (int t = 0; t < 8; ++t) f[t] = n > 0 ? __uint_as_float(v[e + t]) * inv : 0.f;
-          uint4 u;
-          __nv_bfloat162 t0 = __floats2bfloat162_rn(f[0], f[1]);
-          __nv_bfloat162 t1 = __floats2bfloat162_rn(f[2], f[3]);
-          __nv_bfloat162 t2 = __floats2bfloat162_rn(f[4], f[5]);
-          __nv_bfloat162 t3 = __floats2bfloat162_rn(f[6], f[7]);
-          u.x = *reinterpret_cast<uint32_t*>(&t0);
-          u.y = *reinterpret_cast<uint32_t*>(&t1);
-          u.z = *reinterpret_cast<uint32_t*>(&t2);
-          u.w = *reinterpret_cast<uint32_t*>(&t3);
-          *reinterpret_cast<uint4*>(dst + 32 * c + e) = u;
+          for (int t = 0; t < 4; ++t) {
+            const float x0 = __uint_as_float(o[c & 1][e + 2 * t]);
+            const float x1 = __uint_as_float(o[c & 1][e + 2 * t + 1]);
+            const __nv_bfloat162 h2 =  // (n == 0: no P V ran, O holds another item's rows)
+                __floats2bfloat162_rn(n > 0 ? x0 * inv : 0.f, n > 0 ? x1 * inv : 0.f);
+            u[t] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+          // row `lane`, 16-byte chunk e/8, placed so that 8 rows cover all banks
+          *reinterpret_cast<uint4*>(stage + lane * 64 + (((e >> 3) ^ ((lane >> 1) & 3)) << 4)) =
+              make_uint4(u[0], u[1], u[2], u[3]);
         }
+        __syncwarp();
+        uint4 u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          u[q] = *reinterpret_cast<const uint4*>(stage + (q * 8 + rr) * 64 +
+                                                 ((ch ^ ((rr >> 1) & 3)) << 4));
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (rb + q * 8 + rr < p.Tq)
+            *reinterpret_cast<uint4*>(drow + q * 8 * pitch + 32 * c) = u[q];
       }
+      tc::fence_before_sync();
+      if (lane == 0) mbar_arrive(&info_empty[slot]);  // (behind a __syncwarp of the staging)
     }
+    if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
   }
   // Every MMA this CTA issued has completed (each was waited on through its
   // commit barrier, or the CTA gave up after a bounded wait); release TMEM.
@@ -466,8 +705,7 @@ cudaError_t launch_hd(const CUtensorMap& q, const CUtensorMap& k, const CUtensor
   if (cudaError_t e = opt_in_smem(kern, (size_t)PShape<HD>::SMEM, smem_set); e != cudaSuccess)
     return e;
   cudaLaunchConfig_t cfg = {};
-  const int rows_cta = p.pair ? kPM : kQT * kPM;
-  cfg.gridDim = dim3((p.Tq + rows_cta - 1) / rows_cta, p.pair ? p.Hq / kQT : p.Hq, p.B);
+  cfg.gridDim = dim3((unsigned)((int64_t)p.nblk * p.heads * p.B));
   cfg.blockDim = dim3(kPThreads);
   cfg.dynamicSmemBytes = PShape<HD>::SMEM;
   cfg.stream = s;
@@ -508,6 +746,17 @@ cudaError_t launch_prefill_attn(const PrefillLaunch& L, cudaStream_t s) {
   int lg = 0;
   while ((1 << lg) < L.P) ++lg;
   p.log2P = lg;
+  const int rows_item = p.pair ? kPM : kQT * kPM;
+  p.nblk = (L.Tq + rows_item - 1) / rows_item;
+  p.heads = p.pair ? L.Hq / kQT : L.Hq;
+  if ((int64_t)p.nblk * p.heads * L.B > INT32_MAX) return cudaErrorInvalidConfiguration;
+  // Items run in the order of their index: within a group of (sequence, head)
+  // units all last row blocks first, so that the launch ends with short items;
+  // a group's K and V (64 MB at most) stay in L2 while its row blocks pass.
+  const int64_t kv_bytes = (int64_t)L.max_pages * L.P * L.d * 4;
+  const int64_t fit = (64ll << 20) / kv_bytes, units = (int64_t)p.heads * L.B;
+  const int64_t groups = fit < 1 ? units : (units + fit - 1) / fit;  // of near-equal size
+  p.group = (int)((units + groups - 1) / groups);
   p.qscale = (float)(1.4426950408889634 / sqrt((double)L.d));
   switch (L.d) {
     case 64: return launch_hd<64>(tq, tk, tv, p, s);
