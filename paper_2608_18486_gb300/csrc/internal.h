@@ -122,7 +122,9 @@ struct MixParams {
   float* zpart;                   // [2][nsplit_r][B][k*L] router partial sums
   float* rope_cs;                 // [B][d/2][2] cos, sin at pos = slot - 1
   void* xop;                      // [2][k][B][D] normed channels, dtype
-  float* proj;                    // [2][k][B][Hkv*d] projection outputs
+  float* proj;                    // [2][k][B][Hkv*d] projection outputs (fp32 path)
+  float* ssq;                     // [2][k][mix_parts][B] sums of htilde^2 over parts of D (bf16)
+  int32_t mix_parts;
   int32_t nsplit_r;
   int32_t* status;
   double inv_freq[kMaxRopeHalf];  // theta^(-2i/d), computed on the host in fp64
@@ -134,7 +136,7 @@ struct MixWorkspace {
 };
 
 MixWorkspace mix_workspace_layout(const wm_config& cfg, int32_t B, int sm_count);
-cudaError_t launch_kv_mix(MixParams& p, int dtype, cudaStream_t s);
+cudaError_t launch_kv_mix(MixParams& p, int dtype, int sms, cudaStream_t s);
 int kv_mix_launches(const MixParams& p, int dtype);  // kernels launch_kv_mix enqueues
 
 // tcgen05 projection with the fused key/value epilogue, and the tcgen05

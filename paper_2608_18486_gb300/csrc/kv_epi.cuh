@@ -20,8 +20,8 @@ struct KvEpiArgs {
 
 // T: shared [token][128] fp32 projection outputs of rows mt*HPT*HD.. of
 // channel j, branch X (0 = K, 1 = V), for the nb tokens of the tile.
-// row_scale (optional, per tile token): multiplies the projection output
-// first (the 1/RMS of the channel state when the operand was not normed).
+// row_scale (per tile token): multiplies the projection output first (the
+// 1/RMS of the channel state: the operand is not normed).
 // s_slot / s_page: each tile token's cache slot and physical page (-1: bad,
 // skipped and reported).  cs_tab: RoPE (cos, sin) pairs [row][HD/2], row =
 // cs_row0 + tile token.  Executed by all NW warps of the block.
@@ -62,16 +62,12 @@ __device__ __forceinline__ void kv_epilogue_tile(const float* T, int nb, int mt,
       if (it < nitems && hh_[q] < a.Hkv && pg_[q] < 0 && reporter && hl == 0 && lane == 0)
         report(a.status, WM_ERR_BOUNDS);
       const float* src = T + n * kM + hl * HD;
-      const float sc = (row_scale != nullptr && it < nitems) ? row_scale[n] : 1.f;
+      const float sc = it < nitems ? row_scale[n] : 1.f;
 #pragma unroll
       for (int t = 0; t < NP; ++t) {
         const int i = lane + 32 * t;
-        y0[q][t] = on[q] && i < HALF ? src[i] : 0.f;
-        y1[q][t] = on[q] && i < HALF ? src[i + HALF] : 0.f;
-        if (row_scale != nullptr) {
-          y0[q][t] *= sc;
-          y1[q][t] *= sc;
-        }
+        y0[q][t] = on[q] && i < HALF ? src[i] * sc : 0.f;
+        y1[q][t] = on[q] && i < HALF ? src[i + HALF] * sc : 0.f;
       }
     }
     if (X == 0) {

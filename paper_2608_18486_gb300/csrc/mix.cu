@@ -7,8 +7,10 @@
 //                  per token the RoPE cos/sin at pos = slot - 1.
 //   2. router    : z = Wr[X] xi (split over the L'D reduction), fp32 partials;
 //                  tcgen05 for bf16 (proj_tc.cu), SIMT FMA for fp32.
-//   3. mix       : alpha = reshape(z + br), htilde_j = sum_l alpha[j][l] hhat_l,
-//                  RMSNorm_j, rounded to the projection operand dtype.
+//   3. mix       : alpha = reshape(z + br), htilde_j = sum_l alpha[j][l] hhat_l;
+//                  bf16: on the tensor cores, the operand is htilde_j times the
+//                  RMSNorm_j gain and the sum of squares goes to the projection's
+//                  epilogue, which scales by 1/RMS; fp32: RMSNorm_j here.
 //   4. projection: W^X_j x^X_j for every branch and channel; for bf16 on
 //                  tcgen05 with the epilogue fused (proj_tc.cu).
 //   5. epilogue  : (fp32) keys: per-head QK-norm then RoPE; keys and values
@@ -292,15 +294,300 @@ __global__ void __launch_bounds__(256) gemm_wxT_simt(const GemmArgs a) {
   }
 }
 
-// ---------------------------------------------------------------- mix
+// ---------------------------------------------------------------- mix (bf16)
+// Per token and branch, htilde = (alpha r) H with alpha [k][L] (r_l = 1/RMS of
+// layer l folded in) and H [L][D] the token's states: a contraction, so it runs
+// on the tensor cores, m16n8k16 with channels as M, layers as K and 8 elements
+// of D as N (the matrices are per token and 16 wide: too small for tcgen05's
+// 128-row tiles).  The states are bf16 as they are; alpha stays fp32 by being
+// three bf16 terms of 8 bits each, three MMAs into one fp32 accumulator, so
+// products and sums are those of fp32 arithmetic.  The pre-mix gain g, a factor
+// per element, multiplies the sum.
+//
+// A unit is one token and one part of D; a warp takes 64 elements at a time for
+// both branches, so h is read once per 16 channels.  Lane (t = lane % 4, g =
+// lane / 4) loads 16 bytes of layers 2t, 2t+1, 2t+8, 2t+9 at vector v(g); element
+// i of the vectors is column g of MMA i, so the eight MMAs' results of one column
+// are 8 consecutive elements, one 16-byte store, and the four t of a store cover
+// 64 bytes.  RMSNorm_j's 1/RMS is left to the projection's epilogue (it is one
+// factor per token and channel), so parts of D need not meet.  Decode steps
+// (COOP): a CTA per unit, its warps share the sum of the router's many split
+// partials and a warp has one or a few 64-element steps.  Groups of tokens: a
+// warp per unit, nothing shared, the next step's states in flight while this
+// step's are used (a CTA per token spent its time waiting for them: 105 us).
+//
+// Bound by memory: h in, the operand out (201 MB at 4096 tokens, L = k = 16, D =
+// 512).  There the scalar kernel before took 194 us, this one 59; at 32
+// tokens, L = 32, k = 16, D = 4096: 40 and 20 (cold caches).
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void mma_16816_first(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+// alpha[j][l] r_l of one token, branch X, for N (j, l) pairs: (bias + the router's
+// split partials) r_l, 0 outside.  The N loads of a split are in flight together.
+template <int N>
+__device__ __forceinline__ void mix_alpha(const MixParams& p, int b, int X, const int (&j)[N],
+                                          const int (&l)[N], float (&a)[N]) {
+  const int kL = p.k * p.L;
+  const float* zp = p.zpart + ((int64_t)X * p.nsplit_r * p.B + b) * kL;
+  const __nv_bfloat16* br = reinterpret_cast<const __nv_bfloat16*>(p.br[X]);
+  int o[N];
+  float r[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const bool in = j[i] < p.k && l[i] < p.L;
+    o[i] = in ? j[i] * p.L + l[i] : 0;
+    r[i] = in ? p.inv_rms[b * p.L + l[i]] : 0.f;
+    a[i] = in ? __bfloat162float(br[o[i]]) : 0.f;
+  }
+#pragma unroll 2
+  for (int s = 0; s < p.nsplit_r; ++s, zp += (int64_t)p.B * kL)
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] += zp[o[i]];
+#pragma unroll
+  for (int i = 0; i < N; ++i) a[i] = j[i] < p.k && l[i] < p.L ? a[i] * r[i] : 0.f;
+}
+
+constexpr int kCoopWarps = 8, kTokenWarps = 4;  // warps per CTA
+
+// KSR: blocks of 16 layers whose states a warp keeps in registers (L <= 16 KSR);
+// 0: any L, the states read again for the second branch.
+template <bool COOP, int KSR>
+__global__ void __launch_bounds__((COOP ? kCoopWarps : kTokenWarps) * 32, COOP ? 2 : KSR == 2 ? 3 : 4)
+    mix_mma_kernel(const MixParams p, int ks_count, int csteps) {
+  const int KS = KSR > 0 ? KSR : ks_count;
+  constexpr int KB = KSR > 0 ? KSR : 1;
+  constexpr int NW = COOP ? kCoopWarps : kTokenWarps;
+  // alpha of 16 channels in the MMA's operand layout, [X][KS][3 terms][32 lanes]
+  // (one for the CTA, or one per warp), then (COOP) sums of squares [warps][X][16]
+  extern __shared__ uint4 frag_s[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint4* frag = frag_s + (COOP ? 0 : warp * 2 * KS * 3 * 32);
+  float* wss = reinterpret_cast<float*>(frag_s + 2 * KS * 3 * 32);
+  const int nparts = p.mix_parts;
+  const int unit = COOP ? (int)blockIdx.x : (int)blockIdx.x * NW + warp;
+  const int b = unit / nparts, part = unit - b * nparts;
+  const int t = lane & 3, g = lane >> 2;
+  const int L = p.L, nvec = p.D / 8;
+  const int vg = (g >> 1) + 4 * (g & 1);  // the vector lane column g stands for
+  const int c0 = part * csteps + (COOP ? warp : 0), cstep = COOP ? NW : 1;
+  const int c_end = min((nvec + 7) / 8, (part + 1) * csteps);
+  if (COOP) {  // gains and (a hint: the data may still be on its way) states towards L2
+    for (int i = tid; i < (p.k + 1) * 2 * (c_end - part * csteps); i += NW * 32) {
+      const int c = part * csteps + i / ((p.k + 1) * 2), r = i % ((p.k + 1) * 2);
+      const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(r < 2 ? p.pre_g[r] : p.ch_g[r & 1]);
+      if (c * 64 < p.D) prefetch_l2(q + (r < 2 ? 0 : (int64_t)((r - 2) >> 1) * p.D) + c * 64);
+    }
+  }
+  pdl_wait();
+  if (!COOP && b >= p.B) return;  // (no block barrier below)
+  const __nv_bfloat16* hp = reinterpret_cast<const __nv_bfloat16*>(p.h) + (int64_t)b * L * p.D;
+  // 16 bytes of the lane's four layers of block ks, step c
+  auto load_h = [&](int c, int ks, uint4 (&hv)[4]) {
+    const int vi = c * 8 + vg;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int l = ks * 16 + 2 * t + (q & 1) + 8 * (q >> 1);
+      hv[q] = c < c_end && l < L && vi < nvec
+                  ? __ldcg(reinterpret_cast<const uint4*>(hp + (int64_t)l * p.D + vi * 8))
+                  : make_uint4(0, 0, 0, 0);
+    }
+  };
+
+  for (int mt = 0; mt * 16 < p.k; ++mt) {
+    uint4 hn[KB][4];
+    if (KSR > 0)
+#pragma unroll
+      for (int ks = 0; ks < KB; ++ks) load_h(c0, ks, hn[ks]);
+    if (COOP) {
+      if (mt > 0) __syncthreads();
+      for (int i = tid; i < 2 * 16 * KS * 8; i += NW * 32) {  // two layers at a time
+        const int lp = i % (KS * 8), rem = i / (KS * 8), jj = rem % 16, X = rem / 16;
+        float a[2];
+        mix_alpha<2>(p, b, X, {mt * 16 + jj, mt * 16 + jj}, {2 * lp, 2 * lp + 1}, a);
+        // operand register and lane of row jj, columns l % 16 and l % 16 + 1
+        const int reg = (jj >> 3) + 2 * ((lp >> 2) & 1), ln = (jj & 7) * 4 + (lp & 3);
+        uint32_t* f = reinterpret_cast<uint32_t*>(frag + (X * KS + (lp >> 3)) * 3 * 32);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {  // the next 8 bits of each
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(a[0], a[1]);
+          a[0] -= __bfloat162float(h2.x);
+          a[1] -= __bfloat162float(h2.y);
+          f[(s * 32 + ln) * 4 + reg] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+      }
+      __syncthreads();
+    } else {
+      __syncwarp();
+      for (int i = 0; i < 2 * KS; ++i) {  // X = i / KS, layer block i % KS
+        const int X = i / KS, ks = i - X * KS;
+        float a[8];  // operand registers r: rows g, g + 8; columns 2t, 2t+1 and + 8
+        int jj[8], ll[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          jj[r] = mt * 16 + g + 8 * ((r >> 1) & 1);
+          ll[r] = ks * 16 + 2 * t + (r & 1) + 8 * (r >> 2);
+        }
+        mix_alpha<8>(p, b, X, jj, ll, a);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          uint32_t w[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a[2 * r], a[2 * r + 1]);
+            a[2 * r] -= __bfloat162float(h2.x);
+            a[2 * r + 1] -= __bfloat162float(h2.y);
+            w[r] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+          frag[(i * 3 + s) * 32 + lane] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+      __syncwarp();
+    }
+
+    float ss[2][2] = {};  // [X][channel g, g + 8]
+    for (int c = c0; c < c_end; c += cstep) {
+      uint32_t bf[KB][8][2];  // element i of layers (2t, 2t+1) and (2t+8, 2t+9)
+      auto pack = [&](const uint4 (&hv)[4], uint32_t (&f)[8][2]) {
+#pragma unroll
+        for (int h2 = 0; h2 < 2; ++h2) {
+          const uint32_t lo[4] = {hv[2 * h2].x, hv[2 * h2].y, hv[2 * h2].z, hv[2 * h2].w};
+          const uint32_t hi[4] = {hv[2 * h2 + 1].x, hv[2 * h2 + 1].y, hv[2 * h2 + 1].z, hv[2 * h2 + 1].w};
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            f[2 * w][h2] = __byte_perm(lo[w], hi[w], 0x5410);
+            f[2 * w + 1][h2] = __byte_perm(lo[w], hi[w], 0x7632);
+          }
+        }
+      };
+      if (KSR > 0) {
+#pragma unroll
+        for (int ks = 0; ks < KB; ++ks) {
+          pack(hn[ks], bf[ks]);
+          if (!COOP) load_h(c + cstep, ks, hn[ks]);  // in flight behind this step's work
+        }
+      }
+#pragma unroll
+      for (int X = 0; X < 2; ++X) {
+        const __nv_bfloat16* pg = reinterpret_cast<const __nv_bfloat16*>(p.pre_g[X]);
+        const __nv_bfloat16* cg = reinterpret_cast<const __nv_bfloat16*>(p.ch_g[X]);
+        __nv_bfloat16* xop = reinterpret_cast<__nv_bfloat16*>(p.xop);
+        // gains of this lane's outputs (column 2t + q: vector t + 4q; channels g, g
+        // + 8), through the read-only path: not held up by the stores
+        uint4 gr[2], cr[2][2];
+        const int v0 = c * 8 + t;
+        const int jr[2] = {mt * 16 + g, mt * 16 + g + 8};
+        const bool in[2] = {v0 < nvec, v0 + 4 < nvec}, ch[2] = {jr[0] < p.k, jr[1] < p.k};
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          gr[q] = in[q] ? __ldg(reinterpret_cast<const uint4*>(pg) + v0 + 4 * q) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+            cr[q][r] = in[q] && ch[r] ? __ldg(reinterpret_cast<const uint4*>(cg + (int64_t)jr[r] * p.D) + v0 + 4 * q)
+                                      : make_uint4(0, 0, 0, 0);
+        }
+        float acc[8][4];
+        for (int ks = 0; ks < KS; ++ks) {
+          if (KSR == 0) {
+            uint4 hv[4];
+            load_h(c, ks, hv);
+            pack(hv, bf[0]);
+          }
+#pragma unroll
+          for (int s = 0; s < 3; ++s) {
+            const uint4 a = frag[((X * KS + ks) * 3 + s) * 32 + lane];
+            const uint32_t(&f)[8][2] = bf[KSR > 0 ? ks : 0];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (ks == 0 && s == 0) mma_16816_first(acc[i], a, f[i][0], f[i][1]);
+              else mma_16816(acc[i], a, f[i][0], f[i][1]);
+            }
+          }
+        }
+        float2 gv[8];  // of both columns, as pairs like the accumulators
+        {
+          float x0[8], x1[8];
+          Elem<__nv_bfloat16>::unpack(gr[0], x0);
+          Elem<__nv_bfloat16>::unpack(gr[1], x1);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) gv[i] = make_float2(x0[i], x1[i]);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          float x0[8], x1[8];
+          Elem<__nv_bfloat16>::unpack(cr[0][r], x0);
+          Elem<__nv_bfloat16>::unpack(cr[1][r], x1);
+          float2 s2 = make_float2(0.f, 0.f);
+          float o0[8], o1[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float2 y = __fmul2_rn(make_float2(acc[i][2 * r], acc[i][2 * r + 1]), gv[i]);
+            s2 = __ffma2_rn(y, y, s2);
+            const float2 o = __fmul2_rn(y, make_float2(x0[i], x1[i]));
+            o0[i] = o.x;
+            o1[i] = o.y;
+          }
+          if (in[0]) ss[X][r] += s2.x;  // (a column past D holds zero times whatever: skipped)
+          if (in[1]) ss[X][r] += s2.y;
+          if (ch[r]) {
+            __nv_bfloat16* dst = xop + (((int64_t)X * p.k + jr[r]) * p.B + b) * p.D + v0 * 8;
+            if (in[0]) store8f<__nv_bfloat16>(dst, o0);
+            if (in[1]) store8f<__nv_bfloat16>(dst + 32, o1);
+          }
+        }
+      }
+      if (COOP && KSR > 0 && c + cstep < c_end) {  // (few steps a warp: no second set of registers)
+#pragma unroll
+        for (int ks = 0; ks < KB; ++ks) load_h(c + cstep, ks, hn[ks]);
+      }
+    }
+    // sums of squares: over the four t of a channel, and the CTA's warps
+#pragma unroll
+    for (int X = 0; X < 2; ++X)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        float v = ss[X][r];
+        v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+        v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+        if (t != 0) continue;
+        const int j = mt * 16 + g + 8 * r;
+        if (COOP)
+          wss[(warp * 2 + X) * 16 + g + 8 * r] = v;
+        else if (j < p.k)
+          p.ssq[(((int64_t)X * p.k + j) * nparts + part) * p.B + b] = v;
+      }
+    if (COOP) {
+      __syncthreads();
+      if (tid < 32) {
+        const int X = tid >> 4, j = mt * 16 + (tid & 15);
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v += wss[(w * 2 + X) * 16 + (tid & 15)];
+        if (j < p.k) p.ssq[(((int64_t)X * p.k + j) * nparts + part) * p.B + b] = v;
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------- mix (fp32)
 // One CTA per (token, branch, group of kChanGroup channels).  Thread t owns
 // the 8-element vectors t, t + 256 of D, so h, gains and the output move as
-// 16-byte vectors.  PRE (decode shapes: L <= kMixPreL, D <= 8 * 256): the
-// thread's h vectors of every layer and its gains are loaded before the
-// router partials are summed, so the kernel waits for one round of loads.
-constexpr int kMixPreL = 16;
-
-template <typename T, bool PRE>
+// 16-byte vectors.  (bf16 takes it only where the driver has no TMA encoder.)
+template <typename T>
 __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
   extern __shared__ float sm[];  // alpha[kChanGroup][L], r[L]
   __shared__ float red[kMixThreads / 32][kChanGroup];
@@ -314,20 +601,6 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
   const T* hp = reinterpret_cast<const T*>(p.h) + (int64_t)b * p.L * p.D;
   const T* g = reinterpret_cast<const T*>(p.pre_g[X]);
   pdl_wait();
-  // PRE: this thread's vector of every layer, of the pre-mix gain and of the
-  // channel gains, all in flight before the router partials are read
-  uint4 hpre[PRE ? kMixPreL : 1], gpre, cpre[kChanGroup];
-  if (PRE && tid < nvec) {
-#pragma unroll
-    for (int l = 0; l < (PRE ? kMixPreL : 1); ++l)
-      if (l < p.L) hpre[l] = __ldg(reinterpret_cast<const uint4*>(hp + (int64_t)l * p.D + tid * 8));
-    gpre = __ldg(reinterpret_cast<const uint4*>(g + tid * 8));
-#pragma unroll
-    for (int jj = 0; jj < kChanGroup; ++jj)
-      if (jj < nj)
-        cpre[jj] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(p.ch_g[X]) +
-                                                        (int64_t)(j0 + jj) * p.D + tid * 8));
-  }
   const T* br = reinterpret_cast<const T*>(p.br[X]);
   // alpha[j][l] = z[j*L + l] = bias + sum of the router's split partials
   for (int i = tid; i < nj * p.L; i += kMixThreads) {
@@ -346,54 +619,29 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
 #pragma unroll
   for (int v = 0; v < kVecPerThread; ++v) {
     const int vi = tid + v * kMixThreads;
-    if (PRE) {
-      if (v == 0 && vi < nvec) Elem<T>::unpack(gpre, gv[0]);
-    } else if (vi < nvec) {
-      load8f<T>(g + vi * 8, gv[v]);
-    }
+    if (vi < nvec) load8f<T>(g + vi * 8, gv[v]);
 #pragma unroll
     for (int jj = 0; jj < kChanGroup; ++jj)
 #pragma unroll
       for (int i = 0; i < 8; ++i) acc[jj][v][i] = 0.f;
   }
-  if (PRE) {
-    if (tid < nvec) {
+#pragma unroll 4
+  for (int l = 0; l < p.L; ++l) {
+    const float r = rl[l];
+    float a[kChanGroup];
 #pragma unroll
-      for (int l = 0; l < (PRE ? kMixPreL : 1); ++l) {
-        if (l >= p.L) break;
-        const float r = rl[l];
-        float a[kChanGroup];
+    for (int jj = 0; jj < kChanGroup; ++jj) a[jj] = jj < nj ? alpha[jj * p.L + l] : 0.f;
 #pragma unroll
-        for (int jj = 0; jj < kChanGroup; ++jj) a[jj] = jj < nj ? alpha[jj * p.L + l] : 0.f;
+    for (int v = 0; v < kVecPerThread; ++v) {
+      const int vi = tid + v * kMixThreads;
+      if (vi < nvec) {
         float hv[8];
-        Elem<T>::unpack(hpre[l], hv);
+        load8f<T>(hp + (int64_t)l * p.D + vi * 8, hv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const float hh = hv[i] * r * gv[0][i];  // pre-mix RMSNorm with gain
+          const float hh = hv[i] * r * gv[v][i];  // pre-mix RMSNorm with gain
 #pragma unroll
-          for (int jj = 0; jj < kChanGroup; ++jj) acc[jj][0][i] = fmaf(a[jj], hh, acc[jj][0][i]);
-        }
-      }
-    }
-  } else {
-#pragma unroll 4
-    for (int l = 0; l < p.L; ++l) {
-      const float r = rl[l];
-      float a[kChanGroup];
-#pragma unroll
-      for (int jj = 0; jj < kChanGroup; ++jj) a[jj] = jj < nj ? alpha[jj * p.L + l] : 0.f;
-#pragma unroll
-      for (int v = 0; v < kVecPerThread; ++v) {
-        const int vi = tid + v * kMixThreads;
-        if (vi < nvec) {
-          float hv[8];
-          load8f<T>(hp + (int64_t)l * p.D + vi * 8, hv);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float hh = hv[i] * r * gv[v][i];  // pre-mix RMSNorm with gain
-#pragma unroll
-            for (int jj = 0; jj < kChanGroup; ++jj) acc[jj][v][i] = fmaf(a[jj], hh, acc[jj][v][i]);
-          }
+          for (int jj = 0; jj < kChanGroup; ++jj) acc[jj][v][i] = fmaf(a[jj], hh, acc[jj][v][i]);
         }
       }
     }
@@ -430,10 +678,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
       const int vi = tid + v * kMixThreads;
       if (vi < nvec) {
         float cv[8], o[8];
-        if (PRE)
-          Elem<T>::unpack(cpre[jj], cv);
-        else
-          load8f<T>(cg + vi * 8, cv);
+        load8f<T>(cg + vi * 8, cv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[i] = acc[jj][v][i] * ss[jj] * cv[i];
         store8f<T>(xo + vi * 8, o);
@@ -653,6 +898,21 @@ __global__ void __launch_bounds__(128) kv_epilogue_kernel(const MixParams p) {
   }
 }
 
+// Parts of D the mix of one token is split into (units of mix_mma_kernel): in a
+// decode step so many CTAs that four fit each SM, down to one 64-element step per
+// warp; in a group of tokens so many warps that 16 fit each SM, down to four steps
+// per warp (each warp sums its token's alpha first).  At most 64 and at most Hkv*d
+// (the projection outputs' place holds the parts' sums).
+int mix_parts(int B, int D, int sms) {
+  const int nc = (D / 8 + 7) / 8;
+  const bool batched = B >= kBatchedTokens;
+  const int most = batched ? (nc + 3) / 4 : (nc + kCoopWarps - 1) / kCoopWarps;
+  const int want = ((batched ? 16 : 4) * sms + B - 1) / B;
+  const int parts = want < most ? want : most;
+  const int per = (nc + parts - 1) / parts;
+  return (nc + per - 1) / per;  // no empty part
+}
+
 template <typename T>
 cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   const int kL = p.k * p.L;
@@ -687,7 +947,27 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
     e = launch_pdl(gemm_wxT_simt<T, T>, grid, dim3(256), 0, s, a);
   }
   if (e != cudaSuccess) return e;
-  if (batched) {
+  const bool tc_proj = bf16 && proj_tc_supported(p);
+  if (tc_proj) {
+    const int KS = (p.L + 15) / 16, nc = (p.D / 8 + 7) / 8;
+    const int csteps = (nc + p.mix_parts - 1) / p.mix_parts;
+    const size_t fr = (size_t)2 * KS * 3 * 512;
+    static size_t smem_set[6][kSmemOptDevices] = {};
+    const int v = KS <= 2 ? KS : 0;  // variant: layers kept in registers or not
+    const size_t smem = batched ? fr * kTokenWarps : fr + (size_t)kCoopWarps * 2 * 16 * sizeof(float);
+    auto kern = batched ? (v == 1   ? mix_mma_kernel<false, 1>
+                           : v == 2 ? mix_mma_kernel<false, 2>
+                                    : mix_mma_kernel<false, 0>)
+                        : (v == 1   ? mix_mma_kernel<true, 1>
+                           : v == 2 ? mix_mma_kernel<true, 2>
+                                    : mix_mma_kernel<true, 0>);
+    e = opt_in_smem(kern, smem, smem_set[3 * batched + v]);
+    if (e != cudaSuccess) return e;
+    const int units = p.B * p.mix_parts;
+    e = launch_pdl(kern, dim3(batched ? (units + kTokenWarps - 1) / kTokenWarps : units),
+                   dim3((batched ? kTokenWarps : kCoopWarps) * 32), smem, s, p, KS, csteps);
+    if (e != cudaSuccess) return e;
+  } else if (batched) {
     const int nvec = p.D / 8;
     const bool two = nvec > kMixThreads;  // D > 2048: two vectors per thread
     const int per = two ? (nvec + 1) / 2 : nvec;
@@ -709,18 +989,11 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   } else {
     const size_t smem = sizeof(float) * (kChanGroup * p.L + p.L);
     dim3 grid(p.B, 2, (p.k + kChanGroup - 1) / kChanGroup);
-    bool pre = false;  // bf16 decode shapes: every load issued up front
-    if constexpr (sizeof(T) == 2) pre = p.L <= kMixPreL && p.D / 8 <= kMixThreads;
-    if constexpr (sizeof(T) == 2) {
-      e = pre ? launch_pdl(mix_kernel<T, true>, grid, dim3(kMixThreads), smem, s, p)
-              : launch_pdl(mix_kernel<T, false>, grid, dim3(kMixThreads), smem, s, p);
-    } else {
-      e = launch_pdl(mix_kernel<T, false>, grid, dim3(kMixThreads), smem, s, p);
-    }
+    e = launch_pdl(mix_kernel<T>, grid, dim3(kMixThreads), smem, s, p);
     if (e != cudaSuccess) return e;
   }
-  if (bf16 && proj_tc_supported(p)) {
-    // bf16: tensor-core projection, QK-norm, RoPE and cache write in one kernel
+  if (tc_proj) {
+    // tensor-core projection, QK-norm, RoPE and cache write in one kernel
     return launch_proj_tc(p, s);
   }
   {
@@ -790,7 +1063,9 @@ int kv_mix_launches(const MixParams& p, int dtype) {
   return dtype == WM_DT_BF16 && proj_tc_supported(p) ? 4 : 5;
 }
 
-cudaError_t launch_kv_mix(MixParams& p, int dtype, cudaStream_t s) {
+cudaError_t launch_kv_mix(MixParams& p, int dtype, int sms, cudaStream_t s) {
+  p.mix_parts = mix_parts(p.B, p.D, sms);
+  p.ssq = p.proj;  // (bf16: [2][k][parts][B] floats, within the fp32 path's projection outputs)
   if (dtype == WM_DT_F32) return launch_all<float>(p, s);
   return launch_all<__nv_bfloat16>(p, s);
 }

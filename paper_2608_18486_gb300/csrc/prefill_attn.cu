@@ -43,7 +43,7 @@
 //
 // What bounds it: the chain S -> softmax -> P V -> next S of each tile; with
 // two tiles in turn a 128-slot step of both takes about 2900 cycles at d = 128,
-// where the matrix products alone take 2048 and the 16384 exponentials 2048.
+// where the matrix products alone take 2048 and the 32768 exponentials 2048.
 // One launch at 32 heads of 128, two prompts of 8192 positions: 939 us before
 // (one item per CTA; every descriptor moved to uniform registers one by one,
 // 90 cycles per MMA; 16-byte row stores at the end), 773 us now; 6/3 heads of

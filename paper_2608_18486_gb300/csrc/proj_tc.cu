@@ -52,6 +52,9 @@ struct ProjTcParams {
   __nv_bfloat16* v_pool;
   const __nv_bfloat16* qk_g;
   const float* rope_cs;
+  const float* ssq;               // projection: [2][k][parts][B] sums of squares of the operand
+  int32_t parts;
+  float inv_D, eps_rms;
   int32_t* status;
 };
 
@@ -67,6 +70,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __shared__ uint64_t full[kTcMaxStages], empty[kTcMaxStages], done;
   __shared__ uint32_t tmem_base;
   __shared__ int s_slot[kTcMaxTokens], s_page[kTcMaxTokens];
+  __shared__ float s_scale[kTcMaxTokens];  // 1/RMS of channel j's state, per token
 
   const int mt = blockIdx.x, j = blockIdx.y, X = blockIdx.z & 1;
   const int n0 = (blockIdx.z >> 1) * p.BN;      // first token of this tile
@@ -149,6 +153,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         pg = p.page_table[(int64_t)(n0 + n) * p.max_pages + (s >> p.log2P)];
       s_slot[n] = s;
       s_page[n] = (pg >= 0 && pg < p.num_pages) ? pg : -1;
+      const float* sq = p.ssq + (int64_t)(X * p.k + j) * p.parts * p.B + n0 + n;
+      float v = 0.f;
+      for (int q = 0; q < p.parts; ++q) v += sq[(int64_t)q * p.B];
+      s_scale[n] = rsqrtf(v * p.inv_D + p.eps_rms);
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer: 4 MMAs of K = 16 per stage
@@ -218,7 +226,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   ea.v_pool = p.v_pool;
   ea.status = p.status;
   const bool local_tab = p.rope_smem_off > 0;
-  kv_epilogue_tile<HD, kTcThreads / 32>(T, nb, mt, j, X, nullptr, s_slot, s_page,
+  kv_epilogue_tile<HD, kTcThreads / 32>(T, nb, mt, j, X, s_scale, s_slot, s_page,
                                         local_tab ? rope_s : p.rope_cs, local_tab ? 0 : n0,
                                         mt == 0 && j == 0 && X == 0, ea);
 }
@@ -323,6 +331,10 @@ cudaError_t launch_proj_tc(const MixParams& mp, cudaStream_t s) {
   p.v_pool = reinterpret_cast<__nv_bfloat16*>(mp.v_pool);
   p.qk_g = reinterpret_cast<const __nv_bfloat16*>(mp.qk_g);
   p.rope_cs = mp.rope_cs;
+  p.ssq = mp.ssq;
+  p.parts = mp.mix_parts;
+  p.inv_D = 1.f / (float)mp.D;
+  p.eps_rms = mp.eps_rms;
   p.status = mp.status;
   CUtensorMap tmW[2], tmX;
   for (int X = 0; X < 2; ++X)

@@ -484,7 +484,7 @@ wm_status wm_kv_mix(const wm_config* c, const wm_cache* cache, const wm_mix_weig
   p.status = dev_status;
   for (int i = 0; i < c->d / 2 && i < wm::kMaxRopeHalf; ++i)
     p.inv_freq[i] = pow(c->rope_theta, -2.0 * i / c->d);
-  cudaError_t e = wm::launch_kv_mix(p, c->dtype, (cudaStream_t)stream);
+  cudaError_t e = wm::launch_kv_mix(p, c->dtype, sm_count(), (cudaStream_t)stream);
   return e == cudaSuccess ? WM_OK : WM_ERR_CUDA;
 }
 
