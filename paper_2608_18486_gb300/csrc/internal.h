@@ -125,6 +125,7 @@ struct MixParams {
   float* proj;                    // [2][k][B][Hkv*d] projection outputs (fp32 path)
   float* ssq;                     // [2][k][mix_parts][B] sums of htilde^2 over parts of D (bf16)
   int32_t mix_parts;
+  int32_t sms;
   int32_t nsplit_r;
   int32_t* status;
   double inv_freq[kMaxRopeHalf];  // theta^(-2i/d), computed on the host in fp64
@@ -146,5 +147,11 @@ cudaError_t launch_proj_tc(const MixParams& p, cudaStream_t s);
 bool router_tc_supported(int B);
 int router_tc_splits(int k, int L, int Lp, int D, int B, int sms);
 cudaError_t launch_router_tc(const MixParams& p, cudaStream_t s);
+// the same for groups of tokens (proj_rows.cu), from kRowsTokens tokens on
+constexpr int kRowsTokens = 128;
+bool proj_rows_supported(const MixParams& p);
+cudaError_t launch_proj_rows(const MixParams& p, int sms, cudaStream_t s);
+int router_rows_splits(int k, int L, int Lp, int D, int B, int sms);
+cudaError_t launch_router_rows(const MixParams& p, int sms, cudaStream_t s);
 
 }  // namespace wm

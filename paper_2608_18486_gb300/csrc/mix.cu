@@ -928,7 +928,7 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   }
   if (e != cudaSuccess) return e;
   if (bf16 && router_tc_supported(p.B)) {
-    e = launch_router_tc(p, s);
+    e = p.B >= kRowsTokens ? launch_router_rows(p, p.sms, s) : launch_router_tc(p, s);
   } else {
     GemmArgs a{};
     a.W[0] = p.Wr[0];
@@ -994,7 +994,7 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   }
   if (tc_proj) {
     // tensor-core projection, QK-norm, RoPE and cache write in one kernel
-    return launch_proj_tc(p, s);
+    return proj_rows_supported(p) ? launch_proj_rows(p, p.sms, s) : launch_proj_tc(p, s);
   }
   {
     GemmArgs a{};
@@ -1033,7 +1033,8 @@ MixWorkspace mix_workspace_layout(const wm_config& cfg, int32_t B, int sm_count)
   const int64_t Kr = (int64_t)Lp * cfg.D;
   int ns;
   if (cfg.dtype == WM_DT_BF16 && router_tc_supported(B)) {
-    ns = router_tc_splits(cfg.k, cfg.L, Lp, cfg.D, B, sm_count);
+    ns = B >= kRowsTokens ? router_rows_splits(cfg.k, cfg.L, Lp, cfg.D, B, sm_count)
+                          : router_tc_splits(cfg.k, cfg.L, Lp, cfg.D, B, sm_count);
   } else {
     const int tiles = 2 * ((kL + BM - 1) / BM) * ((B + BN - 1) / BN);
     ns = (2 * sm_count + tiles - 1) / tiles;
@@ -1064,6 +1065,7 @@ int kv_mix_launches(const MixParams& p, int dtype) {
 }
 
 cudaError_t launch_kv_mix(MixParams& p, int dtype, int sms, cudaStream_t s) {
+  p.sms = sms;
   p.mix_parts = mix_parts(p.B, p.D, sms);
   p.ssq = p.proj;  // (bf16: [2][k][parts][B] floats, within the fp32 path's projection outputs)
   if (dtype == WM_DT_F32) return launch_all<float>(p, s);
