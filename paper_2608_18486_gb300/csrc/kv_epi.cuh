@@ -24,17 +24,17 @@ struct KvEpiArgs {
 // 1/RMS of the channel state: the operand is not normed).
 // s_slot / s_page: each tile token's cache slot and physical page (-1: bad,
 // skipped and reported).  cs_tab: RoPE (cos, sin) pairs [row][HD/2], row =
-// cs_row0 + tile token.  Executed by all NW warps of the block.
+// cs_row0 + tile token.  Executed by NW warps, warp = 0 .. NW-1.
 template <int HD, int NW>
 __device__ __forceinline__ void kv_epilogue_tile(const float* T, int nb, int mt, int j, int X,
                                                  const float* row_scale, const int* s_slot,
                                                  const int* s_page, const float* cs_tab,
-                                                 int cs_row0, bool reporter, const KvEpiArgs& a) {
+                                                 int cs_row0, bool reporter, const KvEpiArgs& a, int warp) {
   constexpr int kM = 128;
   constexpr int HPT = kM / HD;          // whole heads per 128-row tile
   constexpr int HALF = HD / 2;
   constexpr int NP = (HALF + 31) / 32;  // pairs per lane
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
   __nv_bfloat16* pool = X == 0 ? a.k_pool : a.v_pool;
   float qg0[NP], qg1[NP];  // QK-norm gain of channel j, the same for every item
 #pragma unroll

@@ -31,9 +31,9 @@ namespace {
 constexpr int kMixThreads = 256;
 constexpr int kChanGroup = 4; // channels mixed per CTA
 constexpr int kVecPerThread = 2;  // 8-element vectors per thread: D <= 256*8*2
-// Token counts from which the pool runs its batched forms of prenorm and mix
-// (prefill groups): several tokens per CTA, whole warps on every row.  Below
-// it (decode steps) one token per CTA spreads the few tokens over more SMs.
+// Token counts from which the pool runs its batched form of the mix (prefill
+// groups): several tokens per CTA.  Below it (decode steps) one token per CTA
+// spreads the few tokens over more SMs.
 constexpr int kBatchedTokens = 64;
 constexpr int kMixCG = 8;     // channels per CTA in the batched mix
 constexpr int kMixLC = 8;     // most layers per staged chunk of h in the batched mix
@@ -101,97 +101,77 @@ __device__ __forceinline__ void store8f<__nv_bfloat16>(__nv_bfloat16* dst, const
 }
 
 // ---------------------------------------------------------------- prenorm
-template <typename T>
-__global__ void __launch_bounds__(kMixThreads) prenorm_kernel(const MixParams p) {
-  __shared__ float red[32];
-  __shared__ float s_r;
-  const int l = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-  pdl_wait();
-  const T* hp = reinterpret_cast<const T*>(p.h) + ((int64_t)b * p.L + l) * p.D;
-  float ss = 0.f;
-  for (int e = tid; e < p.D; e += kMixThreads) {
-    const float v = ldf(hp + e);
-    ss = fmaf(v, v, ss);
-  }
-  ss = block_sum(ss, red);
-  if (tid == 0) {
-    s_r = rsqrtf(ss / (float)p.D + p.eps_rms);
-    p.inv_rms[b * p.L + l] = s_r;
-  }
-  __syncthreads();
-  const float r = s_r;
-  // router input block m holds layer L-1-m*p
-  const int from_top = p.L - 1 - l;
-  if (from_top % p.p == 0) {
-    const int m = from_top / p.p;
-    for (int X = 0; X < 2; ++X) {
-      const T* g = reinterpret_cast<const T*>(p.pre_g[X]);
-      T* xo = reinterpret_cast<T*>(p.xi) + ((int64_t)X * p.B + b) * ((int64_t)p.Lp * p.D) +
-              (int64_t)m * p.D;
-      for (int e = tid; e < p.D; e += kMixThreads)
-        xo[e] = Elem<T>::from_f(ldf(hp + e) * r * ldf(g + e));
-    }
-  }
-  if (l == 0) {
-    // RoPE angle pos * theta^(-2i/d) in fp64, reduced to [-pi, pi] before sincosf
-    const int s = p.slot[b];
-    const double pos = (double)(s - 1);
-    for (int i = tid; i < p.d / 2; i += kMixThreads) {
-      const double a = pos * p.inv_freq[i];
-      const double two_pi = 6.283185307179586476925286766559;
-      const float ar = (float)(a - two_pi * rint(a / two_pi));
-      float sn, cs;
-      sincosf(ar, &sn, &cs);
-      p.rope_cs[((int64_t)b * (p.d / 2) + i) * 2] = cs;
-      p.rope_cs[((int64_t)b * (p.d / 2) + i) * 2 + 1] = sn;
-    }
-  }
-}
+// WPR warps per (token, layer) row; a lane keeps its part of the row (at most four
+// 8-element vectors) in registers between the sum of squares and the two router
+// inputs, so the row is read once, 16 bytes at a time.  Bound by memory and, in a
+// decode step, by the latency of that one read (the kernel it replaces read 2
+// bytes per load, twice: 17 us at 32 tokens, L = 32, D = 4096; this one PREUS).
+constexpr int kPrenormWarps = 4;
 
-// Batched form: one warp per (token, layer) row, 8 rows per CTA, 16-byte
-// vectors.  Same outputs as prenorm_kernel.
-template <typename T>
-__global__ void __launch_bounds__(kMixThreads) prenorm_rows_kernel(const MixParams p) {
+template <typename T, int WPR>
+__global__ void __launch_bounds__(kPrenormWarps * 32) prenorm_kernel(const MixParams p) {
+  constexpr int MAXV = 4;
+  __shared__ float red[kPrenormWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = blockIdx.x * (kMixThreads / 32) + warp;  // b * L + l
+  const int row = blockIdx.x * (kPrenormWarps / WPR) + warp / WPR;  // b * L + l
+  const int u = (warp % WPR) * 32 + lane, nu = WPR * 32;            // thread of the row
   pdl_wait();
-  if (row >= p.B * p.L) return;  // warp-level from here on
+  if (WPR == 1 && row >= p.B * p.L) return;
   const int b = row / p.L, l = row % p.L;
   const int nvec = p.D / 8;
   const T* hp = reinterpret_cast<const T*>(p.h) + (int64_t)row * p.D;
-  float ss = 0.f;
-  for (int v = lane; v < nvec; v += 32) {
-    float f[8];
-    load8f<T>(hp + v * 8, f);
+  float f[MAXV][8], ss = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) ss = fmaf(f[i], f[i], ss);
+  for (int v = 0; v < MAXV; ++v) {
+    const int vi = u + v * nu;
+    if (vi < nvec) load8f<T>(hp + vi * 8, f[v]);
+    else
+#pragma unroll
+      for (int i = 0; i < 8; ++i) f[v][i] = 0.f;
   }
-  const float r = rsqrtf(warp_sum(ss) / (float)p.D + p.eps_rms);
-  if (lane == 0) p.inv_rms[row] = r;
+#pragma unroll
+  for (int v = 0; v < MAXV; ++v)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ss = fmaf(f[v][i], f[v][i], ss);
+  ss = warp_sum(ss);
+  if (WPR > 1) {
+    if (lane == 0) red[warp] = ss;
+    __syncthreads();
+    ss = 0.f;
+#pragma unroll
+    for (int w = 0; w < kPrenormWarps; ++w) ss += red[w];
+  }
+  const float r = rsqrtf(ss / (float)p.D + p.eps_rms);
+  if (u == 0) p.inv_rms[row] = r;
   const int from_top = p.L - 1 - l;
   if (from_top % p.p == 0) {  // router input block m holds layer L-1-m*p
     const int m = from_top / p.p;
+#pragma unroll
     for (int X = 0; X < 2; ++X) {
       const T* g = reinterpret_cast<const T*>(p.pre_g[X]);
       T* xo = reinterpret_cast<T*>(p.xi) + ((int64_t)X * p.B + b) * ((int64_t)p.Lp * p.D) +
               (int64_t)m * p.D;
-      for (int v = lane; v < nvec; v += 32) {
-        float f[8], gv[8];
-        load8f<T>(hp + v * 8, f);
-        load8f<T>(g + v * 8, gv);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] *= r * gv[i];
-        store8f<T>(xo + v * 8, f);
+      for (int v = 0; v < MAXV; ++v) {
+        const int vi = u + v * nu;
+        if (vi >= nvec) break;
+        float gv[8], o[8];
+        load8f<T>(g + vi * 8, gv);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = f[v][i] * r * gv[i];
+        store8f<T>(xo + vi * 8, o);
       }
     }
   }
   if (l == 0) {
     // RoPE angle pos * theta^(-2i/d) in fp64, reduced to [-pi, pi] before sincosf
+    // (fp64 is slow here: a product with 1/2pi, not a division)
     const double pos = (double)(p.slot[b] - 1);
-    for (int i = lane; i < p.d / 2; i += 32) {
+    for (int i = u; i < p.d / 2; i += nu) {
       const double a = pos * p.inv_freq[i];
       const double two_pi = 6.283185307179586476925286766559;
-      const float ar = (float)(a - two_pi * rint(a / two_pi));
+      const double inv_two_pi = 0.15915494309189533576888376337251;
+      const float ar = (float)(a - two_pi * rint(a * inv_two_pi));
       float sn, cs;
       sincosf(ar, &sn, &cs);
       p.rope_cs[((int64_t)b * (p.d / 2) + i) * 2] = cs;
@@ -354,7 +334,7 @@ __device__ __forceinline__ void mix_alpha(const MixParams& p, int b, int X, cons
     r[i] = in ? p.inv_rms[b * p.L + l[i]] : 0.f;
     a[i] = in ? __bfloat162float(br[o[i]]) : 0.f;
   }
-#pragma unroll 2
+#pragma unroll(N > 2 ? 2 : 8)
   for (int s = 0; s < p.nsplit_r; ++s, zp += (int64_t)p.B * kL)
 #pragma unroll
     for (int i = 0; i < N; ++i) a[i] += zp[o[i]];
@@ -919,12 +899,14 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   const bool bf16 = sizeof(T) == 2;
   const bool batched = p.B >= kBatchedTokens;
   cudaError_t e;
-  if (batched) {
-    const int rows = p.B * p.L, per = kMixThreads / 32;
-    e = launch_pdl(prenorm_rows_kernel<T>, dim3((rows + per - 1) / per), dim3(kMixThreads), 0, s,
-                   p);
-  } else {
-    e = launch_pdl(prenorm_kernel<T>, dim3(p.L, p.B), dim3(kMixThreads), 0, s, p);
+  {
+    const int rows = p.B * p.L;
+    // a row of at most 1024 elements fits one warp's registers
+    if (p.D <= 1024)
+      e = launch_pdl(prenorm_kernel<T, 1>, dim3((rows + kPrenormWarps - 1) / kPrenormWarps),
+                     dim3(kPrenormWarps * 32), 0, s, p);
+    else
+      e = launch_pdl(prenorm_kernel<T, kPrenormWarps>, dim3(rows), dim3(kPrenormWarps * 32), 0, s, p);
   }
   if (e != cudaSuccess) return e;
   if (bf16 && router_tc_supported(p.B)) {

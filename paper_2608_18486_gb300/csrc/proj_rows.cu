@@ -21,10 +21,11 @@
 //  * warp 0: TMA of activation and weight k-blocks (64 columns, 128-byte
 //    swizzle) through an mbarrier ring;
 //  * warp 1: MMAs, from one elected thread;
-//  * warps 2-3: the RoPE table of the tile's tokens, transposed to [pair][token];
+//  * (warps 2-3 only hand over their registers;)
 //  * warps 4-11: epilogue, two groups of four (one TMEM lane quadrant each)
 //    taking turns at the units; a unit's slot is free again once it is in
-//    registers.  Outputs go through a small staging buffer so that a store
+//    registers.  They also load the RoPE table of the tile's tokens, transposed
+//    to [pair][token] (by two warps alone that took 20 us).  Outputs go through a small staging buffer so that a store
 //    covers whole 64-byte runs of the scattered cache rows.
 // Tiles run token tile by token tile, so the table is loaded once or twice per
 // CTA and the activations of a tile are read once; the weights (9 MB there) come
@@ -43,6 +44,9 @@ constexpr int kRBK = 64;                   // K elements per stage (128 bytes of
 constexpr int kRStages = 3;
 constexpr int kEpiWarp0 = 4, kEpiWarps = 8;
 constexpr int kRThreads = (kEpiWarp0 + kEpiWarps) * 32;
+// An epilogue thread holds a head in registers (128 of them at d = 128): the first
+// warpgroup hands over, (2 x 208 + 88) x 128 threads = the 384 x 168 of the launch.
+constexpr int kEpiRegs = 208, kIssueRegs = 88;
 constexpr uint32_t kRStage = 32 * 64;      // staging of an epilogue warp: 32 rows x 64 bytes
 
 enum { kRowsKV = 0, kRowsPartial = 1 };
@@ -124,7 +128,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
       mbar_init(&sfull[s], 1);
       mbar_init(&sempty[s], 4);
     }
-    mbar_init(&tfull, 2);
+    mbar_init(&tfull, kEpiWarps);
     mbar_init(&tempty, kEpiWarps);
     fence_mbar_init();
     tc::prefetch_tensormap(&tmW0);
@@ -149,6 +153,8 @@ __global__ void __launch_bounds__(kRThreads, 1)
     kb1 = MODE == kRowsKV ? p.nk : min(p.nk, kb0 + p.kb_per_split);
   };
 
+  if (warp < kEpiWarp0) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssueRegs));
   if (warp == 0) {
     if (tc::elect_one()) {
       // ============================================================ TMA
@@ -217,38 +223,10 @@ __global__ void __launch_bounds__(kRThreads, 1)
       if (!ok) report(p.status, WM_ERR_TIMEOUT);
     }
     __syncwarp();
-  } else if (warp < kEpiWarp0) {
-    // ============================================================== RoPE table
-    if (MODE == kRowsKV) {
-      bool ok = true;
-      int last = -1;
-      uint32_t n = 0;  // tables loaded
-      for (int x = x0; x < x1 && ok; ++x) {
-        const int tt = tile_of(x, p.nn, nj).tt;
-        if (tt == last) continue;
-        last = tt;
-        if (n > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tempty, (n - 1) & 1));
-        if (!ok) break;
-        // a lane's own token: two pairs per 16-byte load, conflict-free stores
-        for (int r = lane; r < kRM; r += 32) {
-          const int64_t tok = (int64_t)tt * kRM + r;
-          if (tok >= p.B) continue;
-          const float4* src = reinterpret_cast<const float4*>(p.rope_cs + tok * HD);
-#pragma unroll 8
-          for (int i = warp - 2; i < HALF / 2; i += 2) {
-            const float4 f = src[i];
-            tab[(2 * i) * kRM + r] = make_float2(f.x, f.y);
-            tab[(2 * i + 1) * kRM + r] = make_float2(f.z, f.w);
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tfull);
-        ++n;
-      }
-      if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
-    }
+  }
   } else {
     // ================================================================ epilogue
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
     const int grp = (warp - kEpiWarp0) >> 2, quad = warp & 3;
     const int row = quad * 32 + lane;  // this thread's token of the tile
     const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
@@ -264,9 +242,11 @@ __global__ void __launch_bounds__(kRThreads, 1)
       const Tile t = tile_of(x, p.nn, nj);
       const int nu = min(U, p.nunits - t.n * U);
       if (t.tt != last) {
-        if (MODE == kRowsKV && last >= 0) {
+        if (MODE == kRowsKV && last >= 0) {  // every warp is done with the old table
           __syncwarp();
           if (lane == 0) mbar_arrive(&tempty);
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tempty, (nt - 1) & 1));
+          if (!ok) break;
         }
         last = t.tt;
         if (MODE == kRowsKV) {
@@ -284,6 +264,19 @@ __global__ void __launch_bounds__(kRThreads, 1)
           }
 #pragma unroll
           for (int q = 0; q < 4; ++q) ro[q] = __shfl_sync(0xFFFFFFFFu, mine, q * 8 + sr);
+          // this thread's token, every other pair of pairs: 16-byte loads, all in
+          // flight, conflict-free stores
+          if (tok < p.B) {
+            const float4* src = reinterpret_cast<const float4*>(p.rope_cs + (int64_t)tok * HD);
+#pragma unroll
+            for (int i = 0; i < HALF / 4; ++i) {
+              const float4 f = src[2 * i + grp];
+              tab[(4 * i + 2 * grp) * kRM + row] = make_float2(f.x, f.y);
+              tab[(4 * i + 2 * grp + 1) * kRM + row] = make_float2(f.z, f.w);
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tfull);
           ok = __all_sync(0xFFFFFFFFu, mbar_wait(&tfull, nt & 1));
           ++nt;
           if (!ok) break;
