@@ -27,11 +27,18 @@ int attn_unit_warps_per_cta(int stage_bytes, int dtype, int d, int G) {
   return 0;
 }
 
+// ring bytes of one stage of K and V
+static size_t ring_stage_bytes(int stage_bytes, int dtype, int d, int G) {
+  const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
+  return 2 * ((size_t)attn_stage_slots(stage_bytes, dtype, d) * d * esz +
+              (attn_uses_mma(dtype, G) ? kAttnMmaPad : 0));
+}
+
 size_t attn_smem_bytes(int stage_bytes, int dtype, int d, int G, int B) {
   const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
-  const size_t stage = (size_t)attn_stage_slots(stage_bytes, dtype, d) * 2 * d * esz;
+  const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, G);
   return (size_t)attn_detail::kWarps * attn_detail::kWStages * stage +
-         (size_t)attn_detail::kWarps * attn_detail::kWStages * G * d * esz +
+         (attn_uses_mma(dtype, G) ? 0 : (size_t)attn_detail::kWarps * attn_detail::kWStages * G * d * esz) +
          sizeof(int) * (2 * (size_t)B + 1);
 }
 
@@ -43,8 +50,7 @@ cudaError_t launch_decode_attn(const AttnParams& p, int stage_bytes, int dtype, 
 }
 
 size_t attn_unit_smem_bytes(int stage_bytes, int dtype, int d, int G) {
-  const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
-  const size_t stage = (size_t)attn_stage_slots(stage_bytes, dtype, d) * 2 * d * esz;
+  const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, G);
   return (size_t)attn_unit_warps_per_cta(stage_bytes, dtype, d, G) * attn_unit_detail::kUStages * stage +
          (size_t)(attn_unit_detail::unit_rec(G, d) + 3) / 4 * 4 * sizeof(float);
 }

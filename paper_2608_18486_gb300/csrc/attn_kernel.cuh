@@ -16,7 +16,8 @@
 //    fills it with 1-D bulk async copies (TMA engine, mbarrier completion,
 //    L2 evict-first) of contiguous (page, kv-head) runs; it refills a slot as
 //    soon as it has consumed it, so no block-wide barrier is ever taken.
-//  * Compute.  8 lanes own one slot (16-byte vectors, conflict-free shared
+//  * Compute (VecMath; MmaMath in attn_mma.cuh takes four or eight bf16 query
+//    heads per kv head).  8 lanes own one slot (16-byte vectors, conflict-free shared
 //    loads), reduce q.k with xor shuffles and keep an online softmax
 //    (running max m, sum l, accumulator) per lane group; groups merge with
 //    shuffles at the end of a piece.
@@ -37,6 +38,9 @@
 //    ring's worth), and the merge reads them from shared memory.
 #include <math.h>
 
+#include <type_traits>
+
+#include "attn_mma.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -73,13 +77,14 @@ struct Shape {
 };
 
 // Lane part `lp` owns the 16-byte vectors lp, lp + 8, ... of a slot row.
-template <typename T, int HD, int SB>
+template <typename T, int HD, int SB, bool L2 = false>
 __device__ __forceinline__ void load_row(const T* row, int lp, float2 (&f)[Shape<T, HD, SB>::EPL / 2]) {
   using SH = Shape<T, HD, SB>;
 #pragma unroll
   for (int v = 0; v < SH::NVL; ++v) {
     float t[SH::VEC];
-    Elem<T>::unpack(*reinterpret_cast<const uint4*>(row + (v * SH::LPS + lp) * SH::VEC), t);
+    const uint4* src = reinterpret_cast<const uint4*>(row + (v * SH::LPS + lp) * SH::VEC);
+    Elem<T>::unpack(L2 ? __ldcg(src) : *src, t);
 #pragma unroll
     for (int i = 0; i < SH::VEC / 2; ++i) f[v * SH::VEC / 2 + i] = make_float2(t[2 * i], t[2 * i + 1]);
   }
@@ -137,98 +142,237 @@ __device__ __forceinline__ void advance(Cursor& c, const int* pre, int B, int Hk
 }
 
 
-// Online-softmax state of one lane: G query heads, EPL output elements each.
+// Stage math on the CUDA cores, and the online-softmax state of one lane: G
+// query heads, EPL output elements each.
 template <typename T, int HD, int G, int SB>
-struct SoftState {
+struct VecMath {
+  using SH = Shape<T, HD, SB>;
+  static constexpr int SPW = SH::SPW, ITERS = SH::ITERS, LPS = SH::LPS, E2 = SH::EPL / 2;
+  static constexpr int kPad = 0;
+  static constexpr bool kQueryRing = true;  // queries travel with a piece's first stage
+  float2 q2[G][E2];
   float m[G], l[G];
-  float2 acc[G][Shape<T, HD, SB>::EPL / 2];
+  float2 acc[G][E2];
+
+  __device__ __forceinline__ void reset() {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      m[g] = -INFINITY;
+      l[g] = 0.f;
+#pragma unroll
+      for (int i = 0; i < E2; ++i) acc[g][i] = make_float2(0.f, 0.f);
+    }
+  }
+  // The G query rows; L2: from global memory another grid may just have
+  // written, through L2 (ld.global.cg), so that no stale L1 line is read.
+  template <bool L2>
+  __device__ __forceinline__ void load_q(const T* rows, int lane) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) load_row<T, HD, SB, L2>(rows + g * HD, lane % LPS, q2[g]);
+  }
+
+  // One pipeline stage of K/V rows for this warp's current piece.  FULL: every
+  // slot of the stage is inside the sequence and on a fetched page, so no
+  // masking is needed; otherwise masked slots never touch the sums (NaN-safe).
+  template <bool FULL>
+  __device__ __forceinline__ void consume(const T* Ks, const T* Vs, int lane, float qscale,
+                                          int valid_slots, uint64_t mask, int log2R) {
+    const int lane_slot = lane / LPS, lane_part = lane % LPS;
+    float sc[G][ITERS];
+#pragma unroll
+    for (int it = 0; it < ITERS; ++it) {
+      const int ls = it * SPW + lane_slot;
+      float2 kf[E2];
+      load_row<T, HD, SB>(Ks + ls * HD, lane_part, kf);
+      bool valid = true;
+      if (!FULL) valid = (ls < valid_slots) && ((mask >> (ls >> log2R)) & 1ull);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        float2 a = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < E2; ++i) a = __ffma2_rn(q2[g][i], kf[i], a);
+        float s = group_sum<LPS>(a.x + a.y) * qscale;
+        sc[g][it] = valid ? s : -INFINITY;
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      float mx = sc[g][0];
+#pragma unroll
+      for (int it = 1; it < ITERS; ++it) mx = fmaxf(mx, sc[g][it]);
+      const float mnew = fmaxf(m[g], mx);
+      if (FULL || mnew != -INFINITY) {
+        const float corr = exp2f(m[g] - mnew);  // 0 while m is still -inf
+        l[g] *= corr;
+        const float2 c2 = make_float2(corr, corr);
+#pragma unroll
+        for (int i = 0; i < E2; ++i) acc[g][i] = __fmul2_rn(acc[g][i], c2);
+        m[g] = mnew;
+      }
+    }
+#pragma unroll
+    for (int it = 0; it < ITERS; ++it) {
+      const int ls = it * SPW + lane_slot;
+      float2 vf[E2];
+      load_row<T, HD, SB>(Vs + ls * HD, lane_part, vf);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        if (FULL || sc[g][it] != -INFINITY) {
+          const float pr = exp2f(sc[g][it] - m[g]);
+          l[g] += pr;
+          const float2 p2 = make_float2(pr, pr);
+#pragma unroll
+          for (int i = 0; i < E2; ++i) acc[g][i] = __ffma2_rn(p2, vf[i], acc[g][i]);
+        }
+      }
+    }
+  }
+
+  // The piece is complete: merge the SPW lane groups of the warp.
+  __device__ __forceinline__ void finish() {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      float M = m[g];
+#pragma unroll
+      for (int o = LPS; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+      const float w = (m[g] == -INFINITY) ? 0.f : exp2f(m[g] - M);
+      float Ls = l[g] * w;
+#pragma unroll
+      for (int o = LPS; o < 32; o <<= 1) Ls += __shfl_xor_sync(0xFFFFFFFFu, Ls, o);
+#pragma unroll
+      for (int i = 0; i < E2; ++i) {
+        float2 a = __fmul2_rn(acc[g][i], make_float2(w, w));
+#pragma unroll
+        for (int o = LPS; o < 32; o <<= 1) {
+          a.x += __shfl_xor_sync(0xFFFFFFFFu, a.x, o);
+          a.y += __shfl_xor_sync(0xFFFFFFFFu, a.y, o);
+        }
+        acc[g][i] = a;
+      }
+      m[g] = M;
+      l[g] = Ls;
+    }
+  }
+
+  // The G output rows, normalised (lanes of slot group 0 own vectors lane,
+  // lane + LPS, ...).
+  __device__ __forceinline__ void write_rows(T* rows, int lane) const {
+    if (lane >= LPS) return;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const float inv = l[g] > 0.f ? 1.f / l[g] : 0.f;
+#pragma unroll
+      for (int v = 0; v < SH::NVL; ++v) {
+        float o[SH::VEC];
+#pragma unroll
+        for (int i = 0; i < SH::VEC / 2; ++i) {
+          o[2 * i] = acc[g][v * SH::VEC / 2 + i].x * inv;
+          o[2 * i + 1] = acc[g][v * SH::VEC / 2 + i].y * inv;
+        }
+        store_vec<T>(rows + g * HD + (v * LPS + lane) * SH::VEC, o);
+      }
+    }
+  }
+  // A partial state: G x HD unnormalised outputs, then (max, sum) per head.
+  __device__ __forceinline__ void store_state(float* rec, int lane) const {
+    if (lane < LPS) {
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int v = 0; v < SH::NVL; ++v)
+#pragma unroll
+          for (int i = 0; i < SH::VEC / 2; ++i)
+            reinterpret_cast<float2*>(rec + g * HD + (v * LPS + lane) * SH::VEC)[i] =
+                acc[g][v * SH::VEC / 2 + i];
+    }
+    if (lane == 0) {
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        rec[G * HD + 2 * g] = m[g];
+        rec[G * HD + 2 * g + 1] = l[g];
+      }
+    }
+  }
 };
 
-// One pipeline stage of K/V rows for this warp's current piece.  FULL: every
-// slot of the stage is inside the sequence and on a fetched page, so no
-// masking is needed; otherwise masked slots never touch the sums (NaN-safe).
-template <typename T, int HD, int G, int SB, bool FULL>
-__device__ __forceinline__ void consume_stage(const T* Ks, const T* Vs, int lane_slot, int lane_part,
-                                              const float2 (&q2)[G][Shape<T, HD, SB>::EPL / 2],
-                                              float qscale, int valid_slots, uint64_t mask,
-                                              int log2P_in_stage, SoftState<T, HD, G, SB>& st) {
-  using SH = Shape<T, HD, SB>;
-  constexpr int SPW = SH::SPW, ITERS = SH::ITERS, E2 = SH::EPL / 2;
-  float sc[G][ITERS];
-#pragma unroll
-  for (int it = 0; it < ITERS; ++it) {
-    const int ls = it * SPW + lane_slot;
-    float2 kf[E2];
-    load_row<T, HD, SB>(Ks + ls * HD, lane_part, kf);
-    bool valid = true;
-    if (!FULL) valid = (ls < valid_slots) && ((mask >> (ls >> log2P_in_stage)) & 1ull);
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int i = 0; i < E2; ++i) a = __ffma2_rn(q2[g][i], kf[i], a);
-      float s = group_sum<SH::LPS>(a.x + a.y) * qscale;
-      sc[g][it] = valid ? s : -INFINITY;
-    }
-  }
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    float mx = sc[g][0];
-#pragma unroll
-    for (int it = 1; it < ITERS; ++it) mx = fmaxf(mx, sc[g][it]);
-    const float mnew = fmaxf(st.m[g], mx);
-    if (FULL || mnew != -INFINITY) {
-      const float corr = exp2f(st.m[g] - mnew);  // 0 while m is still -inf
-      st.l[g] *= corr;
-      const float2 c2 = make_float2(corr, corr);
-#pragma unroll
-      for (int i = 0; i < E2; ++i) st.acc[g][i] = __fmul2_rn(st.acc[g][i], c2);
-      st.m[g] = mnew;
-    }
-  }
-#pragma unroll
-  for (int it = 0; it < ITERS; ++it) {
-    const int ls = it * SPW + lane_slot;
-    float2 vf[E2];
-    load_row<T, HD, SB>(Vs + ls * HD, lane_part, vf);
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      if (FULL || sc[g][it] != -INFINITY) {
-        const float pr = exp2f(sc[g][it] - st.m[g]);
-        st.l[g] += pr;
-        const float2 p2 = make_float2(pr, pr);
-#pragma unroll
-        for (int i = 0; i < E2; ++i) st.acc[g][i] = __ffma2_rn(p2, vf[i], st.acc[g][i]);
-      }
-    }
-  }
-}
-
-// Write G rows of d outputs (lanes of slot group 0 own vectors lane, lane+8, ...).
+// Stage math of a launch: the tensor cores where a bf16 K/V row meets four
+// or more query heads (attn_uses_mma in internal.h).
 template <typename T, int HD, int G, int SB>
-__device__ __forceinline__ void write_rows(T* out_rows, int lane_part, const SoftState<T, HD, G, SB>& st) {
-  using SH = Shape<T, HD, SB>;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const float inv = st.l[g] > 0.f ? 1.f / st.l[g] : 0.f;
-#pragma unroll
-    for (int v = 0; v < SH::NVL; ++v) {
-      float o[SH::VEC];
-#pragma unroll
-      for (int i = 0; i < SH::VEC / 2; ++i) {
-        o[2 * i] = st.acc[g][v * SH::VEC / 2 + i].x * inv;
-        o[2 * i + 1] = st.acc[g][v * SH::VEC / 2 + i].y * inv;
+struct MathOf {
+  using type = VecMath<T, HD, G, SB>;
+};
+template <int HD, int SB>
+struct MathOf<__nv_bfloat16, HD, 4, SB> {
+  using type = MmaMath<HD, 4, Shape<__nv_bfloat16, HD, SB>::STAGE_SLOTS>;
+};
+template <int HD, int SB>
+struct MathOf<__nv_bfloat16, HD, 8, SB> {
+  using type = MmaMath<HD, 8, Shape<__nv_bfloat16, HD, SB>::STAGE_SLOTS>;
+};
+
+// Slots per bulk copy of K and of V (a copy never crosses a page), and the
+// place of slot `ls` in the V tile: whole stages where the tile is
+// contiguous, the four shifted blocks of MmaMath otherwise.
+template <typename MATH, int SLOTS>
+struct CopyShape {
+  static constexpr int kVRun = MATH::kPad > 0 ? SLOTS / 4 : SLOTS;
+  __device__ __forceinline__ static int v_shift(int ls) {
+    if constexpr (MATH::kPad > 0) return ls / kVRun * MATH::kSkew;
+    else return 0;
+  }
+};
+
+// One stage's copies, issued by all lanes of a warp together: slots s_begin
+// .. of one sequence (S slots long) and kv head into kd / vd, completing on
+// `bar` (with extra_bytes more to come).  page(i, o): page id of logical page i + o
+// (o per lane).  Returns the mask of V runs on valid pages, which `consume`
+// takes; bit i covers slots i * min(P, kVRun) ...
+template <typename MATH, typename T, int HD, int SLOTS, typename PageOf>
+__device__ __forceinline__ void copy_stage(const AttnParams& p, const T* kb, const T* vb, int s_begin,
+                                           int S, T* kd, T* vd, uint64_t* bar, uint64_t* mask_out,
+                                           uint32_t extra_bytes, uint64_t policy, int lane,
+                                           PageOf page) {
+  using CS = CopyShape<MATH, SLOTS>;
+  constexpr uint32_t ROW = HD * sizeof(T);
+  if (p.P >= SLOTS && CS::kVRun == SLOTS) {  // one copy of each
+    const int pg = page(s_begin >> p.log2P, 0);
+    if (lane == 0) {
+      const bool ok = pg >= 0 && pg < p.num_pages;
+      *mask_out = ok ? 1ull : 0ull;
+      if (!ok) report(p.status, WM_ERR_BOUNDS);
+      mbar_arrive_expect_tx(bar, (ok ? 2 * SLOTS * ROW : 0u) + extra_bytes);
+      if (ok) {
+        const int64_t off = (int64_t)pg * p.page_stride + (int64_t)(s_begin & (p.P - 1)) * HD;
+        bulk_g2s(kd, kb + off, SLOTS * ROW, bar, policy);
+        bulk_g2s(vd, vb + off, SLOTS * ROW, bar, policy);
       }
-      store_vec<T>(out_rows + g * HD + (v * SH::LPS + lane_part) * SH::VEC, o);
     }
+  } else {  // lane i copies the i-th run of V, and of K where one starts there
+    const int vr = min(p.P, CS::kVRun), kr = min(p.P, SLOTS);
+    const int slot = lane * vr, n = (min(SLOTS, S - s_begin) + vr - 1) / vr;  // runs (<= 32)
+    const int lp0 = s_begin >> p.log2P;
+    const int pg = page(lp0, lane < n ? ((s_begin + slot) >> p.log2P) - lp0 : 0);
+    const bool ok = lane < n && pg >= 0 && pg < p.num_pages;
+    const bool okk = ok && (slot & (kr - 1)) == 0;
+    const uint32_t mask = __ballot_sync(0xFFFFFFFFu, ok), maskk = __ballot_sync(0xFFFFFFFFu, okk);
+    if (lane == 0) {
+      *mask_out = mask;
+      if (__popc(mask) < n) report(p.status, WM_ERR_BOUNDS);
+      mbar_arrive_expect_tx(bar, (uint32_t)(vr * __popc(mask) + kr * __popc(maskk)) * ROW + extra_bytes);
+    }
+    __syncwarp();
+    const int64_t off = (int64_t)pg * p.page_stride + (int64_t)((s_begin + slot) & (p.P - 1)) * HD;
+    if (okk) bulk_g2s(kd + slot * HD, kb + off, (uint32_t)kr * ROW, bar, policy);
+    if (ok) bulk_g2s(vd + slot * HD + CS::v_shift(slot), vb + off, (uint32_t)vr * ROW, bar, policy);
   }
 }
 
 template <typename T, int HD, int G, int SB>
 __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn_kernel(const AttnParams p) {
   using SH = Shape<T, HD, SB>;
-  constexpr int VEC = SH::VEC, LPS = SH::LPS, E2 = SH::EPL / 2;
-  constexpr int STAGE_SLOTS = SH::STAGE_SLOTS, STAGE_ELEMS = SH::STAGE_ELEMS;
+  using MATH = typename MathOf<T, HD, G, SB>::type;
+  constexpr int STAGE_SLOTS = SH::STAGE_SLOTS;
+  constexpr int STAGE_ELEMS = SH::STAGE_ELEMS + MATH::kPad;        // of K, and of V, in the ring
   constexpr uint32_t KV_BYTES = STAGE_ELEMS * sizeof(T);
   constexpr uint32_t Q_BYTES = G * HD * sizeof(T);
   constexpr int REC = attn_part_rec(G, HD);                        // floats per partial record
@@ -244,8 +388,8 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* ring = reinterpret_cast<T*>(smem_raw);                       // [W][S][2][STAGE_ELEMS]
-  T* qring = ring + kWarps * kWStages * 2 * STAGE_ELEMS;          // [W][S][G*HD]
-  int* pre = reinterpret_cast<int*>(qring + kWarps * kWStages * G * HD);  // [B+1]
+  T* qring = ring + kWarps * kWStages * 2 * STAGE_ELEMS;          // [W][S][G*HD], if kQueryRing
+  int* pre = reinterpret_cast<int*>(qring + (MATH::kQueryRing ? kWarps * kWStages * G * HD : 0));  // [B+1]
   int* lens = pre + p.B + 1;                                      // [B]
   __shared__ uint64_t bars[kWarps][kWStages];
   __shared__ uint64_t qbars[kWarps];  // query of the warp's first piece
@@ -362,7 +506,6 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
   T* myring = ring + warp * kWStages * 2 * STAGE_ELEMS;
   T* myq = qring + warp * kWStages * G * HD;
   const uint64_t policy = l2_evict_first_policy();
-  const int lane_slot = lane / LPS, lane_part = lane % LPS;
 
   // ---- page-table window of the producer: lane i holds the page id of
   // logical page win0 + i (cur) and win0 + 32 + i (nxt) of sequence win_b.
@@ -416,44 +559,12 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     T* vd = kd + STAGE_ELEMS;
     uint64_t* bar = &bars[warp][buf];
     // the first piece's query arrives on qbars (issued after the dependency wait)
-    const bool with_q = first && pseq > 0;
+    const bool with_q = MATH::kQueryRing && first && pseq > 0;
     const uint32_t qb = with_q ? Q_BYTES : 0u;
     const T* qsrc = reinterpret_cast<const T*>(p.q) + ((int64_t)pc.b * p.Hq + pc.h * G) * HD;
-    if (p.P >= STAGE_SLOTS) {
-      const int pg = page_of(pc.b, s_begin >> p.log2P, 0);
-      if (lane == 0) {
-        const bool ok = pg >= 0 && pg < p.num_pages;
-        masks[warp][buf] = ok ? 1ull : 0ull;
-        if (!ok) report(p.status, WM_ERR_BOUNDS);
-        mbar_arrive_expect_tx(bar, (ok ? 2 * KV_BYTES : 0u) + qb);
-        if (ok) {
-          const int64_t off = (int64_t)pg * p.page_stride + (int64_t)(s_begin & (p.P - 1)) * HD;
-          bulk_g2s(kd, kb + off, KV_BYTES, bar, policy);
-          bulk_g2s(vd, vb + off, KV_BYTES, bar, policy);
-        }
-        if (with_q) bulk_g2s(myq + buf * G * HD, qsrc, Q_BYTES, bar, policy);
-      }
-    } else {
-      const int npp = STAGE_SLOTS >> p.log2P;  // pages per stage (<= 32)
-      const int lp0 = s_begin >> p.log2P;
-      const int lpn = min(npp, ((S - 1) >> p.log2P) - lp0 + 1);
-      const int pg = page_of(pc.b, lp0, lane < lpn ? lane : 0);
-      const bool ok = lane < lpn && pg >= 0 && pg < p.num_pages;
-      const uint32_t mask = __ballot_sync(FULLMASK, ok);
-      const uint32_t bytes = (uint32_t)p.P * HD * sizeof(T);
-      if (lane == 0) {
-        masks[warp][buf] = mask;
-        if (__popc(mask) < lpn) report(p.status, WM_ERR_BOUNDS);
-        mbar_arrive_expect_tx(bar, 2u * bytes * (uint32_t)__popc(mask) + qb);
-        if (with_q) bulk_g2s(myq + buf * G * HD, qsrc, Q_BYTES, bar, policy);
-      }
-      __syncwarp();
-      if (ok) {
-        const int64_t off = (int64_t)pg * p.page_stride;
-        bulk_g2s(kd + lane * p.P * HD, kb + off, bytes, bar, policy);
-        bulk_g2s(vd + lane * p.P * HD, vb + off, bytes, bar, policy);
-      }
-    }
+    copy_stage<MATH, T, HD, STAGE_SLOTS>(p, kb, vb, s_begin, S, kd, vd, bar, &masks[warp][buf], qb, policy,
+                                         lane, [&](int lp, int o) { return page_of(pc.b, lp, o); });
+    if (with_q && lane == 0) bulk_g2s(myq + buf * G * HD, qsrc, Q_BYTES, bar, policy);
     ++pseq;
     ++px;
     advance(pc, pre, B, Hkv);
@@ -490,20 +601,21 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
   for (int s = 0; s < kWStages && !p_done && px < pend; ++s) issue();
   if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (lane == 0) {
-    mbar_arrive_expect_tx(&qbars[warp], Q_BYTES);
-    bulk_g2s(myq, reinterpret_cast<const T*>(p.q) + ((int64_t)pc0.b * p.Hq + pc0.h * G) * HD,
-             Q_BYTES, &qbars[warp], policy);
+    mbar_arrive_expect_tx(&qbars[warp], MATH::kQueryRing ? Q_BYTES : 0u);
+    if (MATH::kQueryRing)
+      bulk_g2s(myq, reinterpret_cast<const T*>(p.q) + ((int64_t)pc0.b * p.Hq + pc0.h * G) * HD,
+               Q_BYTES, &qbars[warp], policy);
   }
   grab_issue();  // the next chunk, requested one ahead
 
   // ---- consumer
-  const int log2P_in_stage = p.P >= STAGE_SLOTS ? 30 : p.log2P;  // stage page index = slot >> this
-  const uint64_t all_pages = p.P >= STAGE_SLOTS ? 1ull : ((1ull << (STAGE_SLOTS >> p.log2P)) - 1ull);
+  constexpr int VRUN = CopyShape<MATH, STAGE_SLOTS>::kVRun;
+  const int log2R = __ffs(min(p.P, VRUN)) - 1;  // mask bit of a slot = slot >> this
+  const uint64_t all_pages = (1ull << (STAGE_SLOTS >> log2R)) - 1ull;
   int64_t c_chunk = gw;
   int64_t cx = chunk_begin(c_chunk), cend = chunk_end_x(c_chunk), cbeg = cx;
   Cursor cc = locate(cx, pre, B, Hkv);
-  float2 q2[G][E2];
-  SoftState<T, HD, G, SB> st;
+  MATH st;
   T* outp = reinterpret_cast<T*>(p.out);
 
   // ---- partial records of units that cross chunk boundaries.  The records
@@ -520,27 +632,6 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     return p.part + (j == 0 ? (int64_t)(p.max_chunks + gf) : (int64_t)(gf + j)) * REC;
   };
   auto flag_at = [&](float* r) -> int* { return reinterpret_cast<int*>(r + FLAG); };
-  // this warp's merged piece (registers) as a record
-  auto store_record = [&](float* po) {
-    float* pm = po + G * HD;
-    if (lane_slot == 0) {
-#pragma unroll
-      for (int g = 0; g < G; ++g)
-#pragma unroll
-        for (int v = 0; v < SH::NVL; ++v)
-#pragma unroll
-          for (int i = 0; i < VEC / 2; ++i)
-            reinterpret_cast<float2*>(po + g * HD + (v * LPS + lane_part) * VEC)[i] =
-                st.acc[g][v * VEC / 2 + i];
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        pm[2 * g] = st.m[g];
-        pm[2 * g + 1] = st.l[g];
-      }
-    }
-  };
   // every other piece has its ticket and at most its stores left: wait
   // (bounded) for their flags; false (and WM_ERR_TIMEOUT) if one never came
   auto wait_flags = [&](int gf, int np, int j_own) -> bool {
@@ -623,15 +714,12 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
       return;
     }
     if (cx == cbeg || cc.st == 0) {
-      const T* qs = myq + buf * G * HD;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        load_row<T, HD, SB>(qs + g * HD, lane_part, q2[g]);
-        st.m[g] = -INFINITY;
-        st.l[g] = 0.f;
-#pragma unroll
-        for (int i = 0; i < E2; ++i) st.acc[g][i] = make_float2(0.f, 0.f);
-      }
+      if constexpr (MATH::kQueryRing)
+        st.template load_q<false>(myq + buf * G * HD, lane);
+      else
+        st.template load_q<true>(reinterpret_cast<const T*>(p.q) + ((int64_t)cc.b * p.Hq + cc.h * G) * HD,
+                                 lane);
+      st.reset();
     }
     // A stage that ends a piece of a unit crossing chunk boundaries takes the
     // piece's ticket before its math, so the atomic's round trip overlaps it.
@@ -650,11 +738,9 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     const T* Ks = myring + buf * 2 * STAGE_ELEMS;
     const T* Vs = Ks + STAGE_ELEMS;
     if (valid_slots >= STAGE_SLOTS && mask == all_pages)
-      consume_stage<T, HD, G, SB, true>(Ks, Vs, lane_slot, lane_part, q2, p.qscale, valid_slots,
-                                        mask, log2P_in_stage, st);
+      st.template consume<true>(Ks, Vs, lane, p.qscale, valid_slots, mask, log2R);
     else
-      consume_stage<T, HD, G, SB, false>(Ks, Vs, lane_slot, lane_part, q2, p.qscale, valid_slots,
-                                         mask, log2P_in_stage, st);
+      st.template consume<false>(Ks, Vs, lane, p.qscale, valid_slots, mask, log2R);
     __syncwarp();  // every lane is done with this ring slot
     producer_step();
 
@@ -674,32 +760,10 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
       pend_np = 0;
     }
     if (piece_end) {
-      // merge the SPW lane groups of the warp
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        float M = st.m[g];
-#pragma unroll
-        for (int o = LPS; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(FULLMASK, M, o));
-        const float w = (st.m[g] == -INFINITY) ? 0.f : exp2f(st.m[g] - M);
-        float Ls = st.l[g] * w;
-#pragma unroll
-        for (int o = LPS; o < 32; o <<= 1) Ls += __shfl_xor_sync(FULLMASK, Ls, o);
-#pragma unroll
-        for (int i = 0; i < E2; ++i) {
-          float2 a = __fmul2_rn(st.acc[g][i], make_float2(w, w));
-#pragma unroll
-          for (int o = LPS; o < 32; o <<= 1) {
-            a.x += __shfl_xor_sync(FULLMASK, a.x, o);
-            a.y += __shfl_xor_sync(FULLMASK, a.y, o);
-          }
-          st.acc[g][i] = a;
-        }
-        st.m[g] = M;
-        st.l[g] = Ls;
-      }
+      st.finish();
       const int rowbase = cc.b * p.Hq + cc.h * G;
       if (g_first == g_last) {
-        if (lane_slot == 0) write_rows<T, HD, G, SB>(outp + (int64_t)rowbase * HD, lane_part, st);
+        st.write_rows(outp + (int64_t)rowbase * HD, lane);
       } else {
         const int gf = (int)g_first;
         const int np = (int)(g_last - g_first + 1);
@@ -710,7 +774,7 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
           // piece, its first): store the record now, read the ticket and
           // raise the flag (or merge) at the chunk's end instead of stalling
           // the stream in its middle.
-          store_record(rec_at(gf, j_own));
+          st.store_state(rec_at(gf, j_own), lane);
           pend_tk = tk;
           pend_np = np;
           pend_g = gf;
@@ -718,7 +782,7 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
         } else {
           const bool last = __shfl_sync(FULLMASK, tk, 0) == np - 1;
           if (!last) {
-            store_record(rec_at(gf, j_own));
+            st.store_state(rec_at(gf, j_own), lane);
             __syncwarp();
             if (lane == 0) st_release_gpu(flag_at(rec_at(gf, j_own)), p.epoch);
           } else if (wait_flags(gf, np, j_own)) {
@@ -761,24 +825,7 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
                 }
                 if (j_own >= r0 && j_own < r0 + n) {
                   // this warp's own piece was never published: take it from registers
-                  float* ro = rs + (j_own - r0) * REC;
-                  if (lane_slot == 0) {
-#pragma unroll
-                    for (int g = 0; g < G; ++g)
-#pragma unroll
-                      for (int v = 0; v < SH::NVL; ++v)
-#pragma unroll
-                        for (int i = 0; i < VEC / 2; ++i)
-                          reinterpret_cast<float2*>(ro + g * HD + (v * LPS + lane_part) * VEC)[i] =
-                              st.acc[g][v * VEC / 2 + i];
-                  }
-                  if (lane == 0) {
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                      ro[G * HD + 2 * g] = st.m[g];
-                      ro[G * HD + 2 * g + 1] = st.l[g];
-                    }
-                  }
+                  st.store_state(rs + (j_own - r0) * REC, lane);
                   __syncwarp();
                 }
 #pragma unroll
@@ -825,7 +872,7 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
             } else {
               // stages in flight: the same batches, straight from global
               // memory (this warp's own record first, for its other lanes)
-              store_record(rec_at(gf, j_own));
+              st.store_state(rec_at(gf, j_own), lane);
               __threadfence();
               __syncwarp();
               merge_global(gf, np, rowbase);

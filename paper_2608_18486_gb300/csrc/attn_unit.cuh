@@ -25,8 +25,9 @@ namespace wm {
 namespace attn_unit_detail {
 
 namespace cg = cooperative_groups;
+using attn_detail::CopyShape;
+using attn_detail::MathOf;
 using attn_detail::Shape;
-using attn_detail::SoftState;
 
 constexpr int kUStages = 3;  // ring depth per warp
 
@@ -42,22 +43,6 @@ constexpr int unit_warps() {
 // registers per SM)
 constexpr int unit_min_blocks(int nw) { return nw <= 4 ? 3 : nw <= 6 ? 2 : 1; }
 
-// A row of global memory another grid may just have written, as the stage
-// math reads it (lane part lp owns 16-byte vectors lp, lp + LPS, ...), through
-// L2 (ld.global.cg): no stale L1 line can be read.
-template <typename T, int HD, int SB>
-__device__ __forceinline__ void load_row_l2(const T* row, int lp,
-                                            float2 (&f)[Shape<T, HD, SB>::EPL / 2]) {
-  using SH = Shape<T, HD, SB>;
-#pragma unroll
-  for (int v = 0; v < SH::NVL; ++v) {
-    float t[SH::VEC];
-    Elem<T>::unpack(__ldcg(reinterpret_cast<const uint4*>(row + (v * SH::LPS + lp) * SH::VEC)), t);
-#pragma unroll
-    for (int i = 0; i < SH::VEC / 2; ++i) f[v * SH::VEC / 2 + i] = make_float2(t[2 * i], t[2 * i + 1]);
-  }
-}
-
 // floats of one partial state: G x HD unnormalised outputs, then (max, sum)
 // per query head (log2 units)
 constexpr int unit_rec(int G, int HD) { return G * HD + 2 * G; }
@@ -68,8 +53,9 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
     decode_attn_unit_kernel(const AttnParams p) {
   using SH = Shape<T, HD, SB>;
   constexpr int NW = unit_warps<T, HD, G, SB>();
-  constexpr int VEC = SH::VEC, LPS = SH::LPS, E2 = SH::EPL / 2;
-  constexpr int STAGE_SLOTS = SH::STAGE_SLOTS, STAGE_ELEMS = SH::STAGE_ELEMS;
+  using MATH = typename MathOf<T, HD, G, SB>::type;
+  constexpr int STAGE_SLOTS = SH::STAGE_SLOTS;
+  constexpr int STAGE_ELEMS = SH::STAGE_ELEMS + MATH::kPad;  // of K, and of V, in the ring
   constexpr uint32_t KV_BYTES = STAGE_ELEMS * sizeof(T);
   constexpr int E = G * HD;  // output elements of a unit
   constexpr int REC = unit_rec(G, HD);
@@ -147,39 +133,8 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
     T* vd = kd + STAGE_ELEMS;
     uint64_t* bar = &bars[warp][buf];
     const int s_begin = s * STAGE_SLOTS;
-    if (p.P >= STAGE_SLOTS) {
-      const int pg = page_of(s_begin >> p.log2P, 0);
-      if (lane == 0) {
-        const bool ok = pg >= 0 && pg < p.num_pages;
-        masks[warp][buf] = ok ? 1ull : 0ull;
-        if (!ok) report(p.status, WM_ERR_BOUNDS);
-        mbar_arrive_expect_tx(bar, ok ? 2 * KV_BYTES : 0u);
-        if (ok) {
-          const int64_t off = (int64_t)pg * p.page_stride + (int64_t)(s_begin & (p.P - 1)) * HD;
-          bulk_g2s(kd, kbase + off, KV_BYTES, bar, policy);
-          bulk_g2s(vd, vbase + off, KV_BYTES, bar, policy);
-        }
-      }
-    } else {
-      const int npp = STAGE_SLOTS >> p.log2P;  // pages per stage (<= 32)
-      const int lp0 = s_begin >> p.log2P;
-      const int lpn = min(npp, ((S - 1) >> p.log2P) - lp0 + 1);
-      const int pg = page_of(lp0, lane < lpn ? lane : 0);
-      const bool ok = lane < lpn && pg >= 0 && pg < p.num_pages;
-      const uint32_t mask = __ballot_sync(FULLMASK, ok);
-      const uint32_t bytes = (uint32_t)p.P * HD * sizeof(T);
-      if (lane == 0) {
-        masks[warp][buf] = mask;
-        if (__popc(mask) < lpn) report(p.status, WM_ERR_BOUNDS);
-        mbar_arrive_expect_tx(bar, 2u * bytes * (uint32_t)__popc(mask));
-      }
-      __syncwarp();
-      if (ok) {
-        const int64_t off = (int64_t)pg * p.page_stride;
-        bulk_g2s(kd + lane * p.P * HD, kbase + off, bytes, bar, policy);
-        bulk_g2s(vd + lane * p.P * HD, vbase + off, bytes, bar, policy);
-      }
-    }
+    attn_detail::copy_stage<MATH, T, HD, STAGE_SLOTS>(p, kbase, vbase, s_begin, S, kd, vd, bar,
+                                                      &masks[warp][buf], 0u, policy, lane, page_of);
   };
 
   int issued = 0;
@@ -187,25 +142,15 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
   if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // ---- stream this warp's stages
-  const int lane_slot = lane / LPS, lane_part = lane % LPS;
-  const int log2P_in_stage = p.P >= STAGE_SLOTS ? 30 : p.log2P;  // stage page index = slot >> this
-  const uint64_t all_pages = p.P >= STAGE_SLOTS ? 1ull : ((1ull << (STAGE_SLOTS >> p.log2P)) - 1ull);
-  SoftState<T, HD, G, SB> st;
-  float2 q2[G][E2];
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    st.m[g] = -INFINITY;
-    st.l[g] = 0.f;
-#pragma unroll
-    for (int i = 0; i < E2; ++i) st.acc[g][i] = make_float2(0.f, 0.f);
-  }
+  constexpr int VRUN = CopyShape<MATH, STAGE_SLOTS>::kVRun;
+  const int log2R = __ffs(min(p.P, VRUN)) - 1;  // mask bit of a slot = slot >> this
+  const uint64_t all_pages = (1ull << (STAGE_SLOTS >> log2R)) - 1ull;
+  MATH st;
+  st.reset();
   // the unit's G query rows, read through L2 after the dependency wait (the
   // previous grid may have written them)
-  if (nmine > 0) {
-    const T* qrow = reinterpret_cast<const T*>(p.q) + ((int64_t)b * p.Hq + h * G) * HD;
-#pragma unroll
-    for (int g = 0; g < G; ++g) load_row_l2<T, HD, SB>(qrow + g * HD, lane_part, q2[g]);
-  }
+  if (nmine > 0)
+    st.template load_q<true>(reinterpret_cast<const T*>(p.q) + ((int64_t)b * p.Hq + h * G) * HD, lane);
   bool alive = true;
   int done = 0;  // stages consumed
   for (; done < nmine && alive; ++done) {
@@ -221,11 +166,9 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
     const T* Ks = myring + buf * 2 * STAGE_ELEMS;
     const T* Vs = Ks + STAGE_ELEMS;
     if (valid_slots >= STAGE_SLOTS && mask == all_pages)
-      attn_detail::consume_stage<T, HD, G, SB, true>(Ks, Vs, lane_slot, lane_part, q2, p.qscale,
-                                                     valid_slots, mask, log2P_in_stage, st);
+      st.template consume<true>(Ks, Vs, lane, p.qscale, valid_slots, mask, log2R);
     else
-      attn_detail::consume_stage<T, HD, G, SB, false>(Ks, Vs, lane_slot, lane_part, q2, p.qscale,
-                                                      valid_slots, mask, log2P_in_stage, st);
+      st.template consume<false>(Ks, Vs, lane, p.qscale, valid_slots, mask, log2R);
     __syncwarp();  // every lane is done with this ring slot
     if (issued < nmine) issue(s0 + issued++);
   }
@@ -235,50 +178,13 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
     if (lane == 0)
       for (int y = done; y < issued; ++y) mbar_wait(&bars[warp][y % kUStages], (y / kUStages) & 1);
     __syncwarp();
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      st.m[g] = -INFINITY;
-      st.l[g] = 0.f;
-#pragma unroll
-      for (int i = 0; i < E2; ++i) st.acc[g][i] = make_float2(0.f, 0.f);
-    }
+    st.reset();
   }
 
-  // ---- merge the SPW lane groups of the warp, then store the warp's state
-  // in its (idle) ring
-  float* wrec = reinterpret_cast<float*>(myring);
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    float M = st.m[g];
-#pragma unroll
-    for (int o = LPS; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(FULLMASK, M, o));
-    const float w = (st.m[g] == -INFINITY) ? 0.f : exp2f(st.m[g] - M);
-    float Ls = st.l[g] * w;
-#pragma unroll
-    for (int o = LPS; o < 32; o <<= 1) Ls += __shfl_xor_sync(FULLMASK, Ls, o);
-#pragma unroll
-    for (int i = 0; i < E2; ++i) {
-      float2 a = __fmul2_rn(st.acc[g][i], make_float2(w, w));
-#pragma unroll
-      for (int o = LPS; o < 32; o <<= 1) {
-        a.x += __shfl_xor_sync(FULLMASK, a.x, o);
-        a.y += __shfl_xor_sync(FULLMASK, a.y, o);
-      }
-      st.acc[g][i] = a;
-    }
-    if (lane_slot == 0) {
-#pragma unroll
-      for (int v = 0; v < SH::NVL; ++v)
-#pragma unroll
-        for (int i = 0; i < VEC / 2; ++i)
-          reinterpret_cast<float2*>(wrec + g * HD + (v * LPS + lane_part) * VEC)[i] =
-              st.acc[g][v * VEC / 2 + i];
-    }
-    if (lane == 0) {
-      wrec[E + 2 * g] = M;
-      wrec[E + 2 * g + 1] = Ls;
-    }
-  }
+  // ---- merge the lanes of the warp, then store the warp's state in its
+  // (idle) ring
+  st.finish();
+  st.store_state(reinterpret_cast<float*>(myring), lane);
   __syncthreads();
 
   // ---- merge the CTA's NW warp states, element by element

@@ -60,6 +60,12 @@ constexpr int attn_ctas_per_sm(int stage_bytes, int G) { return stage_bytes == 4
 // one bulk copy.
 constexpr int attn_part_rec(int G, int d) { return G * d + (2 * G + 1 + 3) / 4 * 4; }
 
+// Launches whose stage math runs on the tensor cores (attn_mma.cuh): bf16
+// with four or eight query heads per kv head.  Their K and V tiles in shared
+// memory are kAttnMmaPad bytes longer.
+constexpr bool attn_uses_mma(int dtype, int G) { return dtype == WM_DT_BF16 && G >= 4; }
+constexpr int kAttnMmaPad = 128;
+
 int attn_stage_slots(int stage_bytes, int dtype, int d);
 int attn_warps_per_cta();
 size_t attn_smem_bytes(int stage_bytes, int dtype, int d, int G, int B);
