@@ -47,7 +47,7 @@
 // One launch at 32 heads of 128, two prompts of 8192 positions: 939 us before
 // (one item per CTA; every descriptor moved to uniform registers one by one,
 // 90 cycles per MMA; 16-byte row stores at the end), 773 us now; 6/3 heads of
-// 96, sixteen prompts of 2048: 126 and 86 us.
+// 96, sixteen prompts of 2048: 126 and 78 us.
 #include <math.h>
 
 #include "internal.h"
@@ -72,6 +72,7 @@ constexpr int kPThreads = (kSoftWarps + 4) * 32;
 constexpr int kSoftRegs = 208, kIssueRegs = 88;
 constexpr uint32_t kBlock = 128u * 128u;    // one 64-column block of a 128-row tile
 constexpr uint32_t kTmemCols = 512;         // S_i at 128 i (P over its first 64), O_i at 256 + 128 i
+constexpr int kAbsent = -2;                 // position of a row past the sequence's last
 constexpr float kStaleMax = 8.f;            // log2 headroom before O is rescaled
 constexpr float kStaleSum = 16384.f;        // ... as a sum of 64 probabilities
 constexpr uint32_t kStageBytes = 32 * 64;   // output staging of a softmax warp: 32 rows x 32 columns
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   __shared__ uint64_t sfull[kQT], pfull[kQT][2], odone[kQT];  // pfull: first, second half of P
   __shared__ uint32_t tmem_base;
   __shared__ Item items[2];
-  __shared__ int spos[2][kQT * kPM];        // positions of the item's rows (-1: absent or invalid)
+  __shared__ int spos[2][kQT * kPM];        // positions of the item's rows (-1: invalid, kAbsent: past Tq)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rows_item = p.pair ? kPM : kQT * kPM;
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
           const bool there = row < rows_item && r0 + row < p.Tq;
           const int v = there && ps[u] >= 0 && ps[u] < max_slots ? ps[u] : -1;
           bad |= there && v < 0;
-          if (row < rows_item) spos[slot][row] = v;
+          if (row < rows_item) spos[slot][row] = there ? v : kAbsent;
           if (u < kPM / 32) mx[0] = max(mx[0], v);
           else mx[1] = max(mx[1], v);
         }
@@ -505,7 +506,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
       if (!ok) break;
       const int n = items[slot].valid ? items[slot].nt[i] : -1;
       if (n < 0) break;
-      const int mypos = spos[slot][p.pair ? row : i * kPM + row];
+      // Absent rows are computed as the warp's last present one and never
+      // stored: on their own masks they held every tile to the masked path.
+      int mypos = spos[slot][p.pair ? row : i * kPM + row];
+      const int wpos = __reduce_max_sync(0xFFFFFFFFu, mypos);
+      if (mypos == kAbsent) mypos = wpos;
       float m = -INFINITY, l = 0.f;  // max used for P (log2 units) and running sum
       // tcgen05.ld / st are warp-collective: every lane of the warp issues each
       // one, and the wait outcomes are made warp-uniform before any branch
@@ -514,76 +519,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         if (!ok) break;
         ++cnt;
         tc::fence_after_sync();
-        // Visible slots of this row in the tile: e < vis (all 128 unless the
-        // diagonal crosses the tile).  The masked path only runs there.
-        const int vis = min(max(mypos - j * kPN + 1, 0), kPN);
-        const bool whole = __all_sync(0xFFFFFFFFu, vis == kPN);
-        uint32_t v[4][32];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tc::tmem_ld32(scol + 32 * c, v[c]);
-        tc::tmem_ld_wait();
-        // max of 64 scores (log2 units), two chains per 32 of them
-        auto half_max = [&](int half) {
-          float mc[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) mc[c] = -INFINITY;
-          if (whole) {
-#pragma unroll
-            for (int e = 0; e < 16; e += 2)
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const int cc = 2 * half + (c >> 1), o = 16 * (c & 1) + e;
-                mc[c] = max3(mc[c], __uint_as_float(v[cc][o]), __uint_as_float(v[cc][o + 1]));
-              }
-          } else {
-#pragma unroll
-            for (int e = 0; e < 16; ++e)
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                const int cc = 2 * half + (c >> 1), o = 16 * (c & 1) + e;
-                if (32 * cc + o < vis) mc[c] = fmaxf(mc[c], __uint_as_float(v[cc][o]));
-              }
-          }
-          // qscale > 0: the max commutes with the scale
-          return fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3])) * p.qscale;
-        };
-        // Half of P (64 slots): p = 2^(s * qscale - m) in pairs; masked slots
-        // (and rows with nothing visible yet) give 0.  w: packed pairs.
-        float2 sum2[4];
-        auto half_p = [&](int half, uint32_t (&w)[2][16]) {
-          const float2 qs2 = make_float2(p.qscale, p.qscale), nm2 = make_float2(-m, -m);
-          const bool live = m != -INFINITY;
-          const bool open = whole && __all_sync(0xFFFFFFFFu, live);
-          const int lim0 = live ? vis - 64 * half : 0;
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int cc = 2 * half + c, lim = lim0 - 32 * c;
-            sum2[cc] = make_float2(0.f, 0.f);
-            if (open) {
-#pragma unroll
-              for (int e = 0; e < 32; e += 2) {
-                const float2 x = __ffma2_rn(
-                    make_float2(__uint_as_float(v[cc][e]), __uint_as_float(v[cc][e + 1])), qs2, nm2);
-                const float2 pr = make_float2(ex2(x.x), ex2(x.y));
-                sum2[cc] = __fadd2_rn(sum2[cc], pr);
-                const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
-                w[c][e / 2] = *reinterpret_cast<const uint32_t*>(&h);
-              }
-            } else {
-#pragma unroll
-              for (int e = 0; e < 32; e += 2) {
-                const float2 x = __ffma2_rn(
-                    make_float2(__uint_as_float(v[cc][e]), __uint_as_float(v[cc][e + 1])), qs2, nm2);
-                const float2 pr =
-                    make_float2(e < lim ? ex2(x.x) : 0.f, e + 1 < lim ? ex2(x.y) : 0.f);
-                sum2[cc] = __fadd2_rn(sum2[cc], pr);
-                const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
-                w[c][e / 2] = *reinterpret_cast<const uint32_t*>(&h);
-              }
-            }
-          }
-        };
-        // P goes over the S columns (all read above), slots 2c, 2c + 1 in column c
+        // P goes over the S columns, slots 2c, 2c + 1 in column c
         auto hand_over = [&](int half, const uint32_t (&w)[2][16]) {
           tc::tmem_st16(scol + 32 * half, w[0]);
           tc::tmem_st16(scol + 32 * half + 16, w[1]);
@@ -593,6 +529,65 @@ __global__ void __launch_bounds__(kPThreads, 1)
           if (lane == 0) mbar_arrive(&pfull[i][half]);
         };
         uint32_t w[2][16];
+        if (wpos < j * kPN) {  // no row of the warp sees the tile (or none is present)
+#pragma unroll
+          for (int e = 0; e < 16; ++e) w[0][e] = w[1][e] = 0u;
+          hand_over(0, w);
+          hand_over(1, w);
+          continue;
+        }
+        uint32_t v[4][32];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc::tmem_ld32(scol + 32 * c, v[c]);
+        tc::tmem_ld_wait();
+        // Slots past the row's position become -inf (all 128 are visible unless
+        // the diagonal crosses the tile; 32 columns at a time).
+        const int vis = mypos - j * kPN + 1;
+        if (!__all_sync(0xFFFFFFFFu, vis >= kPN)) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (!__all_sync(0xFFFFFFFFu, vis >= 32 * c + 32)) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (32 * c + e >= vis) v[c][e] = __float_as_uint(-INFINITY);
+            }
+        }
+        // max of 64 scores (log2 units), two chains per 32 of them
+        auto half_max = [&](int half) {
+          float mc[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mc[c] = -INFINITY;
+#pragma unroll
+          for (int e = 0; e < 16; e += 2)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const int cc = 2 * half + (c >> 1), o = 16 * (c & 1) + e;
+              mc[c] = max3(mc[c], __uint_as_float(v[cc][o]), __uint_as_float(v[cc][o + 1]));
+            }
+          // qscale > 0: the max commutes with the scale
+          return fmaxf(fmaxf(mc[0], mc[1]), fmaxf(mc[2], mc[3])) * p.qscale;
+        };
+        // Half of P (64 slots): p = 2^(s * qscale - m) in pairs; masked slots give
+        // 0 (also while the row's max is -inf).  w: packed pairs.
+        float2 sum2[4];
+        auto half_p = [&](int half, uint32_t (&w)[2][16]) {
+          const float nm = m == -INFINITY ? 0.f : -m;
+          const float2 qs2 = make_float2(p.qscale, p.qscale), nm2 = make_float2(nm, nm);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int cc = 2 * half + c;
+            sum2[cc] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < 32; e += 2) {
+              const float2 x = __ffma2_rn(
+                  make_float2(__uint_as_float(v[cc][e]), __uint_as_float(v[cc][e + 1])), qs2, nm2);
+              const float2 pr = make_float2(ex2(x.x), ex2(x.y));
+              sum2[cc] = __fadd2_rn(sum2[cc], pr);
+              const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
+              w[c][e / 2] = *reinterpret_cast<const uint32_t*>(&h);
+            }
+          }
+        };
         if (j == 0) m = fmaxf(half_max(0), half_max(1));
         half_p(0, w);
         if (j > 0) {
