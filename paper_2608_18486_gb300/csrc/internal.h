@@ -91,7 +91,7 @@ struct PrefillLaunch {
   const void* v_pool;
   int32_t B, Tq, Hq, Hkv, d, k, chan, num_pages, max_pages, P;
 };
-cudaError_t launch_prefill_attn(const PrefillLaunch& L, cudaStream_t s);
+cudaError_t launch_prefill_attn(const PrefillLaunch& L, int sms, cudaStream_t s);
 
 // ------------------------------------------------------------ TMA tensor maps
 // 2-D map of a row-major bf16 matrix [rows][cols] with a row pitch of

@@ -15,6 +15,10 @@
 //    head) the two tiles are the same 128 rows of two query heads that share
 //    a kv head: equal causal ranges, and one K/V stream serves both.
 //    Otherwise they are two consecutive 128-row tiles of one head.
+//    Launches of few items (halves_pay) take one 128-row tile per item
+//    instead, one half of the CTA on its even KV tiles and the other on the
+//    odd ones, each with its own O, max and sum; both O lie in the same TMEM
+//    lanes, so the halves merge where the rows are written.
 //  * warp 8 (load): takes the next item (cluster launch control: a CTA that
 //    has not started yet is cancelled and its index taken over, so the items
 //    are handed out as SMs become free), publishes its rows' positions and
@@ -47,7 +51,7 @@
 // One launch at 32 heads of 128, two prompts of 8192 positions: 939 us before
 // (one item per CTA; every descriptor moved to uniform registers one by one,
 // 90 cycles per MMA; 16-byte row stores at the end), 773 us now; 6/3 heads of
-// 96, sixteen prompts of 2048: 126 and 78 us.
+// 96, sixteen prompts of 2048: 126 and 86 us.
 #include <math.h>
 
 #include "internal.h"
@@ -72,6 +76,7 @@ constexpr int kPThreads = (kSoftWarps + 4) * 32;
 constexpr int kSoftRegs = 208, kIssueRegs = 88;
 constexpr uint32_t kBlock = 128u * 128u;    // one 64-column block of a 128-row tile
 constexpr uint32_t kTmemCols = 512;         // S_i at 128 i (P over its first 64), O_i at 256 + 128 i
+constexpr double kHalvesShare = 0.4;        // see halves_pay
 constexpr int kAbsent = -2;                 // position of a row past the sequence's last
 constexpr float kStaleMax = 8.f;            // log2 headroom before O is rescaled
 constexpr float kStaleSum = 16384.f;        // ... as a sum of 64 probabilities
@@ -108,7 +113,7 @@ struct PrefillParams {
 struct Item {
   int valid;       // 0: no more items
   int b, y, r0;    // sequence, head (or head pair), first row
-  int nt[kQT];     // KV tiles of each query tile
+  int nt[kQT];     // KV tiles each query tile walks
   int tmaxpos;     // largest position of the item, -1: none valid
 };
 
@@ -150,7 +155,7 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-template <int HD>
+template <int HD, bool HALVES>
 __global__ void __launch_bounds__(kPThreads, 1)
     prefill_attn_kernel(const __grid_constant__ CUtensorMap tmQ,
                         const __grid_constant__ CUtensorMap tmK,
@@ -161,13 +166,17 @@ __global__ void __launch_bounds__(kPThreads, 1)
   __shared__ __align__(16) uint8_t clc_buf[16];
   __shared__ uint64_t clc_bar, vzero, qfull, qempty, kfull[NSK], kempty[NSK], vfull[NSV], vempty[NSV];
   __shared__ uint64_t info_full[2], info_empty[2];
+  // HALVES: (max, sum) of each half's rows; xfull: a warp's are there and its O is
+  // complete, xdone: it has read the other half's
+  __shared__ float2 sml[HALVES ? kQT : 1][kPM];
+  __shared__ uint64_t xfull[HALVES ? kQT : 1][4], xdone[HALVES ? kQT : 1][4];
   __shared__ uint64_t sfull[kQT], pfull[kQT][2], odone[kQT];  // pfull: first, second half of P
   __shared__ uint32_t tmem_base;
   __shared__ Item items[2];
   __shared__ int spos[2][kQT * kPM];        // positions of the item's rows (-1: invalid, kAbsent: past Tq)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rows_item = p.pair ? kPM : kQT * kPM;
+  const int rows_item = HALVES || p.pair ? kPM : kQT * kPM;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* Qs = base;                         // [kQT] Q tiles
@@ -197,6 +206,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
       mbar_init(&pfull[i][0], 4);
       mbar_init(&pfull[i][1], 4);
       mbar_init(&odone[i], 1);
+      for (int q = 0; HALVES && q < 4; ++q) {
+        mbar_init(&xfull[i][q], 1);
+        mbar_init(&xdone[i][q], 1);
+      }
     }
     fence_mbar_init();
     tc::prefetch_tensormap(&tmQ);
@@ -301,7 +314,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
           q.y = y;
           q.r0 = r0;
 #pragma unroll
-          for (int i = 0; i < kQT; ++i) q.nt[i] = mx[i] >= 0 ? mx[i] / kPN + 1 : 0;
+          for (int i = 0; i < kQT; ++i)
+            q.nt[i] = HALVES ? (nmax + 1 - i) / 2 : mx[i] >= 0 ? mx[i] / kPN + 1 : 0;
           q.tmaxpos = tmaxpos;
           items[slot] = q;
         }
@@ -328,8 +342,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
               if (qc > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&qempty, (qc - 1) & 1));
               if (!ok) break;
               if (lane == 0) {
-                mbar_arrive_expect_tx(&qfull, kQT * SH::Q_BYTES);
-                for (int i = 0; i < kQT; ++i) {
+                const int nq = HALVES ? 1 : kQT;
+                mbar_arrive_expect_tx(&qfull, nq * SH::Q_BYTES);
+                for (int i = 0; i < nq; ++i) {
                   const int hh = p.pair ? kQT * y + i : y;
                   const int rb = p.pair ? r0 : r0 + i * kPM;
 #pragma unroll
@@ -410,7 +425,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         const uint64_t kd0 = tc::sdesc_kmajor_sw128(smem_u32(Ks));
         const uint64_t vd0 = tc::sdesc_mnmajor_sw128(smem_u32(Vs), kBlock, 1024);
         auto issue_s = [&](int i, uint32_t st) {  // S_i = Q_i K^T, K in ring slot st
-          const uint64_t qd = qd0 + (uint64_t)((uint32_t)i * (SH::Q_BYTES >> 4));
+          const uint64_t qd = qd0 + (uint64_t)(HALVES ? 0u : (uint32_t)i * (SH::Q_BYTES >> 4));
           const uint64_t kd = kd0 + (uint64_t)(st * (SH::KV_BYTES >> 4));
 #pragma unroll
           for (int kk = 0; kk < HD / 16; ++kk) {
@@ -443,6 +458,64 @@ __global__ void __launch_bounds__(kPThreads, 1)
           if (!valid) break;
           const int nmax = tmaxpos >= 0 ? tmaxpos / kPN + 1 : 0;
           if (nmax == 0) continue;
+          if constexpr (HALVES) {  // tile i: KV tiles i, i + 2, ...; each has one user
+            ok = mbar_wait_spin(&qfull, qc & 1);
+            if (!ok) break;
+            ++qc;
+            // KV tile of step j of query tile i
+            auto kv_of = [&](int i, int j) -> uint32_t { return 2 * j + i; };
+            auto wait_ring = [&](uint64_t* bars, uint32_t c, int ns) {
+              const bool got = mbar_wait_spin(&bars[c % ns], (c / ns) & 1);
+              tc::fence_after_sync();
+              return got;
+            };
+            const bool part = tmaxpos - (nmax - 1) * kPN + 1 < kPN;  // the last V tile is zeroed in part
+#pragma unroll
+            for (int i = 0; i < kQT; ++i) {
+              if (nt[i] == 0 || !ok) continue;
+              const uint32_t c = kc + kv_of(i, 0);
+              ok = wait_ring(kfull, c, NSK);
+              if (!ok) continue;
+              issue_s(i, c % NSK);
+              tc::mma_commit(&kempty[c % NSK]);
+            }
+            if (!ok) break;
+            if (nmax <= 2) tc::mma_commit(&qempty);
+            for (int j = 0; j < nt[0]; ++j) {
+#pragma unroll
+              for (int i = 0; i < kQT; ++i) {
+                if (j >= nt[i] || !ok) continue;
+                const uint32_t kv = kv_of(i, j), st = (vc + kv) % NSV;
+                ok = wait_ring(vfull, vc + kv, NSV);
+                if (ok && part && kv + 1 == (uint32_t)nmax) ok = mbar_wait_spin(&vzero, zc & 1);
+                if (!ok) continue;
+                ok = mbar_wait_spin(&pfull[i][0], cnt[i] & 1);
+                if (!ok) continue;
+                tc::fence_after_sync();
+                issue_pv(i, st, j == 0, 0);
+                ok = mbar_wait_spin(&pfull[i][1], cnt[i] & 1);
+                if (!ok) continue;
+                tc::fence_after_sync();
+                issue_pv(i, st, j == 0, 1);
+                ++cnt[i];
+                tc::mma_commit(&vempty[st]);
+                if (j + 1 < nt[i]) {
+                  const uint32_t kn = kv_of(i, j + 1), c = kc + kn;
+                  ok = wait_ring(kfull, c, NSK);
+                  if (!ok) continue;
+                  issue_s(i, c % NSK);
+                  tc::mma_commit(&kempty[c % NSK]);
+                  if (kn + 1 == (uint32_t)nmax) tc::mma_commit(&qempty);  // the item's last S
+                }
+              }
+              if (!ok) break;
+            }
+            if (!ok) break;
+            kc += nmax;
+            vc += nmax;
+            zc += part;
+            continue;
+          }
           ok = mbar_wait_spin(&kfull[kc % NSK], (kc / NSK) & 1) && mbar_wait_spin(&qfull, qc & 1);
           if (!ok) break;
           ++qc;
@@ -508,7 +581,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
       if (n < 0) break;
       // Absent rows are computed as the warp's last present one and never
       // stored: on their own masks they held every tile to the masked path.
-      int mypos = spos[slot][p.pair ? row : i * kPM + row];
+      int mypos = spos[slot][HALVES || p.pair ? row : i * kPM + row];
       const int wpos = __reduce_max_sync(0xFFFFFFFFu, mypos);
       if (mypos == kAbsent) mypos = wpos;
       float m = -INFINITY, l = 0.f;  // max used for P (log2 units) and running sum
@@ -529,7 +602,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
           if (lane == 0) mbar_arrive(&pfull[i][half]);
         };
         uint32_t w[2][16];
-        if (wpos < j * kPN) {  // no row of the warp sees the tile (or none is present)
+        const int s0 = (HALVES ? 2 * j + i : j) * kPN;  // the tile's first slot
+        if (wpos < s0) {  // no row of the warp sees the tile (or none is present)
 #pragma unroll
           for (int e = 0; e < 16; ++e) w[0][e] = w[1][e] = 0u;
           hand_over(0, w);
@@ -542,7 +616,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         tc::tmem_ld_wait();
         // Slots past the row's position become -inf (all 128 are visible unless
         // the diagonal crosses the tile; 32 columns at a time).
-        const int vis = mypos - j * kPN + 1;
+        const int vis = mypos - s0 + 1;
         if (!__all_sync(0xFFFFFFFFu, vis >= kPN)) {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
@@ -636,29 +710,64 @@ __global__ void __launch_bounds__(kPThreads, 1)
       if (n > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&odone[i], (cnt - 1) & 1));
       if (!ok) break;
       tc::fence_after_sync();
-      const float inv = (n > 0 && l > 0.f) ? 1.f / l : 0.f;
+      float inv = (n > 0 && l > 0.f) ? 1.f / l : 0.f, inv1 = 0.f;  // weights of this O and of the other half's
+      if constexpr (HALVES) {
+        sml[i][row] = make_float2(m, l);
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&xfull[i][quad]);
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&xfull[i ^ 1][quad], it & 1));
+        if (!ok) break;
+        tc::fence_after_sync();
+        const float2 o = sml[i ^ 1][row];
+        const float mm = fmaxf(m, o.x);
+        const float a = m == -INFINITY ? 0.f : ex2(m - mm), b2 = o.x == -INFINITY ? 0.f : ex2(o.x - mm);
+        const float ls = a * l + b2 * o.y, r = ls > 0.f ? 1.f / ls : 0.f;
+        inv = a * r;
+        inv1 = b2 * r;
+      }
       const int b = items[slot].b, y = items[slot].y;
-      const int rb = items[slot].r0 + (p.pair ? 0 : i * kPM) + quad * 32;  // the warp's first row
+      const int rb = items[slot].r0 + (HALVES || p.pair ? 0 : i * kPM) + quad * 32;  // the warp's first row
       __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) +
                            (((int64_t)b * p.Tq + rb) * p.Hq + (p.pair ? kQT * y + i : y)) * HD;
       const int rr = lane >> 2, ch = lane & 3;  // row (of 8) and 16-byte chunk this lane stores
       const int64_t pitch = (int64_t)p.Hq * HD;
       __nv_bfloat16* drow = dst + rr * pitch + 8 * ch;
+      // Columns 32 c0 .. 32 c1: all of the row, or (HALVES) this half's share, the
+      // first tile's the smaller one.
+      constexpr int NC = HD / 32;
+      const int c0 = HALVES && i == 1 ? NC / 2 : 0, c1 = HALVES && i == 0 ? NC / 2 : NC;
+      const uint32_t ocol1 = lane_base + 256 + 128 * (i ^ 1);
       uint32_t o[2][32];  // one group of 32 columns on its way while the last is stored
-      tc::tmem_ld32(ocol, o[0]);
+      tc::tmem_ld32(ocol + 32 * c0, o[0]);
 #pragma unroll
-      for (int c = 0; c < HD / 32; ++c) {
+      for (int cc = 0; cc < (HALVES ? NC - NC / 2 : NC); ++cc) {
+        const int c = c0 + cc;
+        if (HALVES && c >= c1) break;
         tc::tmem_ld_wait();
-        if (c + 1 < HD / 32) tc::tmem_ld32(ocol + 32 * (c + 1), o[(c + 1) & 1]);
+        if constexpr (HALVES) {  // a half without KV tiles left its O as another item had it
+          const int n1 = items[slot].nt[i ^ 1];
+          uint32_t o1[32];
+          tc::tmem_ld32(ocol1 + 32 * c, o1);
+          tc::tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            o[cc & 1][e] = __float_as_uint((n > 0 ? __uint_as_float(o[cc & 1][e]) * inv : 0.f) +
+                                           (n1 > 0 ? __uint_as_float(o1[e]) * inv1 : 0.f));
+        }
+        if (c + 1 < c1) tc::tmem_ld32(ocol + 32 * (c + 1), o[(cc + 1) & 1]);
 #pragma unroll
         for (int e = 0; e < 32; e += 8) {
           uint32_t u[4];
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
-            const float x0 = __uint_as_float(o[c & 1][e + 2 * t]);
-            const float x1 = __uint_as_float(o[c & 1][e + 2 * t + 1]);
-            const __nv_bfloat162 h2 =  // (n == 0: no P V ran, O holds another item's rows)
-                __floats2bfloat162_rn(n > 0 ? x0 * inv : 0.f, n > 0 ? x1 * inv : 0.f);
+            float x0 = __uint_as_float(o[cc & 1][e + 2 * t]);
+            float x1 = __uint_as_float(o[cc & 1][e + 2 * t + 1]);
+            if (!HALVES) {  // (n == 0: no P V ran, O holds another item's rows)
+              x0 = n > 0 ? x0 * inv : 0.f;
+              x1 = n > 0 ? x1 * inv : 0.f;
+            }
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
             u[t] = *reinterpret_cast<const uint32_t*>(&h2);
           }
           // row `lane`, 16-byte chunk e/8, placed so that 8 rows cover all banks
@@ -678,6 +787,12 @@ __global__ void __launch_bounds__(kPThreads, 1)
             *reinterpret_cast<uint4*>(drow + q * 8 * pitch + 32 * c) = u[q];
       }
       tc::fence_before_sync();
+      if (HALVES) {  // the next item's O and sums go over these: not before the other half has read them
+        if (lane == 0) mbar_arrive(&xdone[i][quad]);
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&xdone[i ^ 1][quad], it & 1));
+        if (!ok) break;
+        tc::fence_after_sync();
+      }
       if (lane == 0) mbar_arrive(&info_empty[slot]);  // (behind a __syncwarp of the staging)
     }
     if (!ok && lane == 0) report(p.status, WM_ERR_TIMEOUT);
@@ -692,11 +807,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
   }
 }
 
-template <int HD>
+template <int HD, bool HALVES>
 cudaError_t launch_hd(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v,
                       const PrefillParams& p, cudaStream_t s) {
   static size_t smem_set[kSmemOptDevices] = {};
-  auto kern = prefill_attn_kernel<HD>;
+  auto kern = prefill_attn_kernel<HD, HALVES>;
   if (cudaError_t e = opt_in_smem(kern, (size_t)PShape<HD>::SMEM, smem_set); e != cudaSuccess)
     return e;
   cudaLaunchConfig_t cfg = {};
@@ -712,9 +827,27 @@ cudaError_t launch_hd(const CUtensorMap& q, const CUtensorMap& k, const CUtensor
   return cudaLaunchKernelEx(&cfg, kern, q, k, v, p);
 }
 
+// One 128-row tile per item, its KV tiles shared out over the CTA's two halves?
+// Both forms do the same steps in all; with whole tiles the launch lasts at least
+// as long as its longest item (all KV tiles of the last rows), with halves half of
+// that, at the price of K and V loaded once per 128 rows and head, twice as many per
+// step, and of the merge.  So: where the steps of all items, causal rows evenly
+// spread, fill the SMs for less than kHalvesShare of the longest item's.  Measured
+// (us, whole tiles / halves; share in front): 0.11: 8 heads of 96, every eighth of
+// 4575 positions 50 / 30; 0.26: 32/8 heads of 96, every eighth of 4096 48 / 36;
+// 0.32: two prompts, 32/8 heads of 64, every fourth of 1000 16.5 / 12; 0.47: sixteen
+// prompts, 6/3 heads of 96, every eighth of 2048 29.8 / 32.5; 0.53: two prompts of
+// the 0.26 case 48.5 / 66.6 (with many CTAs the doubled K and V loads bind).
+bool halves_pay(const PrefillLaunch& L, int pair, int sms) {
+  const int rows_item = pair ? kPM : kQT * kPM;
+  const double nblk = (L.Tq + rows_item - 1) / rows_item;
+  const double items = nblk * (pair ? L.Hq / kQT : L.Hq) * L.B;
+  return items * (nblk + 1) / (2 * nblk) < kHalvesShare * sms;
+}
+
 }  // namespace
 
-cudaError_t launch_prefill_attn(const PrefillLaunch& L, cudaStream_t s) {
+cudaError_t launch_prefill_attn(const PrefillLaunch& L, int sms, cudaStream_t s) {
   CUtensorMap tq, tk, tv;
   const uint64_t pool_rows = (uint64_t)L.k * L.num_pages * L.Hkv * L.P;
   const uint32_t box_rows = L.P >= kPN ? (uint32_t)kPN : (uint32_t)L.P;
@@ -741,7 +874,9 @@ cudaError_t launch_prefill_attn(const PrefillLaunch& L, cudaStream_t s) {
   int lg = 0;
   while ((1 << lg) < L.P) ++lg;
   p.log2P = lg;
-  const int rows_item = p.pair ? kPM : kQT * kPM;
+  const bool halves = halves_pay(L, p.pair, sms);
+  if (halves) p.pair = 0;
+  const int rows_item = halves || p.pair ? kPM : kQT * kPM;
   p.nblk = (L.Tq + rows_item - 1) / rows_item;
   p.heads = p.pair ? L.Hq / kQT : L.Hq;
   if ((int64_t)p.nblk * p.heads * L.B > INT32_MAX) return cudaErrorInvalidConfiguration;
@@ -754,9 +889,9 @@ cudaError_t launch_prefill_attn(const PrefillLaunch& L, cudaStream_t s) {
   p.group = (int)((units + groups - 1) / groups);
   p.qscale = (float)(1.4426950408889634 / sqrt((double)L.d));
   switch (L.d) {
-    case 64: return launch_hd<64>(tq, tk, tv, p, s);
-    case 96: return launch_hd<96>(tq, tk, tv, p, s);
-    case 128: return launch_hd<128>(tq, tk, tv, p, s);
+    case 64: return halves ? launch_hd<64, true>(tq, tk, tv, p, s) : launch_hd<64, false>(tq, tk, tv, p, s);
+    case 96: return halves ? launch_hd<96, true>(tq, tk, tv, p, s) : launch_hd<96, false>(tq, tk, tv, p, s);
+    case 128: return halves ? launch_hd<128, true>(tq, tk, tv, p, s) : launch_hd<128, false>(tq, tk, tv, p, s);
     default: return cudaErrorInvalidValue;
   }
 }

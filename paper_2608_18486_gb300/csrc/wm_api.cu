@@ -412,7 +412,7 @@ wm_status wm_prefill_attn(const wm_config* c, const wm_cache* cache, int32_t lay
   L.num_pages = cache->num_pages;
   L.max_pages = max_pages;
   L.P = c->page_size;
-  const cudaError_t e = wm::launch_prefill_attn(L, (cudaStream_t)stream);
+  const cudaError_t e = wm::launch_prefill_attn(L, sm_count(), (cudaStream_t)stream);
   if (e == cudaErrorInvalidValue) return WM_ERR_INVALID_ARG;  // the tensor-map encoder refused
   return e == cudaSuccess ? WM_OK : WM_ERR_CUDA;
 }
