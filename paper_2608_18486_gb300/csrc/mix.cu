@@ -105,7 +105,7 @@ __device__ __forceinline__ void store8f<__nv_bfloat16>(__nv_bfloat16* dst, const
 // 8-element vectors) in registers between the sum of squares and the two router
 // inputs, so the row is read once, 16 bytes at a time.  Bound by memory and, in a
 // decode step, by the latency of that one read (the kernel it replaces read 2
-// bytes per load, twice: 17 us at 32 tokens, L = 32, D = 4096; this one PREUS).
+// bytes per load, twice: 17 us at 32 tokens, L = 32, D = 4096; this one: 7 us).
 constexpr int kPrenormWarps = 4;
 
 template <typename T, int WPR>
@@ -272,6 +272,112 @@ __global__ void __launch_bounds__(256) gemm_wxT_simt(const GemmArgs a) {
       if (m < a.M) out[(int64_t)n * a.M + m] = acc[i][j];
     }
   }
+}
+
+// The same product for few tokens of fp32: a decode step of a small batch reads
+// every weight once for a handful of multiply-adds, so it is a stream of W (and,
+// at small sizes, one chain of load latencies).  A warp takes R weight rows at a
+// time against NT tokens, a lane every 32nd 16-byte vector of them, U of each row
+// in flight and the next U requested before these are used; the first ones before
+// the dependency wait (no kernel of the step writes weights), and past L1.  The
+// tokens' vectors come through L1, which the CTA's warps share; with more tokens
+// than NT the CTAs of all token groups of a row block are neighbours, so W comes
+// from HBM once.  Four rows where a token group is wide: that halves the loads of
+// tokens, which bind there.  The tiled kernel above, two barriers per 32 elements
+// of K and ceil(M / 64) CTAs per split, has 32 tokens in a tile whatever their
+// number: the line lies where it is as fast.  Pools (us, tiled / streamed; L = k = 16,
+// D = 512, 3 heads of 96, then L = 32, k = 16, D = 4096, 32 heads of 128): one token
+// 70 / 21 and 2061 / 394; 8 tokens 145 / 29 and 2076 / 709; 16 tokens 134 / 39 and
+// 2096 / 1199.
+constexpr int kGemvTokens = 16;
+constexpr int kGemvWarps = 4;
+
+template <int NT, int R, int U>
+__global__ void __launch_bounds__(kGemvWarps * 32) gemv_wxT_f32(const GemmArgs a) {
+  constexpr int STEP = 32 * 4;
+  const int split = blockIdx.z % a.nsplit, bi = blockIdx.z / a.nsplit;
+  const int lane = threadIdx.x & 31;
+  const int groups = (a.N + NT - 1) / NT, n0 = (int)blockIdx.x % groups * NT;  // this CTA's tokens
+  const int m0 = ((int)blockIdx.x / groups * kGemvWarps + (threadIdx.x >> 5)) * R;
+  const int kend = min(a.K, (split + 1) * a.k_per_split);
+  int k = split * a.k_per_split + lane * 4;
+  const float* W = reinterpret_cast<const float*>(bi < a.per_branch ? a.W[0] : a.W[1]) +
+                   (int64_t)(bi % a.per_branch) * a.w_stride;
+  const float* X = reinterpret_cast<const float*>(a.X) + (int64_t)bi * a.x_stride + (int64_t)n0 * a.K;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const bool live = m0 < a.M;
+  auto load_w = [&](float4 (&w)[U][R], int k0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int kk = k0 + u * STEP;
+        w[u][r] = live && m0 + r < a.M && kk < kend
+                      ? __ldcg(reinterpret_cast<const float4*>(W + (int64_t)(m0 + r) * a.K + kk))
+                      : zero;
+      }
+  };
+  float4 w[U][R], wn[U][R];
+  load_w(w, k);
+  pdl_wait();
+  if (!live) return;
+  float acc[R][NT];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int t = 0; t < NT; ++t) acc[r][t] = 0.f;
+  // (the bound is the warp's, so that lanes past the split's end stay with it: their weights are 0)
+  for (; k - lane * 4 < kend; k += U * STEP) {
+    load_w(wn, k + U * STEP);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int kk = k + u * STEP;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const float4 x = kk < kend && n0 + t < a.N
+                             ? *reinterpret_cast<const float4*>(X + (int64_t)t * a.K + kk)
+                             : zero;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          acc[r][t] = fmaf(w[u][r].x, x.x, acc[r][t]);
+          acc[r][t] = fmaf(w[u][r].y, x.y, acc[r][t]);
+          acc[r][t] = fmaf(w[u][r].z, x.z, acc[r][t]);
+          acc[r][t] = fmaf(w[u][r].w, x.w, acc[r][t]);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int r = 0; r < R; ++r) w[u][r] = wn[u][r];
+  }
+  float* out = a.out + (int64_t)blockIdx.z * a.N * a.M;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const float v = warp_sum(acc[r][t]);
+      if (lane == 0 && n0 + t < a.N && m0 + r < a.M) out[(int64_t)(n0 + t) * a.M + m0 + r] = v;
+    }
+}
+
+// out[batch][split][n][m] = sum over the split's k of W[m][k] X[n][k]
+template <typename T>
+cudaError_t launch_simt_gemm(const GemmArgs& a, int batch, cudaStream_t s) {
+  const unsigned z = (unsigned)(batch * a.nsplit);
+  if (sizeof(T) == 4 && a.N <= kGemvTokens) {
+    auto go = [&](auto kern, int nt, int r) {
+      const int rows = kGemvWarps * r, groups = (a.N + nt - 1) / nt;
+      return launch_pdl(kern, dim3((unsigned)((a.M + rows - 1) / rows * groups), 1, z), dim3(kGemvWarps * 32),
+                        0, s, a);
+    };
+    if (a.N == 1) return go(gemv_wxT_f32<1, 2, 4>, 1, 2);
+    if (a.N == 2) return go(gemv_wxT_f32<2, 2, 4>, 2, 2);
+    if (a.N <= 4) return go(gemv_wxT_f32<4, 4, 2>, 4, 4);
+    return go(gemv_wxT_f32<8, 4, 2>, 8, 4);
+  }
+  return launch_pdl(gemm_wxT_simt<T, T>, dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), dim3(256), 0,
+                    s, a);
 }
 
 // ---------------------------------------------------------------- mix (bf16)
@@ -925,8 +1031,7 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
     a.K = p.Lp * p.D;
     a.nsplit = p.nsplit_r;
     a.k_per_split = ((a.K + p.nsplit_r - 1) / p.nsplit_r + BK - 1) / BK * BK;
-    dim3 grid((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, 2 * a.nsplit);
-    e = launch_pdl(gemm_wxT_simt<T, T>, grid, dim3(256), 0, s, a);
+    e = launch_simt_gemm<T>(a, 2, s);
   }
   if (e != cudaSuccess) return e;
   const bool tc_proj = bf16 && proj_tc_supported(p);
@@ -992,8 +1097,7 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
     a.K = p.D;
     a.nsplit = 1;
     a.k_per_split = p.D;
-    dim3 grid((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, 2 * p.k);
-    e = launch_pdl(gemm_wxT_simt<T, T>, grid, dim3(256), 0, s, a);
+    e = launch_simt_gemm<T>(a, 2 * p.k, s);
     if (e != cudaSuccess) return e;
   }
   {

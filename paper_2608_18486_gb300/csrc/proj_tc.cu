@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // tiles, warp 1 issues the MMAs into two TMEM accumulators in turn, and warps 4-7
 // finish tile i (the epilogue of proj_tc_kernel) while tile i + 1 streams.  One
 // token tile (fewer than kRowsTokens tokens).  Bound by the weight stream: 1.07 GB
-// there, 205 us with proj_tc_kernel (3.4 waves of CTAs), STREAMUS with this.
+// there, 205 us with proj_tc_kernel (3.4 waves of CTAs), 195 us with this.
 constexpr int kStreamThreads = 256;
 constexpr int kStreamMaxStages = 12;
 // k-blocks loaded together: a block takes 128 bytes of each of 128 rows, four in
