@@ -30,15 +30,15 @@ int attn_unit_warps_per_cta(int stage_bytes, int dtype, int d, int G) {
 // ring bytes of one stage of K and V
 static size_t ring_stage_bytes(int stage_bytes, int dtype, int d, int G) {
   const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
-  return 2 * ((size_t)attn_stage_slots(stage_bytes, dtype, d) * d * esz +
-              (attn_uses_mma(dtype, G) ? kAttnMmaPad : 0));
+  return 2 * (size_t)attn_stage_slots(stage_bytes, dtype, d) * d * esz +
+         (attn_uses_mma(dtype, d, G) ? kAttnMmaPad : 0);
 }
 
 size_t attn_smem_bytes(int stage_bytes, int dtype, int d, int G, int B) {
   const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
   const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, G);
   return (size_t)attn_detail::kWarps * attn_detail::kWStages * stage +
-         (attn_uses_mma(dtype, G) ? 0 : (size_t)attn_detail::kWarps * attn_detail::kWStages * G * d * esz) +
+         (attn_uses_mma(dtype, d, G) ? 0 : (size_t)attn_detail::kWarps * attn_detail::kWStages * G * d * esz) +
          sizeof(int) * (2 * (size_t)B + 1);
 }
 

@@ -16,8 +16,8 @@
 //    fills it with 1-D bulk async copies (TMA engine, mbarrier completion,
 //    L2 evict-first) of contiguous (page, kv-head) runs; it refills a slot as
 //    soon as it has consumed it, so no block-wide barrier is ever taken.
-//  * Compute (VecMath; MmaMath in attn_mma.cuh takes four or eight bf16 query
-//    heads per kv head).  8 lanes own one slot (16-byte vectors, conflict-free shared
+//  * Compute (VecMath; MmaMath in attn_mma.cuh takes several bf16 query heads per
+//    kv head).  8 lanes own one slot (16-byte vectors, conflict-free shared
 //    loads), reduce q.k with xor shuffles and keep an online softmax
 //    (running max m, sum l, accumulator) per lane group; groups merge with
 //    shuffles at the end of a piece.
@@ -148,7 +148,7 @@ template <typename T, int HD, int G, int SB>
 struct VecMath {
   using SH = Shape<T, HD, SB>;
   static constexpr int SPW = SH::SPW, ITERS = SH::ITERS, LPS = SH::LPS, E2 = SH::EPL / 2;
-  static constexpr int kPad = 0;
+  static constexpr int kPad = 0, kBlocks = 1;
   static constexpr bool kQueryRing = true;  // queries travel with a piece's first stage
   float2 q2[G][E2];
   float m[G], l[G];
@@ -295,29 +295,27 @@ struct VecMath {
   }
 };
 
-// Stage math of a launch: the tensor cores where a bf16 K/V row meets four
-// or more query heads (attn_uses_mma in internal.h).
-template <typename T, int HD, int G, int SB>
-struct MathOf {
+// Stage math of a launch (attn_uses_mma in internal.h)
+template <typename T, int HD, int G, int SB, bool MMA>
+struct MathPick {
   using type = VecMath<T, HD, G, SB>;
 };
-template <int HD, int SB>
-struct MathOf<__nv_bfloat16, HD, 4, SB> {
-  using type = MmaMath<HD, 4, Shape<__nv_bfloat16, HD, SB>::STAGE_SLOTS>;
+template <typename T, int HD, int G, int SB>
+struct MathPick<T, HD, G, SB, true> {
+  using type = MmaMath<HD, G, Shape<T, HD, SB>::STAGE_SLOTS>;
 };
-template <int HD, int SB>
-struct MathOf<__nv_bfloat16, HD, 8, SB> {
-  using type = MmaMath<HD, 8, Shape<__nv_bfloat16, HD, SB>::STAGE_SLOTS>;
-};
+template <typename T, int HD, int G, int SB>
+using MathOf =
+    typename MathPick<T, HD, G, SB, attn_uses_mma(sizeof(T) == 2 ? WM_DT_BF16 : WM_DT_F32, HD, G)>::type;
 
 // Slots per bulk copy of K and of V (a copy never crosses a page), and the
 // place of slot `ls` in the V tile: whole stages where the tile is
-// contiguous, the four shifted blocks of MmaMath otherwise.
+// contiguous, the shifted blocks of MmaMath otherwise.
 template <typename MATH, int SLOTS>
 struct CopyShape {
-  static constexpr int kVRun = MATH::kPad > 0 ? SLOTS / 4 : SLOTS;
+  static constexpr int kVRun = SLOTS / MATH::kBlocks;
   __device__ __forceinline__ static int v_shift(int ls) {
-    if constexpr (MATH::kPad > 0) return ls / kVRun * MATH::kSkew;
+    if constexpr (MATH::kBlocks > 1) return ls / kVRun * MATH::kSkew;
     else return 0;
   }
 };
@@ -370,10 +368,11 @@ __device__ __forceinline__ void copy_stage(const AttnParams& p, const T* kb, con
 template <typename T, int HD, int G, int SB>
 __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn_kernel(const AttnParams p) {
   using SH = Shape<T, HD, SB>;
-  using MATH = typename MathOf<T, HD, G, SB>::type;
+  using MATH = MathOf<T, HD, G, SB>;
   constexpr int STAGE_SLOTS = SH::STAGE_SLOTS;
-  constexpr int STAGE_ELEMS = SH::STAGE_ELEMS + MATH::kPad;        // of K, and of V, in the ring
-  constexpr uint32_t KV_BYTES = STAGE_ELEMS * sizeof(T);
+  constexpr int K_ELEMS = SH::STAGE_ELEMS;             // of K in the ring
+  constexpr int RING_ELEMS = 2 * K_ELEMS + MATH::kPad;  // of K and V
+  constexpr uint32_t KV_BYTES = K_ELEMS * sizeof(T);
   constexpr uint32_t Q_BYTES = G * HD * sizeof(T);
   constexpr int REC = attn_part_rec(G, HD);                        // floats per partial record
   constexpr int FLAG = G * HD + 2 * G;                             // the record's "published" word
@@ -387,8 +386,8 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
   constexpr unsigned FULLMASK = 0xFFFFFFFFu;
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* ring = reinterpret_cast<T*>(smem_raw);                       // [W][S][2][STAGE_ELEMS]
-  T* qring = ring + kWarps * kWStages * 2 * STAGE_ELEMS;          // [W][S][G*HD], if kQueryRing
+  T* ring = reinterpret_cast<T*>(smem_raw);                       // [W][S][RING_ELEMS]
+  T* qring = ring + kWarps * kWStages * RING_ELEMS;          // [W][S][G*HD], if kQueryRing
   int* pre = reinterpret_cast<int*>(qring + (MATH::kQueryRing ? kWarps * kWStages * G * HD : 0));  // [B+1]
   int* lens = pre + p.B + 1;                                      // [B]
   __shared__ uint64_t bars[kWarps][kWStages];
@@ -503,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     return;  // warp-level from here on: no block barriers below
   }
 
-  T* myring = ring + warp * kWStages * 2 * STAGE_ELEMS;
+  T* myring = ring + warp * kWStages * RING_ELEMS;
   T* myq = qring + warp * kWStages * G * HD;
   const uint64_t policy = l2_evict_first_policy();
 
@@ -555,8 +554,8 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     const int s_begin = pc.st * STAGE_SLOTS;
     const T* kb = reinterpret_cast<const T*>(p.k_pool) + (int64_t)pc.h * p.P * HD;
     const T* vb = reinterpret_cast<const T*>(p.v_pool) + (int64_t)pc.h * p.P * HD;
-    T* kd = myring + buf * 2 * STAGE_ELEMS;
-    T* vd = kd + STAGE_ELEMS;
+    T* kd = myring + buf * RING_ELEMS;
+    T* vd = kd + K_ELEMS;
     uint64_t* bar = &bars[warp][buf];
     // the first piece's query arrives on qbars (issued after the dependency wait)
     const bool with_q = MATH::kQueryRing && first && pseq > 0;
@@ -735,8 +734,8 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     }
     const int valid_slots = lens[cc.b] - cc.st * STAGE_SLOTS;
     const uint64_t mask = masks[warp][buf];
-    const T* Ks = myring + buf * 2 * STAGE_ELEMS;
-    const T* Vs = Ks + STAGE_ELEMS;
+    const T* Ks = myring + buf * RING_ELEMS;
+    const T* Vs = Ks + K_ELEMS;
     if (valid_slots >= STAGE_SLOTS && mask == all_pages)
       st.template consume<true>(Ks, Vs, lane, p.qscale, valid_slots, mask, log2R);
     else

@@ -1,31 +1,39 @@
 #pragma once
-// Stage math of decode attention on the tensor cores (bf16 caches, four or
-// eight query heads per kv head), used by both decode-attention kernels.
+// Stage math of decode attention on the tensor cores (bf16 caches, several
+// query heads per kv head; attn_uses_mma in internal.h says which), used by
+// both decode-attention kernels.
 //
-// On the CUDA cores every K and V element is multiplied once per query head
-// and lane group, about 90 warp instructions per slot at eight heads, so a
-// launch with G = 4 or 8 was bound by instruction issue, not by HBM.  Here a
-// warp takes 16 slots at a time through mma.sync.m16n8k16 (fp32
+// On the CUDA cores (VecMath) every K and V element is widened, and multiplied once
+// per query head, so launches with G = 4 or 8 were bound by instruction issue,
+// not by HBM, and the short launches of G = 2 spent most of their streaming time
+// on it.  Here a warp takes 16 slots at a time through mma.sync.m16n8k16 (fp32
 // accumulation): the G query heads are rows of A, the slots the columns of
-// S = q K^T, and the rows of P V.  (tcgen05 wants 64 or more rows of A, sixteen
+// S = q K^T, and the rows of P V.  (tcgen05 wants 64 or more rows of A, eight
 // times the heads there are, and a round trip through TMEM per stage.)
+// Measured (us, before / now): 64 sequences of 2048-4096 slots, 64/8 heads of 128:
+// 726 / 131; 32 of 4096-8192, 32/8 heads of 128: 167 / 133; 8 of up to 4096, 64/8
+// heads of 64: 28.4 / 22.3; a decode step of 16 layers, 16 sequences of 2048,
+// 6/3 heads of 96: 185 / 173.
 //
 //  * Probabilities stay fp32: p is split exactly into three bf16 terms (hi,
-//    mid, lo; 24 bits), and the spare rows of A carry them.  G = 4: rows 0-3
-//    hi, 4-7 mid, 8-11 lo of one MMA.  G = 8: two MMAs, (hi | mid) and
-//    (hi | lo), with the terms taken of p / 2 so that their two hi sums add up to
-//    p's.  The accumulators of hi, mid and lo stay apart and are summed when a
-//    piece ends; where hi's sum is not finite (infinite V) it stands alone,
-//    since 0 * inf in the smaller terms is no part of the result.
+//    mid, lo; 24 bits), and the spare rows of A carry them.  G = 2: rows 0-1
+//    hi, 2-3 mid, 4-5 lo of one MMA; G = 4: rows 0-3, 4-7, 8-11.  G = 8: two
+//    MMAs, (hi | mid) and (hi | lo), with the terms taken of p / 2 so that their
+//    two hi sums add up to p's.  The accumulators of hi, mid and lo stay apart
+//    and are summed when a piece ends; where hi's sum is not finite (infinite V)
+//    it stands alone, since 0 * inf in the smaller terms is no part of the result.
 //  * No ldmatrix and no swizzle: both contractions may run over their index in
 //    any order.  Lane (g, t) = (lane / 4, lane % 4) reads 16 bytes of K per
 //    two MMAs, and the columns of V are dealt so that one 16-byte vector of
 //    each of its four slots makes the B fragments of eight column tiles
 //    (two byte permutes each).
-//  * The V tile lies in four blocks of a quarter of the stage's slots, block
-//    i shifted by 32 i bytes: the 8 lanes of a quarter warp then read 128
-//    bytes on distinct banks.  K reads are two-way conflicted at d = 64 and
-//    128 (shared memory is busy a third of the time at full HBM rate).
+//  * Lanes that read together then read rows four or eight apart, which at d = 64
+//    and 128 start on the same bank: the V tile lies in two blocks of half the
+//    stage's slots, the second shifted by 64 bytes; at d = 96 (192-byte rows)
+//    half of the lanes take the rows of a pair in the other order.  Either way
+//    the reads are two-way conflicted, which costs less than smaller copies: V in
+//    four blocks, without conflicts, took 68.0 us where this takes 58.6 (16
+//    sequences of 4000-8192 slots, 32/8 heads of 96) and 135.6 for 131.2 (128).
 #include "common.cuh"
 #include "internal.h"
 
@@ -51,16 +59,17 @@ __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u 
 template <int HD, int G, int SLOTS>
 struct MmaMath {
   using T = __nv_bfloat16;
-  static_assert(G == 4 || G == 8, "four or eight query heads");
+  static_assert(G == 2 || G == 4 || G == 8, "two, four or eight query heads");
   static_assert(SLOTS % 16 == 0 && HD % 32 == 0, "16 slots and 32 columns per step");
-  static constexpr int kSub = SLOTS / 4;                       // slots per block of the V tile
-  static constexpr int kSkew = 16;                             // elements between blocks
-  static constexpr int kPad = kAttnMmaPad / (int)sizeof(T);    // elements added per matrix
-  // queries come straight from L2 when a piece starts: a ring of them for
-  // three stages (18 KB more per CTA at G = 8, d = 128 than its K and V leave) would
-  // halve the CTAs per SM
+  static constexpr int kSub = SLOTS / 4;                       // slots of a lane per stage
+  static constexpr bool kFlip = HD % 64 != 0;                  // rows of two lane pairs swapped (see above)
+  static constexpr int kBlocks = kFlip ? 1 : 2;                // blocks of the V tile
+  static constexpr int kSkew = 32;                             // elements between blocks
+  static constexpr int kPad = kAttnMmaPad / (int)sizeof(T);    // elements added to V
+  // queries come straight from L2 when a piece starts: a ring of them for three
+  // stages (24 KB per CTA at G = 8, d = 128) would leave one CTA per SM
   static constexpr bool kQueryRing = false;
-  static_assert(3 * kSkew <= kPad, "the shifts fit the padding");
+  static_assert((kBlocks - 1) * kSkew <= kPad, "the shift fits the padding");
   static constexpr int KV = HD / 32;                           // 16-byte K vectors per lane and slot
   static constexpr int NT = HD / 8;                            // column tiles of O
   static constexpr int FULL_I = HD / 64, TAIL = HD % 64 / 32;  // 64-column blocks, a 32-column rest
@@ -101,13 +110,14 @@ struct MmaMath {
     const int g = g_of(lane), t = lane & 3;
 #pragma unroll
     for (int s = 0; s < SLOTS / 16; ++s) {
-      // S: column n of tile j is slot kSub (n / 2) + 4 s + 2 j + n % 2, so that
-      // lane (g, t) holds slots kSub t + 4 s + 0..3, which lie in V block t
+      // S: column n of tile j is slot kSub (n / 2) + 4 s + 2 j + n % 2 (kFlip: with
+      // the last bit flipped in columns 4-7), so that lane (g, t) holds slots kSub t +
+      // 4 s + (0..3 ^ flip), all in one V block
       float c[2][4];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
-        const T* kr = Ks + (kSub * (g >> 1) + 4 * s + 2 * j + (g & 1)) * HD + t * 8;
+        const T* kr = Ks + (kSub * (g >> 1) + 4 * s + 2 * j + ((g ^ (kFlip ? g >> 2 : 0)) & 1)) * HD + t * 8;
 #pragma unroll
         for (int i = 0; i < KV; ++i) {
           const uint4 v = *reinterpret_cast<const uint4*>(kr + i * 32);
@@ -115,13 +125,13 @@ struct MmaMath {
           mma_bf16_16816(c[j], qa[i][2], 0u, qa[i][3], 0u, v.z, v.w);
         }
       }
-      const int ls = kSub * t + 4 * s;
+      const int ls = kSub * t + 4 * s, fx = kFlip ? t >> 1 : 0;
       float sc[4];
       bool ok[4];
       float mx = -INFINITY;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        ok[i] = FULL || ((ls + i < valid_slots) && ((mask >> ((ls + i) >> log2R)) & 1ull));
+        ok[i] = FULL || ((ls + (i ^ fx) < valid_slots) && ((mask >> ((ls + (i ^ fx)) >> log2R)) & 1ull));
         sc[i] = ok[i] ? c[i >> 1][i & 1] * qscale : -INFINITY;
         mx = fmaxf(mx, sc[i]);
       }
@@ -154,21 +164,21 @@ struct MmaMath {
         const float x1 = r * (x - bf16_lo(hi)), y1 = r * (y - bf16_hi(hi));
         const uint32_t mid = pack_bf16(x1, y1);
         const uint32_t lo = pack_bf16(x1 - bf16_lo(mid), y1 - bf16_hi(mid));
-        a0[j] = (G == 4 && g >= 4) ? mid : hi;
-        a1[j] = G == 4 ? lo : mid;
+        a0[j] = G == 8 || g / G == 0 ? hi : g / G == 1 ? mid : lo;
+        a1[j] = G == 8 ? mid : G == 4 ? lo : 0u;
         a2[j] = lo;
       }
       auto pv = [&](float (&o)[4], uint32_t b0, uint32_t b1) {
         mma_bf16_16816(o, a0[0], a1[0], a0[1], a1[1], b0, b1);
         if (G == 8) mma_bf16_16816(o, a0[0], a2[0], a0[1], a2[1], b0, b1);
       };
-      const T* vr = Vs + ls * HD + t * kSkew;
+      const T* vr = Vs + ls * HD + (kBlocks > 1 ? (t >> 1) * kSkew : 0);
 #pragma unroll
       for (int i = 0; i < FULL_I; ++i) {
         uint32_t v[4][4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          uint4 x = *reinterpret_cast<const uint4*>(vr + r * HD + i * 64 + g * 8);
+          uint4 x = *reinterpret_cast<const uint4*>(vr + (r ^ fx) * HD + i * 64 + g * 8);
           if (!FULL && !ok[r]) x = make_uint4(0u, 0u, 0u, 0u);
           v[r][0] = x.x;
           v[r][1] = x.y;
@@ -185,7 +195,7 @@ struct MmaMath {
         uint32_t v[4][2];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          uint2 x = *reinterpret_cast<const uint2*>(vr + r * HD + FULL_I * 64 + g * 4);
+          uint2 x = *reinterpret_cast<const uint2*>(vr + (r ^ fx) * HD + FULL_I * 64 + g * 4);
           if (!FULL && !ok[r]) x = make_uint2(0u, 0u);
           v[r][0] = x.x;
           v[r][1] = x.y;
@@ -210,7 +220,9 @@ struct MmaMath {
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const float hi = acc[n][i];
-        const float rest = G == 4 ? __shfl_xor_sync(0xFFFFFFFFu, hi, 16) + acc[n][i + 2] : acc[n][i + 2];
+        float rest = acc[n][i + 2];
+        if (G == 4) rest += __shfl_xor_sync(0xFFFFFFFFu, hi, 16);
+        if (G == 2) rest = __shfl_xor_sync(0xFFFFFFFFu, hi, 8) + __shfl_xor_sync(0xFFFFFFFFu, hi, 16);
         acc[n][i] = fabsf(hi) < INFINITY ? hi + rest : hi;
       }
   }

@@ -53,10 +53,11 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
     decode_attn_unit_kernel(const AttnParams p) {
   using SH = Shape<T, HD, SB>;
   constexpr int NW = unit_warps<T, HD, G, SB>();
-  using MATH = typename MathOf<T, HD, G, SB>::type;
+  using MATH = MathOf<T, HD, G, SB>;
   constexpr int STAGE_SLOTS = SH::STAGE_SLOTS;
-  constexpr int STAGE_ELEMS = SH::STAGE_ELEMS + MATH::kPad;  // of K, and of V, in the ring
-  constexpr uint32_t KV_BYTES = STAGE_ELEMS * sizeof(T);
+  constexpr int K_ELEMS = SH::STAGE_ELEMS;             // of K in the ring
+  constexpr int RING_ELEMS = 2 * K_ELEMS + MATH::kPad;  // of K and V
+  constexpr uint32_t KV_BYTES = K_ELEMS * sizeof(T);
   constexpr int E = G * HD;  // output elements of a unit
   constexpr int REC = unit_rec(G, HD);
   constexpr unsigned FULLMASK = 0xFFFFFFFFu;
@@ -64,8 +65,8 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
   static_assert((size_t)REC * sizeof(float) <= (size_t)kUStages * 2 * KV_BYTES, "record fits the ring");
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* ring = reinterpret_cast<T*>(smem_raw);  // [NW][S][2][STAGE_ELEMS]
-  float* crec = reinterpret_cast<float*>(ring + NW * kUStages * 2 * STAGE_ELEMS);  // [REC]
+  T* ring = reinterpret_cast<T*>(smem_raw);  // [NW][S][RING_ELEMS]
+  float* crec = reinterpret_cast<float*>(ring + NW * kUStages * RING_ELEMS);  // [REC]
   __shared__ uint64_t bars[NW][kUStages];
   __shared__ uint64_t masks[NW][kUStages];
 
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
   const int s0 = (int)((int64_t)piece * nst / npieces);
   const int nmine = (int)((int64_t)(piece + 1) * nst / npieces) - s0;
 
-  T* myring = ring + warp * kUStages * 2 * STAGE_ELEMS;
+  T* myring = ring + warp * kUStages * RING_ELEMS;
   const uint64_t policy = l2_evict_first_policy();
   const T* kbase = reinterpret_cast<const T*>(p.k_pool) + (int64_t)h * p.P * HD;
   const T* vbase = reinterpret_cast<const T*>(p.v_pool) + (int64_t)h * p.P * HD;
@@ -129,8 +130,8 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
   // Copy stage s of the unit (the i-th of this warp) into ring slot i % S.
   auto issue = [&](int s) {
     const int buf = (s - s0) % kUStages;
-    T* kd = myring + buf * 2 * STAGE_ELEMS;
-    T* vd = kd + STAGE_ELEMS;
+    T* kd = myring + buf * RING_ELEMS;
+    T* vd = kd + K_ELEMS;
     uint64_t* bar = &bars[warp][buf];
     const int s_begin = s * STAGE_SLOTS;
     attn_detail::copy_stage<MATH, T, HD, STAGE_SLOTS>(p, kbase, vbase, s_begin, S, kd, vd, bar,
@@ -163,8 +164,8 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
     const int s = s0 + done;
     const int valid_slots = S - s * STAGE_SLOTS;
     const uint64_t mask = masks[warp][buf];
-    const T* Ks = myring + buf * 2 * STAGE_ELEMS;
-    const T* Vs = Ks + STAGE_ELEMS;
+    const T* Ks = myring + buf * RING_ELEMS;
+    const T* Vs = Ks + K_ELEMS;
     if (valid_slots >= STAGE_SLOTS && mask == all_pages)
       st.template consume<true>(Ks, Vs, lane, p.qscale, valid_slots, mask, log2R);
     else
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
   // ---- merge the CTA's NW warp states, element by element
   T* outp = reinterpret_cast<T*>(p.out) + ((int64_t)b * p.Hq + h * G) * HD;
   auto warp_rec = [&](int w) -> const float* {
-    return reinterpret_cast<const float*>(ring + w * kUStages * 2 * STAGE_ELEMS);
+    return reinterpret_cast<const float*>(ring + w * kUStages * RING_ELEMS);
   };
   for (int e = tid; e < E; e += NW * 32) {
     const int g = e / HD;

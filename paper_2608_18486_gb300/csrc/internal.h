@@ -61,10 +61,16 @@ constexpr int attn_ctas_per_sm(int stage_bytes, int G) { return stage_bytes == 4
 constexpr int attn_part_rec(int G, int d) { return G * d + (2 * G + 1 + 3) / 4 * 4; }
 
 // Launches whose stage math runs on the tensor cores (attn_mma.cuh): bf16
-// with four or eight query heads per kv head.  Their K and V tiles in shared
-// memory are kAttnMmaPad bytes longer.
-constexpr bool attn_uses_mma(int dtype, int G) { return dtype == WM_DT_BF16 && G >= 4; }
-constexpr int kAttnMmaPad = 128;
+// with four or eight query heads per kv head, or two of 64 or 96.  Two heads of
+// 128 stay on the CUDA cores, which were faster there with the 8 warps per SM that
+// its stages leave room for (step of 8 layers, 4 ragged sequences up to 4096, 16/8
+// heads: 115 us, 127 on the tensor cores; of 64, 16 sequences of 2048, 12/6 heads:
+// 123 and 120; of 96, 6/3 heads, 16 layers: 185 and 173).  A stage of theirs is kAttnMmaPad bytes longer in shared
+// memory.
+constexpr bool attn_uses_mma(int dtype, int d, int G) {
+  return dtype == WM_DT_BF16 && (G >= 4 || (G == 2 && d <= 96));
+}
+constexpr int kAttnMmaPad = 64;
 
 int attn_stage_slots(int stage_bytes, int dtype, int d);
 int attn_warps_per_cta();
