@@ -12,19 +12,8 @@ int attn_stage_slots(int stage_bytes, int dtype, int d) {
 }
 
 int attn_warps_per_cta() { return attn_detail::kWarps; }
-int attn_unit_warps_per_cta(int stage_bytes, int dtype, int d, int G) {
-  using namespace attn_unit_detail;
-  if (stage_bytes != 8192) return 0;
-  if (dtype == WM_DT_F32) {
-    if (d == 64) return unit_warps_g<float, 64, 8192>(G);
-    if (d == 96) return unit_warps_g<float, 96, 8192>(G);
-    if (d == 128) return unit_warps_g<float, 128, 8192>(G);
-    return 0;
-  }
-  if (d == 64) return unit_warps_g<__nv_bfloat16, 64, 8192>(G);
-  if (d == 96) return unit_warps_g<__nv_bfloat16, 96, 8192>(G);
-  if (d == 128) return unit_warps_g<__nv_bfloat16, 128, 8192>(G);
-  return 0;
+int attn_unit_warps_per_cta(int stage_bytes, int G) {
+  return stage_bytes == 8192 ? attn_unit_detail::unit_warps(G) : 0;
 }
 
 // ring bytes of one stage of K and V
@@ -49,23 +38,23 @@ cudaError_t launch_decode_attn(const AttnParams& p, int stage_bytes, int dtype, 
   return launch_attn_bf16(p, stage_bytes, d, G, grid, smem, s);
 }
 
-size_t attn_unit_smem_bytes(int stage_bytes, int dtype, int d, int G) {
+size_t attn_unit_smem_bytes(int stage_bytes, int dtype, int d, int G, int warps) {
   const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, G);
-  return (size_t)attn_unit_warps_per_cta(stage_bytes, dtype, d, G) * attn_unit_detail::kUStages * stage +
+  return (size_t)warps * attn_unit_detail::kUStages * stage +
          (size_t)(attn_unit_detail::unit_rec(G, d) + 3) / 4 * 4 * sizeof(float);
 }
 
-int attn_unit_max_clusters(int stage_bytes, int dtype, int d, int G, int cluster) {
-  const size_t smem = attn_unit_smem_bytes(stage_bytes, dtype, d, G);
-  if (dtype == WM_DT_F32) return attn_unit_max_clusters_f32(stage_bytes, d, G, cluster, smem);
-  return attn_unit_max_clusters_bf16(stage_bytes, d, G, cluster, smem);
+int attn_unit_max_clusters(int stage_bytes, int dtype, int d, int G, int warps, int cluster) {
+  const size_t smem = attn_unit_smem_bytes(stage_bytes, dtype, d, G, warps);
+  if (dtype == WM_DT_F32) return attn_unit_max_clusters_f32(stage_bytes, d, G, warps, cluster, smem);
+  return attn_unit_max_clusters_bf16(stage_bytes, d, G, warps, cluster, smem);
 }
 
 cudaError_t launch_decode_attn_unit(const AttnParams& p, int stage_bytes, int dtype, int d, int G,
-                                    int units, int cluster, cudaStream_t s) {
-  const size_t smem = attn_unit_smem_bytes(stage_bytes, dtype, d, G);
-  if (dtype == WM_DT_F32) return launch_attn_unit_f32(p, stage_bytes, d, G, units, cluster, smem, s);
-  return launch_attn_unit_bf16(p, stage_bytes, d, G, units, cluster, smem, s);
+                                    int warps, int units, int cluster, cudaStream_t s) {
+  const size_t smem = attn_unit_smem_bytes(stage_bytes, dtype, d, G, warps);
+  if (dtype == WM_DT_F32) return launch_attn_unit_f32(p, stage_bytes, d, G, warps, units, cluster, smem, s);
+  return launch_attn_unit_bf16(p, stage_bytes, d, G, warps, units, cluster, smem, s);
 }
 
 }  // namespace wm

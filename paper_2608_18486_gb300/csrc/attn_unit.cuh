@@ -33,26 +33,21 @@ constexpr int kUStages = 3;  // ring depth per warp
 
 // Warps per CTA: 4 where a kv head has at most two query heads (two or
 // three CTAs per SM, by the stage size: smaller CTAs keep more clusters
-// resident and more SMs busy), else 8 (one CTA per SM: the states of four or
-// eight query heads take up to 255 registers).
-template <typename T, int HD, int G, int SB>
-constexpr int unit_warps() {
-  return G <= 2 ? 4 : 8;
-}
+// resident and more SMs busy), else 8 (one CTA per SM: fp32 states of four or
+// eight query heads take up to 255 registers, and few units need the warps), or
+// 4 if the planner asks for them (bf16: more units than SMs).
+constexpr int unit_warps(int G) { return G <= 2 ? 4 : 8; }
 // CTAs per SM the register budget is sized for (at most 12 warps of 170
-// registers per SM)
-constexpr int unit_min_blocks(int nw) { return nw <= 4 ? 3 : nw <= 6 ? 2 : 1; }
+// registers per SM; the stages of four or eight heads of 64 or 128 leave room for 8)
+constexpr int unit_min_blocks(int nw, int g, int d) { return nw > 4 ? 1 : g > 2 && d != 96 ? 2 : 3; }
 
 // floats of one partial state: G x HD unnormalised outputs, then (max, sum)
 // per query head (log2 units)
 constexpr int unit_rec(int G, int HD) { return G * HD + 2 * G; }
 
-template <typename T, int HD, int G, int SB>
-__global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
-                                  unit_min_blocks(unit_warps<T, HD, G, SB>()))
-    decode_attn_unit_kernel(const AttnParams p) {
+template <typename T, int HD, int G, int SB, int NW>
+__global__ void __launch_bounds__(NW * 32, unit_min_blocks(NW, G, HD)) decode_attn_unit_kernel(const AttnParams p) {
   using SH = Shape<T, HD, SB>;
-  constexpr int NW = unit_warps<T, HD, G, SB>();
   using MATH = MathOf<T, HD, G, SB>;
   constexpr int STAGE_SLOTS = SH::STAGE_SLOTS;
   constexpr int K_ELEMS = SH::STAGE_ELEMS;             // of K in the ring
@@ -254,15 +249,15 @@ __global__ void __launch_bounds__(unit_warps<T, HD, G, SB>() * 32,
   cluster.sync();
 }
 
-template <typename T, int HD, int G, int SB>
+template <typename T, int HD, int G, int SB, int NW>
 inline cudaError_t launch_unit_t(const AttnParams& p, int units, int cluster, size_t smem,
                                  cudaStream_t stream) {
   static size_t smem_set[kSmemOptDevices] = {};
-  auto kern = decode_attn_unit_kernel<T, HD, G, SB>;
+  auto kern = decode_attn_unit_kernel<T, HD, G, SB, NW>;
   if (cudaError_t e = opt_in_smem(kern, smem, smem_set); e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)units * (unsigned)cluster);
-  cfg.blockDim = dim3(unit_warps<T, HD, G, SB>() * 32);
+  cfg.blockDim = dim3(NW * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -278,16 +273,16 @@ inline cudaError_t launch_unit_t(const AttnParams& p, int units, int cluster, si
 }
 
 // Clusters of `cluster` CTAs that can be resident at once (0: unknown).
-template <typename T, int HD, int G, int SB>
+template <typename T, int HD, int G, int SB, int NW>
 inline int max_clusters_t(int cluster, size_t smem) {
-  auto kern = decode_attn_unit_kernel<T, HD, G, SB>;
+  auto kern = decode_attn_unit_kernel<T, HD, G, SB, NW>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)cluster * 64u);
-  cfg.blockDim = dim3(unit_warps<T, HD, G, SB>() * 32);
+  cfg.blockDim = dim3(NW * 32);
   cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -305,35 +300,38 @@ inline int max_clusters_t(int cluster, size_t smem) {
 }
 
 template <typename T, int HD, int SB>
-inline int unit_warps_g(int G) {
+inline int max_clusters_g(int G, int warps, int cluster, size_t smem) {
+  if (warps != 4 && warps != 8) return 0;
   switch (G) {
-    case 1: return unit_warps<T, HD, 1, SB>();
-    case 2: return unit_warps<T, HD, 2, SB>();
-    case 4: return unit_warps<T, HD, 4, SB>();
-    case 8: return unit_warps<T, HD, 8, SB>();
+    case 1: return warps == 4 ? max_clusters_t<T, HD, 1, SB, 4>(cluster, smem) : 0;
+    case 2: return warps == 4 ? max_clusters_t<T, HD, 2, SB, 4>(cluster, smem) : 0;
+    case 4:
+      if constexpr (sizeof(T) == 2)
+        if (warps == 4) return max_clusters_t<T, HD, 4, SB, 4>(cluster, smem);
+      return warps == 8 ? max_clusters_t<T, HD, 4, SB, 8>(cluster, smem) : 0;
+    case 8:
+      if constexpr (sizeof(T) == 2)
+        if (warps == 4) return max_clusters_t<T, HD, 8, SB, 4>(cluster, smem);
+      return warps == 8 ? max_clusters_t<T, HD, 8, SB, 8>(cluster, smem) : 0;
     default: return 0;
   }
 }
 
 template <typename T, int HD, int SB>
-inline int max_clusters_g(int G, int cluster, size_t smem) {
-  switch (G) {
-    case 1: return max_clusters_t<T, HD, 1, SB>(cluster, smem);
-    case 2: return max_clusters_t<T, HD, 2, SB>(cluster, smem);
-    case 4: return max_clusters_t<T, HD, 4, SB>(cluster, smem);
-    case 8: return max_clusters_t<T, HD, 8, SB>(cluster, smem);
-    default: return 0;
-  }
-}
-
-template <typename T, int HD, int SB>
-inline cudaError_t launch_unit_g(const AttnParams& p, int G, int units, int cluster, size_t smem,
+inline cudaError_t launch_unit_g(const AttnParams& p, int G, int warps, int units, int cluster, size_t smem,
                                  cudaStream_t s) {
+  if (warps != 4 && warps != 8) return cudaErrorInvalidValue;
   switch (G) {
-    case 1: return launch_unit_t<T, HD, 1, SB>(p, units, cluster, smem, s);
-    case 2: return launch_unit_t<T, HD, 2, SB>(p, units, cluster, smem, s);
-    case 4: return launch_unit_t<T, HD, 4, SB>(p, units, cluster, smem, s);
-    case 8: return launch_unit_t<T, HD, 8, SB>(p, units, cluster, smem, s);
+    case 1: return warps == 4 ? launch_unit_t<T, HD, 1, SB, 4>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
+    case 2: return warps == 4 ? launch_unit_t<T, HD, 2, SB, 4>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
+    case 4:
+      if constexpr (sizeof(T) == 2)
+        if (warps == 4) return launch_unit_t<T, HD, 4, SB, 4>(p, units, cluster, smem, s);
+      return warps == 8 ? launch_unit_t<T, HD, 4, SB, 8>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
+    case 8:
+      if constexpr (sizeof(T) == 2)
+        if (warps == 4) return launch_unit_t<T, HD, 8, SB, 4>(p, units, cluster, smem, s);
+      return warps == 8 ? launch_unit_t<T, HD, 8, SB, 8>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
 }
@@ -342,11 +340,11 @@ inline cudaError_t launch_unit_g(const AttnParams& p, int G, int units, int clus
 
 // Per-dtype dispatch of the unit split (one translation unit each); the
 // max_clusters entry points return 0 for an unsupported shape or no device.
-cudaError_t launch_attn_unit_bf16(const AttnParams& p, int stage_bytes, int d, int G, int units,
+cudaError_t launch_attn_unit_bf16(const AttnParams& p, int stage_bytes, int d, int G, int warps, int units,
                                   int cluster, size_t smem, cudaStream_t s);
-cudaError_t launch_attn_unit_f32(const AttnParams& p, int stage_bytes, int d, int G, int units,
+cudaError_t launch_attn_unit_f32(const AttnParams& p, int stage_bytes, int d, int G, int warps, int units,
                                  int cluster, size_t smem, cudaStream_t s);
-int attn_unit_max_clusters_bf16(int stage_bytes, int d, int G, int cluster, size_t smem);
-int attn_unit_max_clusters_f32(int stage_bytes, int d, int G, int cluster, size_t smem);
+int attn_unit_max_clusters_bf16(int stage_bytes, int d, int G, int warps, int cluster, size_t smem);
+int attn_unit_max_clusters_f32(int stage_bytes, int d, int G, int warps, int cluster, size_t smem);
 
 }  // namespace wm

@@ -40,6 +40,7 @@ bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 struct AttnPlan {
   int stage_bytes, grid, nwarps, chunk_stages, max_chunks;
   int unit_ctas;  // > 0: unit split, one cluster of this many CTAs per unit
+  int unit_warps;  // ... of this many warps
   size_t off_part, off_counters, total;
 };
 
@@ -89,19 +90,27 @@ constexpr int kAttnMinStagesPerWarp = 4;
 // and stream-K balances them.
 constexpr double kAttnUnitMinWarpShare = 0.6;
 
-// Resident clusters of C unit-split CTAs for (dtype, d, G) on this device,
-// cached (0: unknown or no device).
-int unit_max_clusters(int dtype, int d, int G, int C) {
-  static std::atomic<int> cache[kMaxDevices][2][3][4][wm::kAttnUnitMaxCluster + 1];
+// With four or eight query heads (8 warps per CTA, one CTA per SM) more units than
+// SMs do not fit; bf16 launches of at most this many bytes of K and V then take CTAs
+// of 4 warps, two per SM.  Four calls and a pool, 256 units of 500-1000 slots, four /
+// eight heads of 64: 90 / 98 us on stream-K, 66 / 72 so; of 128: 120 / 134 and 101 /
+// 110.  Past the line it depends on the lengths (200 units of 64: 3000-6000 slots,
+// 303 MB, 212 and 235; 256 of 64: 388 MB 276 and 254).
+constexpr double kAttnUnitNarrowBytes = 3.0e8;
+
+// Resident clusters of C unit-split CTAs of `warps` warps for (dtype, d, G) on this
+// device, cached (0: unknown or no device).
+int unit_max_clusters(int dtype, int d, int G, int warps, int C) {
+  static std::atomic<int> cache[kMaxDevices][2][3][4][2][wm::kAttnUnitMaxCluster + 1];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
   const int di = d == 64 ? 0 : d == 96 ? 1 : d == 128 ? 2 : -1;
   const int gi = G == 1 ? 0 : G == 2 ? 1 : G == 4 ? 2 : G == 8 ? 3 : -1;
   if (di < 0 || gi < 0 || C < 1 || C > wm::kAttnUnitMaxCluster) return 0;
-  std::atomic<int>& slot = cache[dev][dtype == WM_DT_F32 ? 1 : 0][di][gi][C];
+  std::atomic<int>& slot = cache[dev][dtype == WM_DT_F32 ? 1 : 0][di][gi][warps == 4 ? 0 : 1][C];
   int v = slot.load(std::memory_order_relaxed);
   if (v == 0) {
-    v = 1 + wm::attn_unit_max_clusters(kAttnStageBytes, dtype, d, G, C);
+    v = 1 + wm::attn_unit_max_clusters(kAttnStageBytes, dtype, d, G, warps, C);
     slot.store(v, std::memory_order_relaxed);
   }
   return v - 1;
@@ -159,19 +168,26 @@ AttnPlan attn_plan(const wm_config& c, int32_t B, int32_t max_pages, uint32_t fl
   // the size the workspace query reports)
   const int64_t units = (int64_t)B * c.Hkv;
   const int nsm = sm_count();
-  const int unit_warps = wm::attn_unit_warps_per_cta(pl.stage_bytes, c.dtype, c.d, G);
+  int unit_warps = wm::attn_unit_warps_per_cta(pl.stage_bytes, G);
   if (force_unit) {
     int64_t C = nsm / units;
     pl.unit_ctas = (int)(C < 1 ? 1 : C > wm::kAttnUnitMaxCluster ? wm::kAttnUnitMaxCluster : C);
   } else if (!force_dynamic && (pl.chunk_stages == 0 || B == 1) && unit_warps > 0) {
-    for (int C = wm::kAttnUnitMaxCluster; C >= 1; --C) {
-      if (unit_max_clusters(c.dtype, c.d, G, C) < units) continue;
-      if ((double)(units * C * unit_warps) >= kAttnUnitMinWarpShare * pl.nwarps) pl.unit_ctas = C;
-      break;
+    auto fit = [&](int warps) {  // largest resident cluster, 0 if none fits
+      int C = wm::kAttnUnitMaxCluster;
+      while (C >= 1 && unit_max_clusters(c.dtype, c.d, G, warps, C) < units) --C;
+      return C;
+    };
+    int C = fit(unit_warps);
+    if (C == 0 && unit_warps == 8 && c.dtype == WM_DT_BF16 && kv_bytes <= kAttnUnitNarrowBytes) {
+      unit_warps = 4;
+      C = fit(unit_warps);
     }
+    if ((double)(units * C * unit_warps) >= kAttnUnitMinWarpShare * pl.nwarps) pl.unit_ctas = C;
   }
   if (pl.unit_ctas > 0) {
     pl.grid = (int)(units * pl.unit_ctas);
+    pl.unit_warps = unit_warps;
     pl.nwarps = pl.grid * unit_warps;
     pl.chunk_stages = 0;
   }
@@ -272,7 +288,7 @@ wm_status decode_attn_impl(const wm_config* c, const wm_cache* cache, int32_t la
   cudaError_t e =
       pl.unit_ctas > 0
           ? wm::launch_decode_attn_unit(p, pl.stage_bytes, c->dtype, c->d, c->Hq / c->Hkv,
-                                        B * c->Hkv, pl.unit_ctas, (cudaStream_t)stream)
+                                        pl.unit_warps, B * c->Hkv, pl.unit_ctas, (cudaStream_t)stream)
           : wm::launch_decode_attn(p, pl.stage_bytes, c->dtype, c->d, c->Hq / c->Hkv, pl.grid,
                                    (cudaStream_t)stream);
   return e == cudaSuccess ? WM_OK : WM_ERR_CUDA;
