@@ -680,18 +680,20 @@ __global__ void __launch_bounds__(kPThreads, 1)
             float scale = 1.f;
             const float mt = fmaxf(half_max(0), mt1);
             raise = raise && mt > m;  // (also false while nothing is visible)
+            // (a row of -inf so far starts anew: NaN scores may be in its sums)
+            const bool anew = raise && m == -INFINITY;
             if (raise) {
-              scale = m == -INFINITY ? 0.f : ex2(m - mt);
+              scale = ex2(m - mt);
               m = mt;
             }
-            l *= scale;
+            l = anew ? 0.f : l * scale;
 #pragma unroll 1
             for (int c = 0; c < HD / 8; ++c) {
               uint32_t o[8];
               tc::tmem_ld8(ocol + 8 * c, o);
               tc::tmem_ld_wait();
 #pragma unroll
-              for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * scale);
+              for (int e = 0; e < 8; ++e) o[e] = anew ? 0u : __float_as_uint(__uint_as_float(o[e]) * scale);
               tc::tmem_st8(ocol + 8 * c, o);
             }
             half_p(0, w);
@@ -710,7 +712,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
       if (n > 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&odone[i], (cnt - 1) & 1));
       if (!ok) break;
       tc::fence_after_sync();
-      float inv = (n > 0 && l > 0.f) ? 1.f / l : 0.f, inv1 = 0.f;  // weights of this O and of the other half's
+      // Weights of this O and of the other half's.  O counts if any P V ran (else it
+      // holds another item's rows) and the row saw a score above -inf.
+      bool own = n > 0 && m != -INFINITY, other = false;
+      float inv = (own && l > 0.f) ? 1.f / l : 0.f, inv1 = 0.f;
       if constexpr (HALVES) {
         sml[i][row] = make_float2(m, l);
         tc::fence_before_sync();
@@ -721,8 +726,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
         tc::fence_after_sync();
         const float2 o = sml[i ^ 1][row];
         const float mm = fmaxf(m, o.x);
-        const float a = m == -INFINITY ? 0.f : ex2(m - mm), b2 = o.x == -INFINITY ? 0.f : ex2(o.x - mm);
-        const float ls = a * l + b2 * o.y, r = ls > 0.f ? 1.f / ls : 0.f;
+        other = items[slot].nt[i ^ 1] > 0 && o.x != -INFINITY;
+        const float a = own ? ex2(m - mm) : 0.f, b2 = other ? ex2(o.x - mm) : 0.f;
+        const float ls = (own ? a * l : 0.f) + (other ? b2 * o.y : 0.f), r = ls > 0.f ? 1.f / ls : 0.f;
         inv = a * r;
         inv1 = b2 * r;
       }
@@ -745,15 +751,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
         const int c = c0 + cc;
         if (HALVES && c >= c1) break;
         tc::tmem_ld_wait();
-        if constexpr (HALVES) {  // a half without KV tiles left its O as another item had it
-          const int n1 = items[slot].nt[i ^ 1];
+        if constexpr (HALVES) {
           uint32_t o1[32];
           tc::tmem_ld32(ocol1 + 32 * c, o1);
           tc::tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 32; ++e)
-            o[cc & 1][e] = __float_as_uint((n > 0 ? __uint_as_float(o[cc & 1][e]) * inv : 0.f) +
-                                           (n1 > 0 ? __uint_as_float(o1[e]) * inv1 : 0.f));
+            o[cc & 1][e] = __float_as_uint((own ? __uint_as_float(o[cc & 1][e]) * inv : 0.f) +
+                                           (other ? __uint_as_float(o1[e]) * inv1 : 0.f));
         }
         if (c + 1 < c1) tc::tmem_ld32(ocol + 32 * (c + 1), o[(cc + 1) & 1]);
 #pragma unroll
@@ -763,9 +768,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
           for (int t = 0; t < 4; ++t) {
             float x0 = __uint_as_float(o[cc & 1][e + 2 * t]);
             float x1 = __uint_as_float(o[cc & 1][e + 2 * t + 1]);
-            if (!HALVES) {  // (n == 0: no P V ran, O holds another item's rows)
-              x0 = n > 0 ? x0 * inv : 0.f;
-              x1 = n > 0 ? x1 * inv : 0.f;
+            if (!HALVES) {
+              x0 = own ? x0 * inv : 0.f;
+              x1 = own ? x1 * inv : 0.f;
             }
             const __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
             u[t] = *reinterpret_cast<const uint32_t*>(&h2);
