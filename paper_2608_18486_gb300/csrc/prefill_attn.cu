@@ -164,7 +164,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
   constexpr int CB = SH::CB, NSK = SH::NSK, NSV = SH::NSV;
   extern __shared__ uint8_t smem_dyn[];
   __shared__ __align__(16) uint8_t clc_buf[16];
-  __shared__ uint64_t clc_bar, vzero, qfull, qempty, kfull[NSK], kempty[NSK], vfull[NSV], vempty[NSV];
+  __shared__ uint64_t clc_bar, qfull, qempty, kfull[NSK], kempty[NSK], vfull[NSV], vempty[NSV];
+  // The rows past an item's last slot are zeroed in the V tile of this ring slot.  One
+  // barrier per slot: its next arrival follows the slot's refill, which waits for
+  // vempty, committed by the MMA thread after it has seen this one.  (One barrier for
+  // all slots could be two arrivals on before the MMA thread came to its wait: the
+  // tiles of two short items fit the ring.)
+  __shared__ uint64_t vzero[NSV];
   __shared__ uint64_t info_full[2], info_empty[2];
   // HALVES: (max, sum) of each half's rows; xfull: a warp's are there and its O is
   // complete, xdone: it has read the other half's
@@ -186,7 +192,6 @@ __global__ void __launch_bounds__(kPThreads, 1)
 
   if (tid == 0) {
     mbar_init(&clc_bar, 1);
-    mbar_init(&vzero, 1);
     mbar_init(&qfull, 1);
     mbar_init(&qempty, 1);
     for (int s = 0; s < NSK; ++s) {
@@ -196,6 +201,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     for (int s = 0; s < NSV; ++s) {
       mbar_init(&vfull[s], 1);
       mbar_init(&vempty[s], 1);
+      mbar_init(&vzero[s], 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&info_full[i], 1);
@@ -407,7 +413,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                       make_uint4(0, 0, 0, 0);
             fence_proxy_async_shared();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&vzero);
+            if (lane == 0) mbar_arrive(&vzero[sv]);
           }
         }
       }
@@ -446,8 +452,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
           if (half == 1) tc::mma_commit(&odone[i]);
         };
         bool ok = true;
-        uint32_t kc = 0, vc = 0, qc = 0, zc = 0;  // K, V, items' Q and zeroed V tiles used so far
-        uint32_t cnt[kQT] = {0, 0};               // P tiles used so far
+        uint32_t kc = 0, vc = 0, qc = 0;  // K, V and items' Q tiles used so far
+        uint32_t cnt[kQT] = {0, 0};       // P tiles used so far
+        uint32_t zpar = 0;                // bit s: parity of the zeroed tiles of V slot s seen so far
+        auto wait_zeroed = [&](uint32_t st) {
+          const bool got = mbar_wait_spin(&vzero[st], (zpar >> st) & 1);
+          zpar ^= 1u << st;
+          return got;
+        };
         for (uint32_t it = 0; ok; ++it) {
           const int slot = it & 1;
           ok = mbar_wait_spin(&info_full[slot], (it >> 1) & 1);
@@ -487,7 +499,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 if (j >= nt[i] || !ok) continue;
                 const uint32_t kv = kv_of(i, j), st = (vc + kv) % NSV;
                 ok = wait_ring(vfull, vc + kv, NSV);
-                if (ok && part && kv + 1 == (uint32_t)nmax) ok = mbar_wait_spin(&vzero, zc & 1);
+                if (ok && part && kv + 1 == (uint32_t)nmax) ok = wait_zeroed(st);
                 if (!ok) continue;
                 ok = mbar_wait_spin(&pfull[i][0], cnt[i] & 1);
                 if (!ok) continue;
@@ -513,7 +525,6 @@ __global__ void __launch_bounds__(kPThreads, 1)
             if (!ok) break;
             kc += nmax;
             vc += nmax;
-            zc += part;
             continue;
           }
           ok = mbar_wait_spin(&kfull[kc % NSK], (kc / NSK) & 1) && mbar_wait_spin(&qfull, qc & 1);
@@ -530,7 +541,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             const uint32_t st = vc % NSV;
             ok = mbar_wait_spin(&vfull[st], (vc / NSV) & 1);
             const bool more = j + 1 < nmax;
-            if (ok && !more && tmaxpos - j * kPN + 1 < kPN) ok = mbar_wait_spin(&vzero, zc++ & 1);
+            if (ok && !more && tmaxpos - j * kPN + 1 < kPN) ok = wait_zeroed(st);
             if (!ok) break;
 #pragma unroll
             for (int i = 0; i < kQT; ++i) {
