@@ -52,6 +52,7 @@
 // (one item per CTA; every descriptor moved to uniform registers one by one,
 // 90 cycles per MMA; 16-byte row stores at the end), 738 us now; 6/3 heads of
 // 96, sixteen prompts of 2048: 126 and 78 us.
+#include <limits.h>
 #include <math.h>
 
 #include "internal.h"
@@ -175,6 +176,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
   // HALVES: (max, sum) of each half's rows; xfull: a warp's are there and its O is
   // complete, xdone: it has read the other half's
   __shared__ float2 sml[HALVES ? kQT : 1][kPM];
+  // A tile's NaN scores make the row NaN, unless no tile up to it had a score above -inf:
+  // such a tile counts as all masked (P = 0).  Halves see every second tile, so they note
+  // (first slots of) their first tile with a score above -inf and their last one of NaN
+  // before it, and compare when they merge.
+  __shared__ int2 sblank[HALVES ? kQT : 1][kPM];
   __shared__ uint64_t xfull[HALVES ? kQT : 1][4], xdone[HALVES ? kQT : 1][4];
   __shared__ uint64_t sfull[kQT], pfull[kQT][2], odone[kQT];  // pfull: first, second half of P
   __shared__ uint32_t tmem_base;
@@ -596,6 +602,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
       const int wpos = __reduce_max_sync(0xFFFFFFFFu, mypos);
       if (mypos == kAbsent) mypos = wpos;
       float m = -INFINITY, l = 0.f;  // max used for P (log2 units) and running sum
+      if (HALVES) sblank[i][row] = make_int2(INT_MAX, -1);
       // tcgen05.ld / st are warp-collective: every lane of the warp issues each
       // one, and the wait outcomes are made warp-uniform before any branch
       for (int j = 0; j < n; ++j) {
@@ -673,17 +680,65 @@ __global__ void __launch_bounds__(kPThreads, 1)
             }
           }
         };
-        if (j == 0) m = fmaxf(half_max(0), half_max(1));
+        // The tile once more where a row of the warp has seen nothing above -inf so far:
+        // the same probabilities and sums, and zeros for those rows.  (Rare, so in a loop
+        // over S read again; as a select in the steps below it cost 3-5% of a launch.)
+        auto blank_rows = [&]() {
+          const float nm = m == -INFINITY ? 0.f : -m;
+          const float2 qs2 = make_float2(p.qscale, p.qscale), nm2 = make_float2(nm, nm);
+          float2 t = make_float2(0.f, 0.f), sa = t;
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            uint32_t x[32], u[16];
+            tc::tmem_ld32(scol + 32 * c, x);  // (P's columns 16 c .. are read by now)
+            tc::tmem_ld_wait();
+            float2 sc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < 32; e += 2) {
+              const float2 y = __ffma2_rn(
+                  make_float2(32 * c + e < vis ? __uint_as_float(x[e]) : -INFINITY,
+                              32 * c + e + 1 < vis ? __uint_as_float(x[e + 1]) : -INFINITY), qs2, nm2);
+              const float2 pr = make_float2(ex2(y.x), ex2(y.y));
+              sc = __fadd2_rn(sc, pr);
+              const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
+              u[e / 2] = m == -INFINITY ? 0u : *reinterpret_cast<const uint32_t*>(&h);
+            }
+            if (m == -INFINITY) {
+              if (HALVES && !(sc.x + sc.y == 0.f)) sblank[i][row].y = s0;
+              sc = make_float2(0.f, 0.f);
+            }
+            tc::tmem_st16(scol + 16 * c, u);
+            if ((c & 1) == 0) {
+              t = sc;
+              continue;
+            }
+            t = __fadd2_rn(t, sc);
+            if (c == 1) sa = t;
+            tc::tmem_st_wait();
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pfull[i][c >> 1]);
+          }
+          l += (sa.x + t.x) + (sa.y + t.y);
+        };
+        if (j == 0) {
+          m = fmaxf(half_max(0), half_max(1));
+          if (HALVES && m != -INFINITY) sblank[i][row].x = s0;
+        }
         half_p(0, w);
+        // Did the row's max grow past the headroom?  The first half's sum of
+        // probabilities tells (64 of at most 2^8 each stay below 2^14, and one
+        // above 2^14 shows, infinities included), the second half's max is taken
+        // beside the exponentials.
+        const float2 s2 = __fadd2_rn(sum2[0], sum2[1]);
+        float mt1 = 0.f;
+        bool raise = m == -INFINITY;
         if (j > 0) {
-          // Did the row's max grow past the headroom?  The first half's sum of
-          // probabilities tells (64 of at most 2^8 each stay below 2^14, and one
-          // above 2^14 shows, infinities included), the second half's max is taken
-          // beside the exponentials.
-          const float2 s2 = __fadd2_rn(sum2[0], sum2[1]);
-          const float mt1 = half_max(1);
-          bool raise = s2.x + s2.y > kStaleSum || mt1 > m + kStaleMax || m == -INFINITY;
-          if (__any_sync(0xFFFFFFFFu, raise)) {
+          mt1 = half_max(1);
+          raise |= s2.x + s2.y > kStaleSum || mt1 > m + kStaleMax;
+        }
+        if (__any_sync(0xFFFFFFFFu, raise)) {
+          if (j > 0) {
             // A row's max grew past the headroom: rescale O (every lane of the
             // warp takes part; rows that did not raise their max scale by 1)
             // and take the probabilities again.  P V of the previous tile is
@@ -691,24 +746,27 @@ __global__ void __launch_bounds__(kPThreads, 1)
             float scale = 1.f;
             const float mt = fmaxf(half_max(0), mt1);
             raise = raise && mt > m;  // (also false while nothing is visible)
-            // (a row of -inf so far starts anew: NaN scores may be in its sums)
-            const bool anew = raise && m == -INFINITY;
             if (raise) {
+              if (HALVES && m == -INFINITY) sblank[i][row].x = s0;
               scale = ex2(m - mt);
               m = mt;
             }
-            l = anew ? 0.f : l * scale;
+            l *= scale;
 #pragma unroll 1
             for (int c = 0; c < HD / 8; ++c) {
               uint32_t o[8];
               tc::tmem_ld8(ocol + 8 * c, o);
               tc::tmem_ld_wait();
 #pragma unroll
-              for (int e = 0; e < 8; ++e) o[e] = anew ? 0u : __float_as_uint(__uint_as_float(o[e]) * scale);
+              for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * scale);
               tc::tmem_st8(ocol + 8 * c, o);
             }
-            half_p(0, w);
           }
+          if (__any_sync(0xFFFFFFFFu, m == -INFINITY)) {
+            blank_rows();
+            continue;
+          }
+          half_p(0, w);
         }
         hand_over(0, w);
         half_p(1, w);
@@ -724,8 +782,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
       if (!ok) break;
       tc::fence_after_sync();
       // Weights of this O and of the other half's.  O counts if any P V ran (else it
-      // holds another item's rows) and the row saw a score above -inf.
-      bool own = n > 0 && m != -INFINITY, other = false;
+      // holds another item's rows) and one of its slots is visible to the row.
+      bool own = n > 0 && mypos >= (HALVES ? i * kPN : 0), other = false;
       float inv = (own && l > 0.f) ? 1.f / l : 0.f, inv1 = 0.f;
       if constexpr (HALVES) {
         sml[i][row] = make_float2(m, l);
@@ -736,10 +794,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
         if (!ok) break;
         tc::fence_after_sync();
         const float2 o = sml[i ^ 1][row];
+        const int2 mine = sblank[i][row], theirs = sblank[i ^ 1][row];
         const float mm = fmaxf(m, o.x);
-        other = items[slot].nt[i ^ 1] > 0 && o.x != -INFINITY;
-        const float a = own ? ex2(m - mm) : 0.f, b2 = other ? ex2(o.x - mm) : 0.f;
-        const float ls = (own ? a * l : 0.f) + (other ? b2 * o.y : 0.f), r = ls > 0.f ? 1.f / ls : 0.f;
+        other = items[slot].nt[i ^ 1] > 0 && mypos >= (i ^ 1) * kPN;
+        const float a = m != -INFINITY ? ex2(m - mm) : 0.f, b2 = o.x != -INFINITY ? ex2(o.x - mm) : 0.f;
+        const float ls = a * l + b2 * o.y;
+        float r = ls > 0.f ? 1.f / ls : 0.f;
+        if (mine.y > theirs.x || theirs.y > mine.x) r = NAN;
         inv = a * r;
         inv1 = b2 * r;
       }
