@@ -31,7 +31,7 @@ namespace {
 constexpr int kMixThreads = 256;
 constexpr int kChanGroup = 4; // channels mixed per CTA
 constexpr int kVecPerThread = 2;  // 8-element vectors per thread: D <= 256*8*2
-// Token counts from which the pool runs its batched form of the mix (prefill
+// Token counts from which the fp32 pool runs its batched form of the mix (prefill
 // groups): several tokens per CTA.  Below it (decode steps) one token per CTA
 // spreads the few tokens over more SMs.
 constexpr int kBatchedTokens = 64;
@@ -396,11 +396,12 @@ cudaError_t launch_simt_gemm(const GemmArgs& a, int batch, cudaStream_t s) {
 // i of the vectors is column g of MMA i, so the eight MMAs' results of one column
 // are 8 consecutive elements, one 16-byte store, and the four t of a store cover
 // 64 bytes.  RMSNorm_j's 1/RMS is left to the projection's epilogue (it is one
-// factor per token and channel), so parts of D need not meet.  Decode steps
-// (COOP): a CTA per unit, its warps share the sum of the router's many split
-// partials and a warp has one or a few 64-element steps.  Groups of tokens: a
-// warp per unit, nothing shared, the next step's states in flight while this
-// step's are used (a CTA per token spent its time waiting for them: 105 us).
+// factor per token and channel), so parts of D need not meet.  Decode steps and
+// small groups (COOP): a CTA per unit, its warps share the sum of the router's many
+// split partials and a warp has one or a few 64-element steps.  Large groups of
+// tokens (mix_token_warps): a warp per unit, nothing shared, the next step's states
+// in flight while this step's are used (as CTAs, which wait for them, 75 us at the
+// 4096 tokens below).
 //
 // Bound by memory: h in, the operand out (201 MB at 4096 tokens, L = k = 16, D =
 // 512).  There the scalar kernel before took 194 us, this one 59; at 32
@@ -443,7 +444,8 @@ __device__ __forceinline__ void mix_alpha(const MixParams& p, int b, int X, cons
 #pragma unroll(N > 2 ? 2 : 8)
   for (int s = 0; s < p.nsplit_r; ++s, zp += (int64_t)p.B * kL)
 #pragma unroll
-    for (int i = 0; i < N; ++i) a[i] += zp[o[i]];
+    for (int i = 0; i < N; ++i)
+      if (j[i] < p.k && l[i] < p.L) a[i] += zp[o[i]];
 #pragma unroll
   for (int i = 0; i < N; ++i) a[i] = j[i] < p.k && l[i] < p.L ? a[i] * r[i] : 0.f;
 }
@@ -501,8 +503,14 @@ __global__ void __launch_bounds__((COOP ? kCoopWarps : kTokenWarps) * 32, COOP ?
       for (int ks = 0; ks < KB; ++ks) load_h(c0, ks, hn[ks]);
     if (COOP) {
       if (mt > 0) __syncthreads();
-      for (int i = tid; i < 2 * 16 * KS * 8; i += NW * 32) {  // two layers at a time
-        const int lp = i % (KS * 8), rem = i / (KS * 8), jj = rem % 16, X = rem / 16;
+      // the layer pairs and channels there are; the rest of the operand is 0
+      const int npair = (L + 1) / 2, nch = min(16, p.k - mt * 16);
+      if (npair < KS * 8 || nch < 16) {
+        for (int i = tid; i < 2 * KS * 3 * 32; i += NW * 32) frag[i] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+      }
+      for (int i = tid; i < 2 * nch * npair; i += NW * 32) {  // two layers at a time
+        const int lp = i % npair, rem = i / npair, jj = rem % nch, X = rem / nch;
         float a[2];
         mix_alpha<2>(p, b, X, {mt * 16 + jj, mt * 16 + jj}, {2 * lp, 2 * lp + 1}, a);
         // operand register and lane of row jj, columns l % 16 and l % 16 + 1
@@ -984,17 +992,28 @@ __global__ void __launch_bounds__(128) kv_epilogue_kernel(const MixParams p) {
   }
 }
 
-// Parts of D the mix of one token is split into (units of mix_mma_kernel): in a
-// decode step so many CTAs that four fit each SM, down to one 64-element step per
-// warp; in a group of tokens so many warps that 16 fit each SM, down to four steps
-// per warp (each warp sums its token's alpha first).  At most 64 and at most Hkv*d
-// (the projection outputs' place holds the parts' sums).
-int mix_parts(int B, int D, int sms) {
+// Does the bf16 mix give every token to one warp (mix_mma_kernel without COOP)?  It pays
+// once there are enough tokens to fill the SMs with warps and few router splits, which
+// each warp sums by itself: below, a CTA per token or part of one.  Layers of two
+// blocks, whose next states the warp form keeps in flight, sooner.  Whole pools (us, CTA
+// form / warp form), L = 16, k = 16, D = 1024, 8 heads of 128: 49 / 60 at 128 tokens, 85
+// / 97 at 512, 136 / 159 at 1024, 210 / 218 at 1536, 247 / 247 at 2048; L = 32, k = 4, D
+// = 2048, 8 heads of 128: 67 / 110, 126 / 144, 223 / 204, 311 / 273, 400 / 348 (640: 175 /
+// 167); L = 48: 116 / 180 at 128, 678 / 698 at 1536.
+bool mix_token_warps(int B, int L) { return B >= (L > 16 && L <= 32 ? 768 : 1536); }
+
+// Parts of D the mix of one token is split into (units of mix_mma_kernel): CTAs for the
+// two that fit each SM, down to one 64-element step per warp (D = 4096: eight parts);
+// every part sums the token's alpha again, so never more (pools of 128 / 256 tokens, L =
+// 32, k = 4, D = 2048: four / three parts 85 / 116 us, two / one 73 / 93, when each part
+// also read the logits of absent channels).  In the warp form so many warps that 16 fit
+// each SM, down to four steps per warp (D = 4096: 16 parts).
+int mix_parts(int B, int L, int D, int sms) {
   const int nc = (D / 8 + 7) / 8;
-  const bool batched = B >= kBatchedTokens;
+  const bool batched = mix_token_warps(B, L);
   const int most = batched ? (nc + 3) / 4 : (nc + kCoopWarps - 1) / kCoopWarps;
-  const int want = ((batched ? 16 : 4) * sms + B - 1) / B;
-  const int parts = want < most ? want : most;
+  const int want = batched ? (16 * sms + B - 1) / B : 2 * sms / B;
+  const int parts = want < 1 ? 1 : want < most ? want : most;
   const int per = (nc + parts - 1) / parts;
   return (nc + per - 1) / per;  // no empty part
 }
@@ -1003,7 +1022,7 @@ template <typename T>
 cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   const int kL = p.k * p.L;
   const bool bf16 = sizeof(T) == 2;
-  const bool batched = p.B >= kBatchedTokens;
+  const bool batched = bf16 ? mix_token_warps(p.B, p.L) : p.B >= kBatchedTokens;
   cudaError_t e;
   {
     const int rows = p.B * p.L;
@@ -1152,8 +1171,10 @@ int kv_mix_launches(const MixParams& p, int dtype) {
 
 cudaError_t launch_kv_mix(MixParams& p, int dtype, int sms, cudaStream_t s) {
   p.sms = sms;
-  p.mix_parts = mix_parts(p.B, p.D, sms);
-  p.ssq = p.proj;  // (bf16: [2][k][parts][B] floats, within the fp32 path's projection outputs)
+  p.mix_parts = mix_parts(p.B, p.L, p.D, sms);
+  // bf16: [2][k][parts][B] floats, within the fp32 path's [2][k][B][Hkv*d] projection outputs
+  if (p.mix_parts > p.Hkv * p.d) return cudaErrorInvalidConfiguration;  // (16 parts, 64 outputs)
+  p.ssq = p.proj;
   if (dtype == WM_DT_F32) return launch_all<float>(p, s);
   return launch_all<__nv_bfloat16>(p, s);
 }
