@@ -231,205 +231,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                         mt == 0 && j == 0 && X == 0, ea, warp);
 }
 
-// ---------------------------------------------------------------- streamed projection
-// The decode projection when it has more tiles than SMs (wide models: 1024 tiles
-// of 1 MB at D = 4096, 32 heads of 128, k = 16): persistent CTAs, one per SM, so
-// that the weight stream never stops for a tile's end.  A CTA walks a contiguous
-// run of (branch, channel, 128-row) tiles; warp 0 keeps the TMA ring full across
-// tiles, warp 1 issues the MMAs into two TMEM accumulators in turn, and warps 4-7
-// finish tile i (the epilogue of proj_tc_kernel) while tile i + 1 streams.  One
-// token tile (fewer than kRowsTokens tokens).  Bound by the weight stream: 1.07 GB
-// there, 205 us with proj_tc_kernel (3.4 waves of CTAs), 195 us with this.
-constexpr int kStreamThreads = 256;
-constexpr int kStreamMaxStages = 12;
-// k-blocks loaded together: a block takes 128 bytes of each of 128 rows, four in
-// a row take 512, which DRAM serves better.
-constexpr int kStreamBurst = 4;
-constexpr int kStreamEpi0 = 4, kStreamEpiWarps = 4;
-
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-template <int HD>
-__global__ void __launch_bounds__(kStreamThreads, 1)
-    proj_stream_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
-                       const __grid_constant__ CUtensorMap tmX, const ProjTcParams p, int mtiles,
-                       int tiles) {
-  extern __shared__ uint8_t smem_dyn[];
-  __shared__ uint64_t full[kStreamMaxStages], empty[kStreamMaxStages], afull[2], aempty[2];
-  __shared__ uint32_t tmem_base;
-  __shared__ int s_slot[kRowsTokens], s_page[kRowsTokens], s_ok[kStreamEpiWarps];
-  __shared__ float s_scale[kRowsTokens];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int NS = p.stages;
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) &
-                                             ~static_cast<uintptr_t>(1023));
-  const uint32_t a_bytes = kTcM * 128, b_bytes = (uint32_t)p.BN * 128;
-  uint8_t* As = base;
-  uint8_t* Bs = As + NS * a_bytes;
-  float* T = reinterpret_cast<float*>(Bs + NS * b_bytes);  // [BN][128]
-  float* rope_s = T + p.BN * kTcM;                         // [BN][HD/2][2]
-  constexpr int HPT = kTcM / HD;
-  const int x0 = (int)((int64_t)blockIdx.x * tiles / gridDim.x);
-  const int x1 = (int)((int64_t)(blockIdx.x + 1) * tiles / gridDim.x);
-  const int nkb = (x1 - x0) * p.nk;  // k-blocks of this CTA
-  // tile x: 128-row tile mt of channel j, branch X
-  auto wrow_of = [&](int x) { return (x / mtiles % p.k) * p.M_item + x % mtiles * HPT * HD; };
-  auto branch_of = [&](int x) { return x / (mtiles * p.k); };
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < NS; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&afull[i], 1);
-      mbar_init(&aempty[i], kStreamEpiWarps);
-    }
-    fence_mbar_init();
-    tc::prefetch_tensormap(&tmW0);
-    tc::prefetch_tensormap(&tmW1);
-    tc::prefetch_tensormap(&tmX);
-    // weights no earlier kernel writes: the first ring's worth before the wait
-    // (see proj_tc_kernel)
-    for (int c = 0; c < NS && c < nkb; ++c) {
-      const int x = x0 + c / p.nk;
-      mbar_expect_tx(&full[c], a_bytes);
-      tc::tma_load_2d(As + c * a_bytes, branch_of(x) == 0 ? &tmW0 : &tmW1, c % p.nk * kTcBK,
-                      wrow_of(x), &full[c]);
-    }
-  }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (warp == 0) {
-    tc::tmem_alloc(&tmem_base, p.tmem_cols);
-    tc::tmem_relinquish();
-  }
-  // the tokens' destinations and RoPE table, once
-  for (int n = threadIdx.x; n < p.B; n += kStreamThreads) {
-    const int s = p.slot[n];
-    int pg = -1;
-    if (s >= 1 && s < p.max_pages * p.P)
-      pg = p.page_table[(int64_t)n * p.max_pages + (s >> p.log2P)];
-    s_slot[n] = s;
-    s_page[n] = (pg >= 0 && pg < p.num_pages) ? pg : -1;
-  }
-  for (int i = threadIdx.x; i < p.B * HD; i += kStreamThreads) rope_s[i] = p.rope_cs[i];
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = tmem_base;
-
-  if (warp == 0) {
-    if (tc::elect_one()) {
-      bool ok = true;
-      int x = x0, kb = 0;
-      const int burst = NS % kStreamBurst == 0 ? kStreamBurst : 1;
-      for (int c = 0; c < nkb; ++c) {
-        const int s = c % NS, X = branch_of(x);
-        const int xrow = (X * p.k + x / mtiles % p.k) * p.B;
-        if (c < NS) {
-          mbar_arrive_expect_tx(&full[s], b_bytes);
-        } else {
-          if (c % burst == 0) {  // (the ring is a multiple of the burst)
-            // the last of the burst's stages: the ones before it were freed before it
-            const int e = min(c + burst - 1, nkb - 1);
-            ok = mbar_wait(&empty[e % NS], ((e / NS) - 1) & 1);
-            if (!ok) break;
-          }
-          mbar_arrive_expect_tx(&full[s], a_bytes + b_bytes);
-          tc::tma_load_2d(As + s * a_bytes, X == 0 ? &tmW0 : &tmW1, kb * kTcBK, wrow_of(x), &full[s]);
-        }
-        tc::tma_load_2d(Bs + s * b_bytes, &tmX, kb * kTcBK, xrow, &full[s]);
-        if (++kb == p.nk) {
-          kb = 0;
-          ++x;
-        }
-      }
-      if (!ok) report(p.status, WM_ERR_TIMEOUT);
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    if (tc::elect_one()) {
-      const uint32_t idesc = tc::idesc_bf16_f32(kTcM, p.BN);
-      const uint64_t ad0 = tc::sdesc_kmajor_sw128(smem_u32(As)), bd0 = tc::sdesc_kmajor_sw128(smem_u32(Bs));
-      bool ok = true;
-      int c = 0;
-      for (int x = x0; x < x1 && ok; ++x) {
-        const int i = x - x0, a = i & 1;
-        if (i >= 2) ok = mbar_wait_spin(&aempty[a], ((i >> 1) - 1) & 1);
-        if (!ok) break;
-        tc::fence_after_sync();
-        for (int kb = 0; kb < p.nk; ++kb, ++c) {
-          const int s = c % NS;
-          ok = mbar_wait_spin(&full[s], (c / NS) & 1);
-          if (!ok) break;
-          tc::fence_after_sync();
-          const uint64_t ad = ad0 + (uint64_t)(s * (a_bytes >> 4)), bd = bd0 + (uint64_t)(s * (b_bytes >> 4));
-#pragma unroll
-          for (int kk = 0; kk < kTcBK / 16; ++kk)
-            tc::mma_bf16(tmem + a * p.BN, ad + kk * 2, bd + kk * 2, idesc, (kb | kk) != 0);
-          tc::mma_commit(&empty[s]);
-        }
-        if (ok) tc::mma_commit(&afull[a]);
-      }
-      if (!ok) report(p.status, WM_ERR_TIMEOUT);
-    }
-    __syncwarp();
-  } else if (warp >= kStreamEpi0) {
-    const int ew = warp - kStreamEpi0, et = threadIdx.x - kStreamEpi0 * 32;
-    KvEpiArgs ea;
-    ea.Hkv = p.Hkv;
-    ea.P = p.P;
-    ea.num_pages = p.num_pages;
-    ea.eps_qk = p.eps_qk;
-    ea.qk_g = p.qk_g;
-    ea.k_pool = p.k_pool;
-    ea.v_pool = p.v_pool;
-    ea.status = p.status;
-    for (int x = x0; x < x1; ++x) {
-      const int i = x - x0, a = i & 1;
-      const int mt = x % mtiles, j = x / mtiles % p.k, X = branch_of(x);
-      if (et < p.B) {
-        const float* sq = p.ssq + (int64_t)(X * p.k + j) * p.parts * p.B + et;
-        float v = 0.f;
-        for (int q = 0; q < p.parts; ++q) v += sq[(int64_t)q * p.B];
-        s_scale[et] = rsqrtf(v * p.inv_D + p.eps_rms);
-      }
-      const bool mine = __all_sync(0xFFFFFFFFu, mbar_wait(&afull[a], (i >> 1) & 1));
-      tc::fence_after_sync();
-      if (mine) {
-        const uint32_t quad = (uint32_t)(ew * 32) << 16;
-        for (int c0 = 0; c0 < p.BN; c0 += 16) {
-          uint32_t r[16];
-          tc::tmem_ld16(tmem + quad + (uint32_t)(a * p.BN + c0), r);
-          tc::tmem_ld_wait();
-#pragma unroll
-          for (int q = 0; q < 16; ++q) T[(c0 + q) * kTcM + ew * 32 + lane] = __uint_as_float(r[q]);
-        }
-      }
-      tc::fence_before_sync();
-      // the four warps go on or give up together: none is left at the barrier
-      if (lane == 0) {
-        s_ok[ew] = mine;
-        if (mine) mbar_arrive(&aempty[a]);
-      }
-      epi_sync();
-      if (!(s_ok[0] && s_ok[1] && s_ok[2] && s_ok[3])) {
-        if (et == 0) report(p.status, WM_ERR_TIMEOUT);
-        break;
-      }
-      kv_epilogue_tile<HD, kStreamEpiWarps>(T, p.B, mt, j, X, s_scale, s_slot, s_page, rope_s, 0,
-                                            mt == 0 && j == 0 && X == 0, ea, ew);
-      epi_sync();  // T and the scales may be written again
-    }
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, p.tmem_cols);
-  }
-}
-
 // Row-major bf16 matrix [rows][cols] as a 2-D tensor map with a 64 x box_rows box.
 bool encode_kmajor(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
   return tma_map_bf16_2d(tm, ptr, rows, cols, cols, box_rows);
@@ -441,20 +242,19 @@ uint32_t pow2_at_least(uint32_t x, uint32_t lo) {
   return r;
 }
 
-int sm_count_cur() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-    n = 148;
-  return n;
-}
-
 // Pipeline depth: deep enough to keep one round trip of weights in flight;
-// shallow enough for two CTAs per SM when the grid has more than one wave.
-int pick_stages(int nkb, int BN, int64_t grid, int sms) {
+// shallow enough for two CTAs per SM when the grid has more than one wave, also beside
+// `extra` bytes of table (with 4 KB of static and reserved memory each, two CTAs of 108
+// KB fit), as long as two stages do.  One CTA's weights then stream while the other's
+// tile ends.  Pools of L = 16, k = 16, 32 heads of 128, D = 4096 (us; 100 KB of stages
+// whatever the table, so one CTA per SM / so): 239 / 210 at 32 tokens, 253 / 225 at
+// 48, 255 / 227 at 64, 290 / 267 at 96; D = 1024: 94 / 81, 101 / 87, 106 / 91, 132 / 120.
+int pick_stages(int nkb, int BN, int64_t grid, int sms, int extra) {
   const int stage_bytes = kTcM * 128 + BN * 128;
   const int budget = grid > sms ? 100 * 1024 : 200 * 1024;
   int ns = budget / stage_bytes;
+  const int two = (107 * 1024 - extra) / stage_bytes;  // (1 KB goes to the base's alignment)
+  if (grid > sms && two >= 2 && two < ns) ns = two;
   ns = ns < 2 ? 2 : (ns > kTcMaxStages ? kTcMaxStages : ns);
   return ns > nkb ? (nkb < 2 ? 2 : nkb) : ns;
 }
@@ -463,32 +263,6 @@ size_t tc_smem(int stages, int BN) {
   const size_t pipe = (size_t)stages * (kTcM * 128 + BN * 128);
   const size_t tile = (size_t)BN * kTcM * sizeof(float);  // epilogue reuses the stages
   return (pipe > tile ? pipe : tile) + 1024;
-}
-
-template <int HD>
-cudaError_t launch_stream(const CUtensorMap& w0, const CUtensorMap& w1, const CUtensorMap& x,
-                          ProjTcParams p, int mtiles, int sms, cudaStream_t s) {
-  const size_t fixed = (size_t)p.BN * kTcM * 4 + (size_t)p.BN * HD * 4 + 1024;
-  const size_t stage = kTcM * 128 + (size_t)p.BN * 128;
-  int ns = (int)(((size_t)222 * 1024 - fixed) / stage);
-  ns = ns < 2 ? 2 : ns > kStreamMaxStages ? kStreamMaxStages : ns;
-  p.stages = ns > kStreamBurst ? ns / kStreamBurst * kStreamBurst : ns;
-  const size_t smem = fixed + p.stages * stage;
-  p.tmem_cols = pow2_at_least(2 * (uint32_t)p.BN, 32);
-  static size_t smem_set[kSmemOptDevices] = {};
-  auto kern = proj_stream_kernel<HD>;
-  if (cudaError_t e = opt_in_smem(kern, smem, smem_set); e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)sms);
-  cfg.blockDim = dim3(kStreamThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, w0, w1, x, p, mtiles, 2 * p.k * mtiles);
 }
 
 template <int HD, int MODE>
@@ -570,15 +344,9 @@ cudaError_t launch_proj_tc(const MixParams& mp, cudaStream_t s) {
   const int hpt = kTcM / mp.d;
   const int ntiles = (mp.B + p.BN - 1) / p.BN;
   dim3 grid((mp.Hkv + hpt - 1) / hpt, mp.k, 2 * ntiles);
-  // more tiles than SMs, all of one token tile: stream them
-  if (mp.B < kRowsTokens && (int64_t)grid.x * grid.y * grid.z > mp.sms) {
-    if (mp.d == 64) return launch_stream<64>(tmW[0], tmW[1], tmX, p, (int)grid.x, mp.sms, s);
-    if (mp.d == 96) return launch_stream<96>(tmW[0], tmW[1], tmX, p, (int)grid.x, mp.sms, s);
-    return launch_stream<128>(tmW[0], tmW[1], tmX, p, (int)grid.x, mp.sms, s);
-  }
-  p.stages = pick_stages(p.nk, p.BN, (int64_t)grid.x * grid.y * grid.z, sm_count_cur());
-  size_t smem = tc_smem(p.stages, p.BN);
   const size_t rope_bytes = (size_t)p.BN * mp.d * sizeof(float);
+  p.stages = pick_stages(p.nk, p.BN, (int64_t)grid.x * grid.y * grid.z, mp.sms, (int)rope_bytes);
+  size_t smem = tc_smem(p.stages, p.BN);
   if (smem + rope_bytes <= 200 * 1024) {
     p.rope_smem_off = (int32_t)(smem - 1024);  // offset from the 1 KB-aligned base
     smem += rope_bytes;
@@ -608,7 +376,7 @@ cudaError_t launch_router_tc(const MixParams& mp, cudaStream_t s) {
   if (!encode_kmajor(&tmX, mp.xi, (uint64_t)2 * mp.B, K, (uint32_t)p.BN))
     return cudaErrorInvalidValue;
   dim3 grid((kL + kTcM - 1) / kTcM, mp.nsplit_r, 2 * ((mp.B + p.BN - 1) / p.BN));
-  p.stages = pick_stages(p.kb_per_split, p.BN, (int64_t)grid.x * grid.y * grid.z, sm_count_cur());
+  p.stages = pick_stages(p.kb_per_split, p.BN, (int64_t)grid.x * grid.y * grid.z, mp.sms, 0);
   const size_t smem = tc_smem(p.stages, p.BN);
   return launch_mode<64, kEpiPartial>(grid, smem, tmW[0], tmW[1], tmX, p, s);
 }
