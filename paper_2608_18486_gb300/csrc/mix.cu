@@ -116,9 +116,10 @@ __global__ void __launch_bounds__(kPrenormWarps * 32) prenorm_kernel(const MixPa
   const int row = blockIdx.x * (kPrenormWarps / WPR) + warp / WPR;  // b * L + l
   const int u = (warp % WPR) * 32 + lane, nu = WPR * 32;            // thread of the row
   pdl_wait();
-  if (WPR == 1 && row >= p.B * p.L) return;
+  const bool there = row < p.B * p.L;
+  if (WPR == 1 && !there) return;
   const int b = row / p.L, l = row % p.L;
-  const int nvec = p.D / 8;
+  const int nvec = there ? p.D / 8 : 0;
   const T* hp = reinterpret_cast<const T*>(p.h) + (int64_t)row * p.D;
   float f[MAXV][8], ss = 0.f;
 #pragma unroll
@@ -139,7 +140,8 @@ __global__ void __launch_bounds__(kPrenormWarps * 32) prenorm_kernel(const MixPa
     __syncthreads();
     ss = 0.f;
 #pragma unroll
-    for (int w = 0; w < kPrenormWarps; ++w) ss += red[w];
+    for (int w = 0; w < WPR; ++w) ss += red[warp / WPR * WPR + w];
+    if (!there) return;
   }
   const float r = rsqrtf(ss / (float)p.D + p.eps_rms);
   if (u == 0) p.inv_rms[row] = r;
@@ -1026,12 +1028,14 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
   cudaError_t e;
   {
     const int rows = p.B * p.L;
-    // a row of at most 1024 elements fits one warp's registers
-    if (p.D <= 1024)
-      e = launch_pdl(prenorm_kernel<T, 1>, dim3((rows + kPrenormWarps - 1) / kPrenormWarps),
-                     dim3(kPrenormWarps * 32), 0, s, p);
-    else
-      e = launch_pdl(prenorm_kernel<T, kPrenormWarps>, dim3(rows), dim3(kPrenormWarps * 32), 0, s, p);
+    // as few warps to a row as hold it in registers, 1024 elements each
+    auto go = [&](auto kern, int wpr) {
+      const int per = kPrenormWarps / wpr;
+      return launch_pdl(kern, dim3((rows + per - 1) / per), dim3(kPrenormWarps * 32), 0, s, p);
+    };
+    e = p.D <= 1024   ? go(prenorm_kernel<T, 1>, 1)
+        : p.D <= 2048 ? go(prenorm_kernel<T, 2>, 2)
+                      : go(prenorm_kernel<T, 4>, 4);
   }
   if (e != cudaSuccess) return e;
   if (bf16 && router_tc_supported(p.B)) {
