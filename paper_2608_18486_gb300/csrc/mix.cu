@@ -378,8 +378,12 @@ cudaError_t launch_simt_gemm(const GemmArgs& a, int batch, cudaStream_t s) {
     if (a.N <= 4) return go(gemv_wxT_f32<4, 4, 2>, 4, 4);
     return go(gemv_wxT_f32<8, 4, 2>, 8, 4);
   }
-  return launch_pdl(gemm_wxT_simt<T, T>, dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), dim3(256), 0,
-                    s, a);
+  // Without programmatic launch: placed while the predecessor runs, the few tiles land
+  // side by side on the SMs that have room, and the product takes two or three times as
+  // long (pool of L = 16, k = 8, D = 1024, 8 heads of 64: 227-302 us at 32 tokens, by what
+  // the kernels before it look like; 105 so; 257 and 137 at 64, 394 and 199 at 128).
+  gemm_wxT_simt<T, T><<<dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), 256, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- mix (bf16)
