@@ -322,14 +322,17 @@ struct CopyShape {
 
 // One stage's copies, issued by all lanes of a warp together: slots s_begin
 // .. of one sequence (S slots long) and kv head into kd / vd, completing on
-// `bar` (with extra_bytes more to come).  page(i, o): page id of logical page i + o
-// (o per lane).  Returns the mask of V runs on valid pages, which `consume`
-// takes; bit i covers slots i * min(P, kVRun) ...
-template <typename MATH, typename T, int HD, int SLOTS, typename PageOf>
+// `bar` (with extra_bytes more, which `extra` copies in one lane).  page(i, o): page id
+// of logical page i + o (o per lane).  Returns the mask of V runs on valid pages, which
+// `consume` takes; bit i covers slots i * min(P, kVRun) ...  The issue of a stage is
+// a good part of its time: with the runs of V and K taken apart for contiguous tiles too,
+// 32 ragged sequences of up to 8192 slots, 32 heads of 64, took 295 us for 285 (of 96: 433
+// and 424; of 128: 512 and 510).
+template <typename MATH, typename T, int HD, int SLOTS, typename PageOf, typename Extra>
 __device__ __forceinline__ void copy_stage(const AttnParams& p, const T* kb, const T* vb, int s_begin,
                                            int S, T* kd, T* vd, uint64_t* bar, uint64_t* mask_out,
                                            uint32_t extra_bytes, uint64_t policy, int lane,
-                                           PageOf page) {
+                                           PageOf page, Extra extra) {
   using CS = CopyShape<MATH, SLOTS>;
   constexpr uint32_t ROW = HD * sizeof(T);
   if (p.P >= SLOTS && CS::kVRun == SLOTS) {  // one copy of each
@@ -344,6 +347,26 @@ __device__ __forceinline__ void copy_stage(const AttnParams& p, const T* kb, con
         bulk_g2s(kd, kb + off, SLOTS * ROW, bar, policy);
         bulk_g2s(vd, vb + off, SLOTS * ROW, bar, policy);
       }
+      extra();
+    }
+  } else if constexpr (MATH::kBlocks == 1) {  // lane i copies the i-th page of both
+    const int npp = SLOTS >> p.log2P;  // pages per stage (<= 32)
+    const int lp0 = s_begin >> p.log2P;
+    const int lpn = min(npp, ((S - 1) >> p.log2P) - lp0 + 1);
+    const int pg = page(lp0, lane < lpn ? lane : 0);
+    const bool ok = lane < lpn && pg >= 0 && pg < p.num_pages;
+    const uint32_t mask = __ballot_sync(0xFFFFFFFFu, ok), bytes = (uint32_t)p.P * ROW;
+    if (lane == 0) {
+      *mask_out = mask;
+      if (__popc(mask) < lpn) report(p.status, WM_ERR_BOUNDS);
+      mbar_arrive_expect_tx(bar, 2u * bytes * (uint32_t)__popc(mask) + extra_bytes);
+      extra();
+    }
+    __syncwarp();
+    if (ok) {
+      const int64_t off = (int64_t)pg * p.page_stride;
+      bulk_g2s(kd + lane * p.P * HD, kb + off, bytes, bar, policy);
+      bulk_g2s(vd + lane * p.P * HD, vb + off, bytes, bar, policy);
     }
   } else {  // lane i copies the i-th run of V, and of K where one starts there
     const int vr = min(p.P, CS::kVRun), kr = min(p.P, SLOTS);
@@ -357,6 +380,7 @@ __device__ __forceinline__ void copy_stage(const AttnParams& p, const T* kb, con
       *mask_out = mask;
       if (__popc(mask) < n) report(p.status, WM_ERR_BOUNDS);
       mbar_arrive_expect_tx(bar, (uint32_t)(vr * __popc(mask) + kr * __popc(maskk)) * ROW + extra_bytes);
+      extra();
     }
     __syncwarp();
     const int64_t off = (int64_t)pg * p.page_stride + (int64_t)((s_begin + slot) & (p.P - 1)) * HD;
@@ -562,8 +586,10 @@ __global__ void __launch_bounds__(kThreads, attn_ctas_per_sm(SB, G)) decode_attn
     const uint32_t qb = with_q ? Q_BYTES : 0u;
     const T* qsrc = reinterpret_cast<const T*>(p.q) + ((int64_t)pc.b * p.Hq + pc.h * G) * HD;
     copy_stage<MATH, T, HD, STAGE_SLOTS>(p, kb, vb, s_begin, S, kd, vd, bar, &masks[warp][buf], qb, policy,
-                                         lane, [&](int lp, int o) { return page_of(pc.b, lp, o); });
-    if (with_q && lane == 0) bulk_g2s(myq + buf * G * HD, qsrc, Q_BYTES, bar, policy);
+                                         lane, [&](int lp, int o) { return page_of(pc.b, lp, o); },
+                                         [&]() {
+                                           if (with_q) bulk_g2s(myq + buf * G * HD, qsrc, Q_BYTES, bar, policy);
+                                         });
     ++pseq;
     ++px;
     advance(pc, pre, B, Hkv);

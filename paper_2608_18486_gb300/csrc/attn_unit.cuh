@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(NW * 32, unit_min_blocks(NW, G, HD)) decode_at
     uint64_t* bar = &bars[warp][buf];
     const int s_begin = s * STAGE_SLOTS;
     attn_detail::copy_stage<MATH, T, HD, STAGE_SLOTS>(p, kbase, vbase, s_begin, S, kd, vd, bar,
-                                                      &masks[warp][buf], 0u, policy, lane, page_of);
+                                                      &masks[warp][buf], 0u, policy, lane, page_of, []() {});
   };
 
   int issued = 0;
