@@ -52,7 +52,8 @@ __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <typename... KArgs, typename... Args>
+// PDL: may start before its predecessor has ended.
+template <bool PDL = true, typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -64,7 +65,7 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = PDL ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
@@ -382,8 +383,8 @@ cudaError_t launch_simt_gemm(const GemmArgs& a, int batch, cudaStream_t s) {
   // side by side on the SMs that have room, and the product takes two or three times as
   // long (pool of L = 16, k = 8, D = 1024, 8 heads of 64: 227-302 us at 32 tokens, by what
   // the kernels before it look like; 105 so; 257 and 137 at 64, 394 and 199 at 128).
-  gemm_wxT_simt<T, T><<<dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl<false>(gemm_wxT_simt<T, T>, dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), dim3(256),
+                           0, s, a);
 }
 
 // ---------------------------------------------------------------- mix (bf16)
