@@ -451,8 +451,7 @@ __device__ __forceinline__ void mix_alpha(const MixParams& p, int b, int X, cons
 #pragma unroll(N > 2 ? 2 : 8)
   for (int s = 0; s < p.nsplit_r; ++s, zp += (int64_t)p.B * kL)
 #pragma unroll
-    for (int i = 0; i < N; ++i)
-      if (j[i] < p.k && l[i] < p.L) a[i] += zp[o[i]];
+    for (int i = 0; i < N; ++i) a[i] += zp[o[i]];
 #pragma unroll
   for (int i = 0; i < N; ++i) a[i] = j[i] < p.k && l[i] < p.L ? a[i] * r[i] : 0.f;
 }
