@@ -156,6 +156,52 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// P of a KV tile for a warp in which a row has seen no score above -inf yet (m =
+// -inf): zeros for such rows, and *nan_tile = s0 where they have NaN scores in the tile;
+// for the others the probabilities and sums of the steps in the kernel.  S at scol is
+// read again and P handed over half by half; returns the sum.  Rare, so a loop in a
+// function of its own (32 heads of 128, two prompts of 8192: 672 us without it, 674 so,
+// 684 as a branch of the step; as selects in the step 683 where 666 without).
+__device__ __noinline__ float blank_tile(uint32_t scol, int vis, float m, float qscale, uint64_t* pfull,
+                                         int lane, int* nan_tile, int s0) {
+  const float nm = m == -INFINITY ? 0.f : -m;
+  const float2 qs2 = make_float2(qscale, qscale), nm2 = make_float2(nm, nm);
+  float2 t = make_float2(0.f, 0.f), sa = t;
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    uint32_t x[32], w[16];
+    tc::tmem_ld32(scol + 32 * c, x);  // (P's columns 16 c .. are read by now)
+    tc::tmem_ld_wait();
+    float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < 32; e += 2) {
+      const float2 y = __ffma2_rn(make_float2(32 * c + e < vis ? __uint_as_float(x[e]) : -INFINITY,
+                                              32 * c + e + 1 < vis ? __uint_as_float(x[e + 1]) : -INFINITY),
+                                  qs2, nm2);
+      const float2 pr = make_float2(ex2(y.x), ex2(y.y));
+      sum = __fadd2_rn(sum, pr);
+      const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
+      w[e / 2] = m == -INFINITY ? 0u : *reinterpret_cast<const uint32_t*>(&h);
+    }
+    if (m == -INFINITY) {
+      if (nan_tile != nullptr && !(sum.x + sum.y == 0.f)) *nan_tile = s0;
+      sum = make_float2(0.f, 0.f);
+    }
+    tc::tmem_st16(scol + 16 * c, w);
+    if ((c & 1) == 0) {
+      t = sum;
+      continue;
+    }
+    t = __fadd2_rn(t, sum);
+    if (c == 1) sa = t;
+    tc::tmem_st_wait();
+    tc::fence_before_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&pfull[c >> 1]);
+  }
+  return (sa.x + t.x) + (sa.y + t.y);
+}
+
 template <int HD, bool HALVES>
 __global__ void __launch_bounds__(kPThreads, 1)
     prefill_attn_kernel(const __grid_constant__ CUtensorMap tmQ,
@@ -680,47 +726,6 @@ __global__ void __launch_bounds__(kPThreads, 1)
             }
           }
         };
-        // The tile once more where a row of the warp has seen nothing above -inf so far:
-        // the same probabilities and sums, and zeros for those rows.  (Rare, so in a loop
-        // over S read again; as a select in the steps below it cost 3-5% of a launch.)
-        auto blank_rows = [&]() {
-          const float nm = m == -INFINITY ? 0.f : -m;
-          const float2 qs2 = make_float2(p.qscale, p.qscale), nm2 = make_float2(nm, nm);
-          float2 t = make_float2(0.f, 0.f), sa = t;
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t x[32], u[16];
-            tc::tmem_ld32(scol + 32 * c, x);  // (P's columns 16 c .. are read by now)
-            tc::tmem_ld_wait();
-            float2 sc = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int e = 0; e < 32; e += 2) {
-              const float2 y = __ffma2_rn(
-                  make_float2(32 * c + e < vis ? __uint_as_float(x[e]) : -INFINITY,
-                              32 * c + e + 1 < vis ? __uint_as_float(x[e + 1]) : -INFINITY), qs2, nm2);
-              const float2 pr = make_float2(ex2(y.x), ex2(y.y));
-              sc = __fadd2_rn(sc, pr);
-              const __nv_bfloat162 h = __floats2bfloat162_rn(pr.x, pr.y);
-              u[e / 2] = m == -INFINITY ? 0u : *reinterpret_cast<const uint32_t*>(&h);
-            }
-            if (m == -INFINITY) {
-              if (HALVES && !(sc.x + sc.y == 0.f)) sblank[i][row].y = s0;
-              sc = make_float2(0.f, 0.f);
-            }
-            tc::tmem_st16(scol + 16 * c, u);
-            if ((c & 1) == 0) {
-              t = sc;
-              continue;
-            }
-            t = __fadd2_rn(t, sc);
-            if (c == 1) sa = t;
-            tc::tmem_st_wait();
-            tc::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&pfull[i][c >> 1]);
-          }
-          l += (sa.x + t.x) + (sa.y + t.y);
-        };
         if (j == 0) {
           m = fmaxf(half_max(0), half_max(1));
           if (HALVES && m != -INFINITY) sblank[i][row].x = s0;
@@ -763,7 +768,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             }
           }
           if (__any_sync(0xFFFFFFFFu, m == -INFINITY)) {
-            blank_rows();
+            l += blank_tile(scol, vis, m, p.qscale, pfull[i], lane, HALVES ? &sblank[i][row].y : nullptr, s0);
             continue;
           }
           half_p(0, w);
