@@ -91,12 +91,15 @@ constexpr int kAttnMinStagesPerWarp = 4;
 constexpr double kAttnUnitMinWarpShare = 0.6;
 
 // With four or eight query heads (8 warps per CTA, one CTA per SM) more units than
-// SMs do not fit; bf16 launches of at most this many bytes of K and V then take CTAs
-// of 4 warps, two per SM.  Four calls and a pool, 256 units of 500-1000 slots, four /
-// eight heads of 64: 90 / 98 us on stream-K, 66 / 72 so; of 128: 120 / 134 and 101 /
-// 110.  Past the line it depends on the lengths (200 units of 64: 3000-6000 slots,
-// 303 MB, 212 and 235; 256 of 64: 388 MB 276 and 254).
-constexpr double kAttnUnitNarrowBytes = 3.0e8;
+// SMs do not fit; bf16 launches whose units have room for at most this many bytes of K
+// and V then take CTAs of 4 warps, two per SM.  The line is for lengths that differ: one
+// CTA streams the longest unit at about 25 KB/us, stream-K spreads it.  26 x 8 units, four
+// heads of 64, one sequence at full length, the rest at a tenth or less (us, stream-K /
+// so): 307 KB a unit 20.7 / 16.6, 512 KB 22.8 / 24.6, 768 KB 24.6 / 32.8, 1.15 MB 29.7 /
+// 43.3; eight heads of 128: 614 KB 28.9 / 27.7, 1.02 MB 38.9 / 42.0.  With near-equal
+// lengths it wins up to the line and past it (of stream-K's time: 400-600 KB 0.61-1.05,
+// 0.8-1.1 MB 0.79-1.03).
+constexpr double kAttnUnitNarrowBytes = 6.0e5;
 
 // Resident clusters of C unit-split CTAs of `warps` warps for (dtype, d, G) on this
 // device, cached (0: unknown or no device).
@@ -179,7 +182,7 @@ AttnPlan attn_plan(const wm_config& c, int32_t B, int32_t max_pages, uint32_t fl
       return C;
     };
     int C = fit(unit_warps);
-    if (C == 0 && unit_warps == 8 && c.dtype == WM_DT_BF16 && kv_bytes <= kAttnUnitNarrowBytes) {
+    if (C == 0 && unit_warps == 8 && c.dtype == WM_DT_BF16 && kv_bytes <= kAttnUnitNarrowBytes * units) {
       unit_warps = 4;
       C = fit(unit_warps);
     }
