@@ -156,8 +156,7 @@ int kv_mix_launches(const MixParams& p, int dtype);  // kernels launch_kv_mix en
 // router with split-K fp32 partials (bf16 only)
 bool proj_tc_supported(const MixParams& p);
 cudaError_t launch_proj_tc(const MixParams& p, cudaStream_t s);
-bool router_tc_supported(int B);
-int router_tc_splits(int k, int L, int Lp, int D, int B, int sms);
+int router_tc_splits(int k, int L, int Lp, int D, int sms);
 cudaError_t launch_router_tc(const MixParams& p, cudaStream_t s);
 // the same for groups of tokens (proj_rows.cu), from kRowsTokens tokens on
 constexpr int kRowsTokens = 128;

@@ -6,17 +6,18 @@
 //                  input xi = [hhat_{L-1}, hhat_{L-1-p}, ...] for both branches;
 //                  per token the RoPE cos/sin at pos = slot - 1.
 //   2. router    : z = Wr[X] xi (split over the L'D reduction), fp32 partials;
-//                  tcgen05 for bf16 (proj_tc.cu), SIMT FMA for fp32.
+//                  tcgen05 for bf16 (proj_tc.cu, proj_rows.cu), FMA for fp32.
 //   3. mix       : alpha = reshape(z + br), htilde_j = sum_l alpha[j][l] hhat_l;
 //                  bf16: on the tensor cores, the operand is htilde_j times the
 //                  RMSNorm_j gain and the sum of squares goes to the projection's
 //                  epilogue, which scales by 1/RMS; fp32: RMSNorm_j here.
 //   4. projection: W^X_j x^X_j for every branch and channel; for bf16 on
-//                  tcgen05 with the epilogue fused (proj_tc.cu).
+//                  tcgen05 with the epilogue fused (proj_tc.cu, proj_rows.cu).
 //   5. epilogue  : (fp32) keys: per-head QK-norm then RoPE; keys and values
 //                  are written to the token's cache slot.
-// Every kernel is launched with programmatic dependent launch and waits for
-// its predecessor with griddepcontrol.wait before reading anything.
+// The kernels are launched with programmatic dependent launch (but gemm_wxT_simt, see
+// launch_gemm_f32) and wait for their predecessor with griddepcontrol.wait before they
+// read anything but weights.
 #include <math.h>
 
 #include <utility>
@@ -198,21 +199,6 @@ struct GemmArgs {
   int M, N, K, nsplit, k_per_split;
 };
 
-template <typename T>
-__device__ __forceinline__ void load8(const T* src, float* f);
-template <>
-__device__ __forceinline__ void load8<float>(const float* src, float* f) {
-  const float4 a = *reinterpret_cast<const float4*>(src);
-  const float4 c = *reinterpret_cast<const float4*>(src + 4);
-  f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
-  f[4] = c.x; f[5] = c.y; f[6] = c.z; f[7] = c.w;
-}
-template <>
-__device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* src, float* f) {
-  Elem<__nv_bfloat16>::unpack(*reinterpret_cast<const uint4*>(src), f);
-}
-
-template <typename TW, typename TX>
 __global__ void __launch_bounds__(256) gemm_wxT_simt(const GemmArgs a) {
   __shared__ float Ws[BK][BM + 4];
   __shared__ float Xs[BK][BN + 4];
@@ -220,9 +206,9 @@ __global__ void __launch_bounds__(256) gemm_wxT_simt(const GemmArgs a) {
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
   const int kbeg = split * a.k_per_split;
   const int kend = min(a.K, kbeg + a.k_per_split);
-  const TW* W = reinterpret_cast<const TW*>(a.W[bi / a.per_branch]) +
+  const float* W = reinterpret_cast<const float*>(a.W[bi / a.per_branch]) +
                 (int64_t)(bi % a.per_branch) * a.w_stride;
-  const TX* X = reinterpret_cast<const TX*>(a.X) + (int64_t)bi * a.x_stride;
+  const float* X = reinterpret_cast<const float*>(a.X) + (int64_t)bi * a.x_stride;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   pdl_wait();
   float acc[4][2] = {};
@@ -232,7 +218,7 @@ __global__ void __launch_bounds__(256) gemm_wxT_simt(const GemmArgs a) {
       const int m = m0 + r, k = k0 + kk;
       float f[8];
       if (m < a.M && k + 8 <= kend) {
-        load8<TW>(W + (int64_t)m * a.K + k, f);
+        load8f<float>(W + (int64_t)m * a.K + k, f);
       } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -365,10 +351,9 @@ __global__ void __launch_bounds__(kGemvWarps * 32) gemv_wxT_f32(const GemmArgs a
 }
 
 // out[batch][split][n][m] = sum over the split's k of W[m][k] X[n][k]
-template <typename T>
-cudaError_t launch_simt_gemm(const GemmArgs& a, int batch, cudaStream_t s) {
+cudaError_t launch_gemm_f32(const GemmArgs& a, int batch, cudaStream_t s) {
   const unsigned z = (unsigned)(batch * a.nsplit);
-  if (sizeof(T) == 4 && a.N <= kGemvTokens) {
+  if (a.N <= kGemvTokens) {
     auto go = [&](auto kern, int nt, int r) {
       const int rows = kGemvWarps * r, groups = (a.N + nt - 1) / nt;
       return launch_pdl(kern, dim3((unsigned)((a.M + rows - 1) / rows * groups), 1, z), dim3(kGemvWarps * 32),
@@ -383,7 +368,7 @@ cudaError_t launch_simt_gemm(const GemmArgs& a, int batch, cudaStream_t s) {
   // side by side on the SMs that have room, and the product takes two or three times as
   // long (pool of L = 16, k = 8, D = 1024, 8 heads of 64: 227-302 us at 32 tokens, by what
   // the kernels before it look like; 105 so; 257 and 137 at 64, 394 and 199 at 128).
-  return launch_pdl<false>(gemm_wxT_simt<T, T>, dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), dim3(256),
+  return launch_pdl<false>(gemm_wxT_simt, dim3((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, z), dim3(256),
                            0, s, a);
 }
 
@@ -686,8 +671,7 @@ __global__ void __launch_bounds__((COOP ? kCoopWarps : kTokenWarps) * 32, COOP ?
 // ---------------------------------------------------------------- mix (fp32)
 // One CTA per (token, branch, group of kChanGroup channels).  Thread t owns
 // the 8-element vectors t, t + 256 of D, so h, gains and the output move as
-// 16-byte vectors.  (bf16 takes it only where the driver has no TMA encoder.)
-template <typename T>
+// 16-byte vectors.
 __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
   extern __shared__ float sm[];  // alpha[kChanGroup][L], r[L]
   __shared__ float red[kMixThreads / 32][kChanGroup];
@@ -698,10 +682,10 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
   const int nj = min(kChanGroup, p.k - j0);
   const int kL = p.k * p.L;
   const int nvec = p.D / 8;
-  const T* hp = reinterpret_cast<const T*>(p.h) + (int64_t)b * p.L * p.D;
-  const T* g = reinterpret_cast<const T*>(p.pre_g[X]);
+  const float* hp = reinterpret_cast<const float*>(p.h) + (int64_t)b * p.L * p.D;
+  const float* g = reinterpret_cast<const float*>(p.pre_g[X]);
   pdl_wait();
-  const T* br = reinterpret_cast<const T*>(p.br[X]);
+  const float* br = reinterpret_cast<const float*>(p.br[X]);
   // alpha[j][l] = z[j*L + l] = bias + sum of the router's split partials
   for (int i = tid; i < nj * p.L; i += kMixThreads) {
     const int o = j0 * p.L + i;
@@ -719,7 +703,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
 #pragma unroll
   for (int v = 0; v < kVecPerThread; ++v) {
     const int vi = tid + v * kMixThreads;
-    if (vi < nvec) load8f<T>(g + vi * 8, gv[v]);
+    if (vi < nvec) load8f<float>(g + vi * 8, gv[v]);
 #pragma unroll
     for (int jj = 0; jj < kChanGroup; ++jj)
 #pragma unroll
@@ -736,7 +720,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
       const int vi = tid + v * kMixThreads;
       if (vi < nvec) {
         float hv[8];
-        load8f<T>(hp + (int64_t)l * p.D + vi * 8, hv);
+        load8f<float>(hp + (int64_t)l * p.D + vi * 8, hv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const float hh = hv[i] * r * gv[v][i];  // pre-mix RMSNorm with gain
@@ -766,22 +750,22 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
     for (int w = 0; w < kMixThreads / 32; ++w) t += red[w][jj];
     ss[jj] = rsqrtf(t / (float)p.D + p.eps_rms);
   }
-  T* xop = reinterpret_cast<T*>(p.xop);
+  float* xop = reinterpret_cast<float*>(p.xop);
 #pragma unroll
   for (int jj = 0; jj < kChanGroup; ++jj) {
     if (jj >= nj) break;
     const int j = j0 + jj;
-    const T* cg = reinterpret_cast<const T*>(p.ch_g[X]) + (int64_t)j * p.D;
-    T* xo = xop + (((int64_t)X * p.k + j) * p.B + b) * p.D;
+    const float* cg = reinterpret_cast<const float*>(p.ch_g[X]) + (int64_t)j * p.D;
+    float* xo = xop + (((int64_t)X * p.k + j) * p.B + b) * p.D;
 #pragma unroll
     for (int v = 0; v < kVecPerThread; ++v) {
       const int vi = tid + v * kMixThreads;
       if (vi < nvec) {
         float cv[8], o[8];
-        load8f<T>(cg + vi * 8, cv);
+        load8f<float>(cg + vi * 8, cv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[i] = acc[jj][v][i] * ss[jj] * cv[i];
-        store8f<T>(xo + vi * 8, o);
+        store8f<float>(xo + vi * 8, o);
       }
     }
   }
@@ -794,14 +778,14 @@ __global__ void __launch_bounds__(kMixThreads) mix_kernel(const MixParams p) {
 // own vectors of h through a private 2 x kMixLC-layer buffer in shared memory
 // with asynchronous copies, so many loads are in flight without holding
 // registers.
-template <typename T, int VPT>
+template <int VPT>
 __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams p, int tpt, int tb,
                                                                   int lc) {
   // alpha[tb][kMixCG][L], rl[tb][L], red[warps][kMixCG], then (16-byte
   // aligned) the h staging buffers [2][lc][VPT][threads] of one vector
   // (8 elements: VB 16-byte units) each; lc <= kMixLC layers per chunk
   extern __shared__ float sm[];
-  constexpr int VB = 8 * (int)sizeof(T) / 16;
+  constexpr int VB = 8 * (int)sizeof(float) / 16;
   const int X = blockIdx.y, j0 = blockIdx.z * kMixCG;
   const int nj = min(kMixCG, p.k - j0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -818,7 +802,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
   auto hslot = [&](int stage, int l, int v) -> uint4* {
     return hbuf + (((stage * lc + l) * VPT + v) * nth + tid) * VB;
   };
-  const T* hp = reinterpret_cast<const T*>(p.h) + (int64_t)b * L * p.D;
+  const float* hp = reinterpret_cast<const float*>(p.h) + (int64_t)b * L * p.D;
   // copies of layers [l0, l0 + lc) of this thread's vectors into `stage`
   auto stage_chunk = [&](int stage, int l0) {
     if (live)
@@ -837,7 +821,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
   pdl_wait();
   stage_chunk(0, 0);
   stage_chunk(1, lc);
-  const T* br = reinterpret_cast<const T*>(p.br[X]);
+  const float* br = reinterpret_cast<const float*>(p.br[X]);
   for (int i = tid; i < tb * nj * L; i += blockDim.x) {
     const int tt = i / (nj * L), rem = i % (nj * L);
     const int bb = b0 + tt, o = j0 * L + rem;
@@ -856,13 +840,13 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
   }
   __syncthreads();
 
-  const T* g = reinterpret_cast<const T*>(p.pre_g[X]);
+  const float* g = reinterpret_cast<const float*>(p.pre_g[X]);
   float gv[VPT][8];
   float acc[kMixCG][VPT][8];
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
     const int vi = u + v * tpt;
-    if (live && vi < nvec) load8f<T>(g + vi * 8, gv[v]);
+    if (live && vi < nvec) load8f<float>(g + vi * 8, gv[v]);
 #pragma unroll
     for (int jj = 0; jj < kMixCG; ++jj)
 #pragma unroll
@@ -883,7 +867,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
         const int vi = u + v * tpt;
         if (vi < nvec) {
           float hv[8];
-          load8f<T>(reinterpret_cast<const T*>(hslot(c & 1, l - l0, v)), hv);
+          load8f<float>(reinterpret_cast<const float*>(hslot(c & 1, l - l0, v)), hv);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float hh = hv[i] * r * gv[v][i];  // pre-mix RMSNorm with gain
@@ -911,7 +895,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
   __syncthreads();
   if (!live) return;
   const int w0 = t * (tpt / 32), nw = tpt / 32;
-  T* xop = reinterpret_cast<T*>(p.xop);
+  float* xop = reinterpret_cast<float*>(p.xop);
 #pragma unroll
   for (int jj = 0; jj < kMixCG; ++jj) {
     if (jj >= nj) break;
@@ -919,17 +903,17 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
     for (int w = 0; w < nw; ++w) q += red[(w0 + w) * kMixCG + jj];
     const float sc = rsqrtf(q / (float)p.D + p.eps_rms);
     const int j = j0 + jj;
-    const T* cg = reinterpret_cast<const T*>(p.ch_g[X]) + (int64_t)j * p.D;
-    T* xo = xop + (((int64_t)X * p.k + j) * p.B + b) * p.D;
+    const float* cg = reinterpret_cast<const float*>(p.ch_g[X]) + (int64_t)j * p.D;
+    float* xo = xop + (((int64_t)X * p.k + j) * p.B + b) * p.D;
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
       const int vi = u + v * tpt;
       if (vi < nvec) {
         float cv[8], o[8];
-        load8f<T>(cg + vi * 8, cv);
+        load8f<float>(cg + vi * 8, cv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) o[i] = acc[jj][v][i] * sc * cv[i];
-        store8f<T>(xo + vi * 8, o);
+        store8f<float>(xo + vi * 8, o);
       }
     }
   }
@@ -938,7 +922,7 @@ __global__ void __launch_bounds__(kMixThreads) mix_tokens_kernel(const MixParams
 // ---------------------------------------------------------------- epilogue
 // fp32 path: one CTA per (token, channel, branch), a warp per kv head; lane t
 // handles the RoPE pairs (i, i + HD/2) for i = t, t + 32, ...
-template <typename T, int HD>
+template <int HD>
 __global__ void __launch_bounds__(128) kv_epilogue_kernel(const MixParams p) {
   constexpr int HALF = HD / 2;
   constexpr int NP = (HALF + 31) / 32;
@@ -957,9 +941,9 @@ __global__ void __launch_bounds__(128) kv_epilogue_kernel(const MixParams p) {
   }
   const int nout = p.Hkv * HD;
   const float* src = p.proj + (((int64_t)X * p.k + j) * p.B + b) * nout;
-  T* pool = reinterpret_cast<T*>(X == 0 ? p.k_pool : p.v_pool);
+  float* pool = reinterpret_cast<float*>(X == 0 ? p.k_pool : p.v_pool);
   const int64_t base = (((int64_t)j * p.num_pages + pg) * p.Hkv) * p.P + (s & (p.P - 1));
-  const T* qg = reinterpret_cast<const T*>(p.qk_g) + (int64_t)j * HD;
+  const float* qg = reinterpret_cast<const float*>(p.qk_g) + (int64_t)j * HD;
   for (int hh = warp; hh < p.Hkv; hh += 4) {
     float y0[NP], y1[NP];
 #pragma unroll
@@ -986,13 +970,13 @@ __global__ void __launch_bounds__(128) kv_epilogue_kernel(const MixParams p) {
         }
       }
     }
-    T* dst = pool + (base + (int64_t)hh * p.P) * HD;
+    float* dst = pool + (base + (int64_t)hh * p.P) * HD;
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
       const int i = lane + 32 * t;
       if (i < HALF) {
-        dst[i] = Elem<T>::from_f(y0[t]);
-        dst[i + HALF] = Elem<T>::from_f(y1[t]);
+        dst[i] = Elem<float>::from_f(y0[t]);
+        dst[i + HALF] = Elem<float>::from_f(y1[t]);
       }
     }
   }
@@ -1025,26 +1009,53 @@ int mix_parts(int B, int L, int D, int sms) {
 }
 
 template <typename T>
-cudaError_t launch_all(MixParams& p, cudaStream_t s) {
-  const int kL = p.k * p.L;
-  const bool bf16 = sizeof(T) == 2;
-  const bool batched = bf16 ? mix_token_warps(p.B, p.L) : p.B >= kBatchedTokens;
-  cudaError_t e;
-  {
-    const int rows = p.B * p.L;
-    // as few warps to a row as hold it in registers, 1024 elements each
-    auto go = [&](auto kern, int wpr) {
-      const int per = kPrenormWarps / wpr;
-      return launch_pdl(kern, dim3((rows + per - 1) / per), dim3(kPrenormWarps * 32), 0, s, p);
-    };
-    e = p.D <= 1024   ? go(prenorm_kernel<T, 1>, 1)
-        : p.D <= 2048 ? go(prenorm_kernel<T, 2>, 2)
-                      : go(prenorm_kernel<T, 4>, 4);
-  }
+cudaError_t launch_prenorm(const MixParams& p, cudaStream_t s) {
+  const int rows = p.B * p.L;
+  // as few warps to a row as hold it in registers, 1024 elements each
+  auto go = [&](auto kern, int wpr) {
+    const int per = kPrenormWarps / wpr;
+    return launch_pdl(kern, dim3((rows + per - 1) / per), dim3(kPrenormWarps * 32), 0, s, p);
+  };
+  return p.D <= 1024   ? go(prenorm_kernel<T, 1>, 1)
+         : p.D <= 2048 ? go(prenorm_kernel<T, 2>, 2)
+                       : go(prenorm_kernel<T, 4>, 4);
+}
+
+cudaError_t launch_bf16(const MixParams& p, cudaStream_t s) {
+  if (!proj_tc_supported(p)) return cudaErrorInvalidValue;  // no TMA encoder
+  cudaError_t e = launch_prenorm<__nv_bfloat16>(p, s);
   if (e != cudaSuccess) return e;
-  if (bf16 && router_tc_supported(p.B)) {
-    e = p.B >= kRowsTokens ? launch_router_rows(p, p.sms, s) : launch_router_tc(p, s);
-  } else {
+  e = p.B >= kRowsTokens ? launch_router_rows(p, p.sms, s) : launch_router_tc(p, s);
+  if (e != cudaSuccess) return e;
+  {
+    const bool warps = mix_token_warps(p.B, p.L);
+    const int KS = (p.L + 15) / 16, nc = (p.D / 8 + 7) / 8;
+    const int csteps = (nc + p.mix_parts - 1) / p.mix_parts;
+    const size_t fr = (size_t)2 * KS * 3 * 512;
+    static size_t smem_set[6][kSmemOptDevices] = {};
+    const int v = KS <= 2 ? KS : 0;  // variant: layers kept in registers or not
+    const size_t smem = warps ? fr * kTokenWarps : fr + (size_t)kCoopWarps * 2 * 16 * sizeof(float);
+    auto kern = warps ? (v == 1   ? mix_mma_kernel<false, 1>
+                         : v == 2 ? mix_mma_kernel<false, 2>
+                                  : mix_mma_kernel<false, 0>)
+                      : (v == 1   ? mix_mma_kernel<true, 1>
+                         : v == 2 ? mix_mma_kernel<true, 2>
+                                  : mix_mma_kernel<true, 0>);
+    e = opt_in_smem(kern, smem, smem_set[3 * warps + v]);
+    if (e != cudaSuccess) return e;
+    const int units = p.B * p.mix_parts;
+    e = launch_pdl(kern, dim3(warps ? (units + kTokenWarps - 1) / kTokenWarps : units),
+                   dim3((warps ? kTokenWarps : kCoopWarps) * 32), smem, s, p, KS, csteps);
+    if (e != cudaSuccess) return e;
+  }
+  // tensor-core projection, QK-norm, RoPE and cache write in one kernel
+  return proj_rows_supported(p) ? launch_proj_rows(p, p.sms, s) : launch_proj_tc(p, s);
+}
+
+cudaError_t launch_f32(const MixParams& p, cudaStream_t s) {
+  cudaError_t e = launch_prenorm<float>(p, s);
+  if (e != cudaSuccess) return e;
+  {
     GemmArgs a{};
     a.W[0] = p.Wr[0];
     a.W[1] = p.Wr[1];
@@ -1053,63 +1064,38 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
     a.X = p.xi;
     a.x_stride = (int64_t)p.B * p.Lp * p.D;
     a.out = p.zpart;
-    a.M = kL;
+    a.M = p.k * p.L;
     a.N = p.B;
     a.K = p.Lp * p.D;
     a.nsplit = p.nsplit_r;
     a.k_per_split = ((a.K + p.nsplit_r - 1) / p.nsplit_r + BK - 1) / BK * BK;
-    e = launch_simt_gemm<T>(a, 2, s);
+    e = launch_gemm_f32(a, 2, s);
+    if (e != cudaSuccess) return e;
   }
-  if (e != cudaSuccess) return e;
-  const bool tc_proj = bf16 && proj_tc_supported(p);
-  if (tc_proj) {
-    const int KS = (p.L + 15) / 16, nc = (p.D / 8 + 7) / 8;
-    const int csteps = (nc + p.mix_parts - 1) / p.mix_parts;
-    const size_t fr = (size_t)2 * KS * 3 * 512;
-    static size_t smem_set[6][kSmemOptDevices] = {};
-    const int v = KS <= 2 ? KS : 0;  // variant: layers kept in registers or not
-    const size_t smem = batched ? fr * kTokenWarps : fr + (size_t)kCoopWarps * 2 * 16 * sizeof(float);
-    auto kern = batched ? (v == 1   ? mix_mma_kernel<false, 1>
-                           : v == 2 ? mix_mma_kernel<false, 2>
-                                    : mix_mma_kernel<false, 0>)
-                        : (v == 1   ? mix_mma_kernel<true, 1>
-                           : v == 2 ? mix_mma_kernel<true, 2>
-                                    : mix_mma_kernel<true, 0>);
-    e = opt_in_smem(kern, smem, smem_set[3 * batched + v]);
-    if (e != cudaSuccess) return e;
-    const int units = p.B * p.mix_parts;
-    e = launch_pdl(kern, dim3(batched ? (units + kTokenWarps - 1) / kTokenWarps : units),
-                   dim3((batched ? kTokenWarps : kCoopWarps) * 32), smem, s, p, KS, csteps);
-    if (e != cudaSuccess) return e;
-  } else if (batched) {
+  if (p.B >= kBatchedTokens) {
     const int nvec = p.D / 8;
     const bool two = nvec > kMixThreads;  // D > 2048: two vectors per thread
     const int per = two ? (nvec + 1) / 2 : nvec;
     const int tpt = (per + 31) / 32 * 32;
     const int tb = tpt >= kMixThreads ? 1 : kMixThreads / tpt;
-    const size_t per_layer = (size_t)2 * (two ? 2 : 1) * tb * tpt * 8 * sizeof(T);  // both stages
+    const size_t per_layer = (size_t)2 * (two ? 2 : 1) * tb * tpt * 8 * sizeof(float);  // both stages
     int lc = kMixLC;
     while (lc > 1 && (size_t)lc * per_layer > kMixStageBudget) lc /= 2;
     const size_t smem = sizeof(float) * ((size_t)tb * kMixCG * p.L + (size_t)tb * p.L +
                                          (size_t)(tb * tpt / 32) * kMixCG) +
                         16 + (size_t)lc * per_layer;
     dim3 grid((p.B + tb - 1) / tb, 2, (p.k + kMixCG - 1) / kMixCG);
-    auto kern = two ? mix_tokens_kernel<T, 2> : mix_tokens_kernel<T, 1>;
+    auto kern = two ? mix_tokens_kernel<2> : mix_tokens_kernel<1>;
     static size_t smem_set[2][kSmemOptDevices] = {};  // per variant and device
     e = opt_in_smem(kern, smem, smem_set[two]);
     if (e != cudaSuccess) return e;
     e = launch_pdl(kern, grid, dim3(tb * tpt), smem, s, p, tpt, tb, lc);
-    if (e != cudaSuccess) return e;
   } else {
     const size_t smem = sizeof(float) * (kChanGroup * p.L + p.L);
     dim3 grid(p.B, 2, (p.k + kChanGroup - 1) / kChanGroup);
-    e = launch_pdl(mix_kernel<T>, grid, dim3(kMixThreads), smem, s, p);
-    if (e != cudaSuccess) return e;
+    e = launch_pdl(mix_kernel, grid, dim3(kMixThreads), smem, s, p);
   }
-  if (tc_proj) {
-    // tensor-core projection, QK-norm, RoPE and cache write in one kernel
-    return proj_rows_supported(p) ? launch_proj_rows(p, p.sms, s) : launch_proj_tc(p, s);
-  }
+  if (e != cudaSuccess) return e;
   {
     GemmArgs a{};
     a.W[0] = p.Wkv[0];
@@ -1124,15 +1110,13 @@ cudaError_t launch_all(MixParams& p, cudaStream_t s) {
     a.K = p.D;
     a.nsplit = 1;
     a.k_per_split = p.D;
-    e = launch_simt_gemm<T>(a, 2 * p.k, s);
+    e = launch_gemm_f32(a, 2 * p.k, s);
     if (e != cudaSuccess) return e;
   }
-  {
-    dim3 grid(p.B, p.k, 2);
-    if (p.d == 64) return launch_pdl(kv_epilogue_kernel<T, 64>, grid, dim3(128), 0, s, p);
-    if (p.d == 96) return launch_pdl(kv_epilogue_kernel<T, 96>, grid, dim3(128), 0, s, p);
-    return launch_pdl(kv_epilogue_kernel<T, 128>, grid, dim3(128), 0, s, p);
-  }
+  dim3 grid(p.B, p.k, 2);
+  if (p.d == 64) return launch_pdl(kv_epilogue_kernel<64>, grid, dim3(128), 0, s, p);
+  if (p.d == 96) return launch_pdl(kv_epilogue_kernel<96>, grid, dim3(128), 0, s, p);
+  return launch_pdl(kv_epilogue_kernel<128>, grid, dim3(128), 0, s, p);
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -1145,9 +1129,9 @@ MixWorkspace mix_workspace_layout(const wm_config& cfg, int32_t B, int sm_count)
   const int kL = cfg.k * cfg.L;
   const int64_t Kr = (int64_t)Lp * cfg.D;
   int ns;
-  if (cfg.dtype == WM_DT_BF16 && router_tc_supported(B)) {
+  if (cfg.dtype == WM_DT_BF16) {
     ns = B >= kRowsTokens ? router_rows_splits(cfg.k, cfg.L, Lp, cfg.D, B, sm_count)
-                          : router_tc_splits(cfg.k, cfg.L, Lp, cfg.D, B, sm_count);
+                          : router_tc_splits(cfg.k, cfg.L, Lp, cfg.D, sm_count);
   } else {
     const int tiles = 2 * ((kL + BM - 1) / BM) * ((B + BN - 1) / BN);
     ns = (2 * sm_count + tiles - 1) / tiles;
@@ -1183,8 +1167,7 @@ cudaError_t launch_kv_mix(MixParams& p, int dtype, int sms, cudaStream_t s) {
   // bf16: [2][k][parts][B] floats, within the fp32 path's [2][k][B][Hkv*d] projection outputs
   if (p.mix_parts > p.Hkv * p.d) return cudaErrorInvalidConfiguration;  // (16 parts, 64 outputs)
   p.ssq = p.proj;
-  if (dtype == WM_DT_F32) return launch_all<float>(p, s);
-  return launch_all<__nv_bfloat16>(p, s);
+  return dtype == WM_DT_F32 ? launch_f32(p, s) : launch_bf16(p, s);
 }
 
 }  // namespace wm

@@ -60,8 +60,9 @@ struct ProjTcParams {
 
 // MODE kEpiKV: grid (ceil(Hkv/hpt), k, 2*ntiles) = (head tile, channel j, branch X + 2*token
 // tile), hpt = 128/HD.
-// MODE kEpiPartial: grid (ceil(kL/128), nsplit, 2*ntiles) = (row tile, split, branch X + 2*token
-// tile).  A token tile is BN <= 256 tokens.
+// MODE kEpiPartial: grid (ceil(kL/128), nsplit, 2) = (row tile, split, branch X).  A token tile
+// is BN <= 256 tokens; from kRowsTokens on only the projection comes here, where the
+// key-norm gain is not 16-byte aligned.
 template <int HD, int MODE>
 __global__ void __launch_bounds__(kTcThreads, 1)
     proj_tc_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
@@ -295,17 +296,13 @@ bool proj_tc_supported(const MixParams& mp) {
   return (mp.d == 64 || mp.d == 96 || mp.d == 128) && mp.B >= 1 && tma_available();
 }
 
-bool router_tc_supported(int B) { return B >= 1; }
-
-int router_tc_splits(int k, int L, int Lp, int D, int B, int sms) {
+int router_tc_splits(int k, int L, int Lp, int D, int sms) {
   const int nk = (Lp * D + kTcBK - 1) / kTcBK;
-  const int ntiles = (B + token_tile(B) - 1) / token_tile(B);
-  const int tiles = 2 * ((k * L + kTcM - 1) / kTcM) * ntiles;
+  const int tiles = 2 * ((k * L + kTcM - 1) / kTcM);  // (fewer than kRowsTokens tokens: one tile of them)
   int ns = (sms + tiles - 1) / tiles;
   const int max_ns = nk / 8 > 1 ? nk / 8 : 1;  // at least 8 k-blocks per split
   ns = ns < 1 ? 1 : (ns > max_ns ? max_ns : ns);
   const int per = (nk + ns - 1) / ns;
-  (void)B;
   return (nk + per - 1) / per;
 }
 
@@ -375,7 +372,7 @@ cudaError_t launch_router_tc(const MixParams& mp, cudaStream_t s) {
     if (!encode_kmajor(&tmW[X], mp.Wr[X], (uint64_t)kL, K, kTcM)) return cudaErrorInvalidValue;
   if (!encode_kmajor(&tmX, mp.xi, (uint64_t)2 * mp.B, K, (uint32_t)p.BN))
     return cudaErrorInvalidValue;
-  dim3 grid((kL + kTcM - 1) / kTcM, mp.nsplit_r, 2 * ((mp.B + p.BN - 1) / p.BN));
+  dim3 grid((kL + kTcM - 1) / kTcM, mp.nsplit_r, 2);
   p.stages = pick_stages(p.kb_per_split, p.BN, (int64_t)grid.x * grid.y * grid.z, mp.sms, 0);
   const size_t smem = tc_smem(p.stages, p.BN);
   return launch_mode<64, kEpiPartial>(grid, smem, tmW[0], tmW[1], tmX, p, s);
