@@ -36,11 +36,14 @@
 //    reads its S row from TMEM, applies the causal mask slot <= pos (on tiles
 //    the diagonal crosses), and writes the bf16 probabilities back over the S
 //    columns it has read, where P V takes them as its A operand, each half as
-//    it is ready.  The running max is raised only when it grows by more than
-//    2^8: only then is the row of O in TMEM rescaled; in between the
-//    probabilities stay below 2^8, and the final O / l is exact either way.
-//    So the probabilities are computed with the max of the tiles before, and
-//    computed again in the rare step that raises it.
+//    it is ready.  The running max is raised, and the row of O in TMEM
+//    rescaled, only when the tile's second half holds a score more than 2^8
+//    above it or the first half's 64 probabilities sum to more than 2^14 (a
+//    sum that is there anyway, where a max would have to be taken first).  So
+//    probabilities of up to 2^14 (first half) and 2^8 (second) are used as they
+//    are: fp32 sums and bf16 operands have the same relative precision
+//    there, and O / l needs no correction.  They are computed with the max of the
+//    tiles before, and computed again in the rare step that raises it.
 // Slots beyond the item's largest position may hold anything (unwritten
 // cache); their V rows are zeroed in shared memory before P V, and masked
 // scores are replaced, never multiplied, so no NaN there reaches the output.

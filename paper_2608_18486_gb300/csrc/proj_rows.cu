@@ -474,8 +474,15 @@ cudaError_t launch_kv(const MixParams& mp, int sms, cudaStream_t s) {
 
 }  // namespace
 
-// From this many tokens on the pool's contractions take the tokens as MMA rows:
-// below, the decode form (proj_tc.cu) pads fewer rows of its 16-token granularity.
+// From kRowsTokens (128: a whole tile) on the pool's contractions take the tokens as
+// MMA rows: below, the decode form (proj_tc.cu) pads fewer rows of its 16-token
+// granularity, above, its accumulators and epilogue grow with the tokens of a CTA.
+// Whole pools (us, decode form / this one) at 64, 96, 128 and 256 tokens: L = k = 16, D =
+// 512, 3 heads of 96: 23.0 / 25.2, 25.7 / 25.7, 29.3 / 28.6, 39.0 / 30.1; L = k = 16, D =
+// 1024, 8 heads of 128: 32.0 / 34.0, 37.9 / 36.5, 62.5 / 39.6, 76.6 / 51.7; L = 32, k =
+// 4, D = 2048, 8 heads of 128: 40.7 / 43.2, 50.6 / 51.5, 57.6 / 56.4, 90.0 / 77.7 (160:
+// 67.0 / 69.2); L = 32, k = 16, D = 4096, 32 heads of 128: 239 / 250, 281 / 267, 361 /
+// 287, 563 / 408.
 bool proj_rows_supported(const MixParams& mp) {
   return mp.B >= kRowsTokens && (reinterpret_cast<uintptr_t>(mp.qk_g) % 16) == 0;
 }

@@ -14,7 +14,7 @@
 // tile covers whole heads (two of d=64, one of d=96 or 128; rows past the
 // last head are computed and ignored).  The work is
 // weight-streaming bound; TMA brings 128x64 weight tiles and Nx64 token
-// tiles (128-byte swizzle) through a 4-stage mbarrier pipeline.  Warp 0 lane
+// tiles (128-byte swizzle) through an mbarrier ring (pick_stages).  Warp 0 lane
 // 0 issues TMA, warp 1 lane 0 issues tcgen05.mma, warps 2-7 fetch what the
 // epilogue needs; all eight warps drain TMEM (warps w and w + 4 share the
 // 32-lane quadrant w % 4) into shared memory, then finish the per-(token,
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       tc::tma_load_2d(Bs + s * b_bytes, &tmX, (kb0 + kb) * kTcBK, xrow, &full[s]);
     }
   } else if (MODE == kEpiKV && warp >= 2) {
-    // meanwhile warps 2-3 fetch what the epilogue needs: the RoPE table of the
+    // meanwhile warps 2-7 fetch what the epilogue needs: the RoPE table of the
     // tile's tokens and each token's destination slot and page
     const int t2 = threadIdx.x - 64, n2 = kTcThreads - 64;
     if (p.rope_smem_off > 0)
