@@ -819,40 +819,15 @@ __global__ void __launch_bounds__(kPThreads, 1)
       const int rr = lane >> 2, ch = lane & 3;  // row (of 8) and 16-byte chunk this lane stores
       const int64_t pitch = (int64_t)p.Hq * HD;
       __nv_bfloat16* drow = dst + rr * pitch + 8 * ch;
-      // Columns 32 c0 .. 32 c1: all of the row, or (HALVES) this half's share, the
-      // first tile's the smaller one.
       constexpr int NC = HD / 32;
-      const int c0 = HALVES && i == 1 ? NC / 2 : 0, c1 = HALVES && i == 0 ? NC / 2 : NC;
-      const uint32_t ocol1 = lane_base + 256 + 128 * (i ^ 1);
-      uint32_t o[2][32];  // one group of 32 columns on its way while the last is stored
-      tc::tmem_ld32(ocol + 32 * c0, o[0]);
-#pragma unroll
-      for (int cc = 0; cc < (HALVES ? NC - NC / 2 : NC); ++cc) {
-        const int c = c0 + cc;
-        if (HALVES && c >= c1) break;
-        tc::tmem_ld_wait();
-        if constexpr (HALVES) {
-          uint32_t o1[32];
-          tc::tmem_ld32(ocol1 + 32 * c, o1);
-          tc::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            o[cc & 1][e] = __float_as_uint((own ? __uint_as_float(o[cc & 1][e]) * inv : 0.f) +
-                                           (other ? __uint_as_float(o1[e]) * inv1 : 0.f));
-        }
-        if (c + 1 < c1) tc::tmem_ld32(ocol + 32 * (c + 1), o[(cc + 1) & 1]);
+      // 32 columns of the rows: staged, and stored
+      auto store_cols = [&](int c, auto x) {
 #pragma unroll
         for (int e = 0; e < 32; e += 8) {
           uint32_t u[4];
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
-            float x0 = __uint_as_float(o[cc & 1][e + 2 * t]);
-            float x1 = __uint_as_float(o[cc & 1][e + 2 * t + 1]);
-            if (!HALVES) {
-              x0 = own ? x0 * inv : 0.f;
-              x1 = own ? x1 * inv : 0.f;
-            }
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(x(e + 2 * t), x(e + 2 * t + 1));
             u[t] = *reinterpret_cast<const uint32_t*>(&h2);
           }
           // row `lane`, 16-byte chunk e/8, placed so that 8 rows cover all banks
@@ -870,6 +845,35 @@ __global__ void __launch_bounds__(kPThreads, 1)
         for (int q = 0; q < 4; ++q)
           if (rb + q * 8 + rr < p.Tq)
             *reinterpret_cast<uint4*>(drow + q * 8 * pitch + 32 * c) = u[q];
+      };
+      if constexpr (HALVES) {
+        // This half's share of the columns, the first one's the smaller.  Not unrolled:
+        // such launches are short, a CTA runs this once or twice, and its instructions
+        // are fetched meanwhile (us, unrolled / so: one prompt of 40, 12 heads of 96: 7.6 /
+        // 6.8; seven of 197, 4/2 heads of 96: 8.7 / 7.4; one of 2593, 8/2 heads of 96: 24.0 /
+        // 22.6; one of 40, 8 heads of 128: 7.9 / 7.0; of 64 the same).
+        const int c0 = i == 1 ? NC / 2 : 0, c1 = i == 0 ? NC / 2 : NC;
+#pragma unroll 1
+        for (int cc = 0; cc < NC - NC / 2; ++cc) {
+          const int c = c0 + cc;
+          if (NC % 2 != 0 && c >= c1) break;
+          uint32_t o[32], o1[32];
+          tc::tmem_ld32(ocol + 32 * c, o);
+          tc::tmem_ld32(lane_base + 256 + 128 * (i ^ 1) + 32 * c, o1);
+          tc::tmem_ld_wait();
+          store_cols(c, [&](int e) {
+            return (own ? __uint_as_float(o[e]) * inv : 0.f) + (other ? __uint_as_float(o1[e]) * inv1 : 0.f);
+          });
+        }
+      } else {
+        uint32_t o[2][32];  // one group of 32 columns on its way while the last is stored
+        tc::tmem_ld32(ocol, o[0]);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          tc::tmem_ld_wait();
+          if (c + 1 < NC) tc::tmem_ld32(ocol + 32 * (c + 1), o[(c + 1) & 1]);
+          store_cols(c, [&](int e) { return own ? __uint_as_float(o[c & 1][e]) * inv : 0.f; });
+        }
       }
       tc::fence_before_sync();
       if (HALVES) {  // the next item's O and sums go over these: not before the other half has read them
