@@ -926,8 +926,11 @@ cudaError_t launch_hd(const CUtensorMap& q, const CUtensorMap& k, const CUtensor
 // 4575 positions 50 / 30; 0.26: 32/8 heads of 96, every eighth of 4096 48 / 36;
 // 0.32: two prompts, 32/8 heads of 64, every fourth of 1000 16.5 / 12; 0.47: sixteen
 // prompts, 6/3 heads of 96, every eighth of 2048 29.8 / 32.5; 0.53: two prompts of
-// the 0.26 case 48.5 / 66.6 (with many CTAs the doubled K and V loads bind).
+// the 0.26 case 48.5 / 66.6 (with many CTAs the doubled K and V loads bind).  A
+// sequence that has room for one KV tile only has nothing to share: one prompt of 40, 12
+// heads of 64 / 96 / 128: 5.7 / 6.3 / 6.5 as whole tiles, 5.9 / 6.8 / 7.0 as halves.
 bool halves_pay(const PrefillLaunch& L, int pair, int sms) {
+  if ((int64_t)L.max_pages * L.P <= kPN) return false;
   const int rows_item = pair ? kPM : kQT * kPM;
   const double nblk = (L.Tq + rows_item - 1) / rows_item;
   const double items = nblk * (pair ? L.Hq / kQT : L.Hq) * L.B;
