@@ -17,15 +17,15 @@ int attn_unit_warps_per_cta(int stage_bytes, int G) {
 }
 
 // ring bytes of one stage of K and V
-static size_t ring_stage_bytes(int stage_bytes, int dtype, int d, int G) {
+static size_t ring_stage_bytes(int stage_bytes, int dtype, int d, bool mma) {
   const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
   return 2 * (size_t)attn_stage_slots(stage_bytes, dtype, d) * d * esz +
-         (attn_uses_mma(dtype, d, G) ? kAttnMmaPad : 0);
+         (mma ? kAttnMmaPad : 0);
 }
 
 size_t attn_smem_bytes(int stage_bytes, int dtype, int d, int G, int B) {
   const size_t esz = dtype == WM_DT_F32 ? 4 : 2;
-  const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, G);
+  const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, attn_uses_mma(dtype, d, G));
   return (size_t)attn_detail::kWarps * attn_detail::kWStages * stage +
          (attn_uses_mma(dtype, d, G) ? 0 : (size_t)attn_detail::kWarps * attn_detail::kWStages * G * d * esz) +
          sizeof(int) * (2 * (size_t)B + 1);
@@ -39,7 +39,8 @@ cudaError_t launch_decode_attn(const AttnParams& p, int stage_bytes, int dtype, 
 }
 
 size_t attn_unit_smem_bytes(int stage_bytes, int dtype, int d, int G, int warps) {
-  const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, G);
+  const bool mma = attn_uses_mma(dtype, d, G) || attn_unit_either(dtype, d, G);
+  const size_t stage = ring_stage_bytes(stage_bytes, dtype, d, mma);
   return (size_t)warps * attn_unit_detail::kUStages * stage +
          (size_t)(attn_unit_detail::unit_rec(G, d) + 3) / 4 * 4 * sizeof(float);
 }

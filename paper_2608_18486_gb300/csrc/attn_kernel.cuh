@@ -304,9 +304,10 @@ template <typename T, int HD, int G, int SB>
 struct MathPick<T, HD, G, SB, true> {
   using type = MmaMath<HD, G, Shape<T, HD, SB>::STAGE_SLOTS>;
 };
+template <typename T>
+constexpr int kDtype = sizeof(T) == 2 ? WM_DT_BF16 : WM_DT_F32;
 template <typename T, int HD, int G, int SB>
-using MathOf =
-    typename MathPick<T, HD, G, SB, attn_uses_mma(sizeof(T) == 2 ? WM_DT_BF16 : WM_DT_F32, HD, G)>::type;
+using MathOf = typename MathPick<T, HD, G, SB, attn_uses_mma(kDtype<T>, HD, G)>::type;
 
 // Slots per bulk copy of K and of V (a copy never crosses a page), and the
 // place of slot `ls` in the V tile: whole stages where the tile is

@@ -26,7 +26,8 @@ namespace attn_unit_detail {
 
 namespace cg = cooperative_groups;
 using attn_detail::CopyShape;
-using attn_detail::MathOf;
+using attn_detail::kDtype;
+using attn_detail::MathPick;
 using attn_detail::Shape;
 
 constexpr int kUStages = 3;  // ring depth per warp
@@ -45,10 +46,11 @@ constexpr int unit_min_blocks(int nw, int g, int d) { return nw > 4 ? 1 : g > 2 
 // per query head (log2 units)
 constexpr int unit_rec(int G, int HD) { return G * HD + 2 * G; }
 
-template <typename T, int HD, int G, int SB, int NW>
+// MMA: stage math on the tensor cores (attn_unit_mma)
+template <typename T, int HD, int G, int SB, int NW, bool MMA>
 __global__ void __launch_bounds__(NW * 32, unit_min_blocks(NW, G, HD)) decode_attn_unit_kernel(const AttnParams p) {
   using SH = Shape<T, HD, SB>;
-  using MATH = MathOf<T, HD, G, SB>;
+  using MATH = typename MathPick<T, HD, G, SB, MMA>::type;
   constexpr int STAGE_SLOTS = SH::STAGE_SLOTS;
   constexpr int K_ELEMS = SH::STAGE_ELEMS;             // of K in the ring
   constexpr int RING_ELEMS = 2 * K_ELEMS + MATH::kPad;  // of K and V
@@ -249,11 +251,11 @@ __global__ void __launch_bounds__(NW * 32, unit_min_blocks(NW, G, HD)) decode_at
   cluster.sync();
 }
 
-template <typename T, int HD, int G, int SB, int NW>
+template <typename T, int HD, int G, int SB, int NW, bool MMA = attn_uses_mma(kDtype<T>, HD, G)>
 inline cudaError_t launch_unit_t(const AttnParams& p, int units, int cluster, size_t smem,
                                  cudaStream_t stream) {
   static size_t smem_set[kSmemOptDevices] = {};
-  auto kern = decode_attn_unit_kernel<T, HD, G, SB, NW>;
+  auto kern = decode_attn_unit_kernel<T, HD, G, SB, NW, MMA>;
   if (cudaError_t e = opt_in_smem(kern, smem, smem_set); e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)units * (unsigned)cluster);
@@ -273,9 +275,9 @@ inline cudaError_t launch_unit_t(const AttnParams& p, int units, int cluster, si
 }
 
 // Clusters of `cluster` CTAs that can be resident at once (0: unknown).
-template <typename T, int HD, int G, int SB, int NW>
+template <typename T, int HD, int G, int SB, int NW, bool MMA = attn_uses_mma(kDtype<T>, HD, G)>
 inline int max_clusters_t(int cluster, size_t smem) {
-  auto kern = decode_attn_unit_kernel<T, HD, G, SB, NW>;
+  auto kern = decode_attn_unit_kernel<T, HD, G, SB, NW, MMA>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -304,7 +306,14 @@ inline int max_clusters_g(int G, int warps, int cluster, size_t smem) {
   if (warps != 4 && warps != 8) return 0;
   switch (G) {
     case 1: return warps == 4 ? max_clusters_t<T, HD, 1, SB, 4>(cluster, smem) : 0;
-    case 2: return warps == 4 ? max_clusters_t<T, HD, 2, SB, 4>(cluster, smem) : 0;
+    case 2:
+      if (warps != 4) return 0;
+      if constexpr (attn_unit_either(kDtype<T>, HD, 2)) {  // as many as fit either way
+        const int a = max_clusters_t<T, HD, 2, SB, 4>(cluster, smem);
+        const int b = max_clusters_t<T, HD, 2, SB, 4, true>(cluster, smem);
+        return a < b ? a : b;
+      }
+      return max_clusters_t<T, HD, 2, SB, 4>(cluster, smem);
     case 4:
       if constexpr (sizeof(T) == 2)
         if (warps == 4) return max_clusters_t<T, HD, 4, SB, 4>(cluster, smem);
@@ -323,7 +332,11 @@ inline cudaError_t launch_unit_g(const AttnParams& p, int G, int warps, int unit
   if (warps != 4 && warps != 8) return cudaErrorInvalidValue;
   switch (G) {
     case 1: return warps == 4 ? launch_unit_t<T, HD, 1, SB, 4>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
-    case 2: return warps == 4 ? launch_unit_t<T, HD, 2, SB, 4>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
+    case 2:
+      if constexpr (attn_unit_either(kDtype<T>, HD, 2))
+        if (warps == 4 && attn_unit_mma(kDtype<T>, HD, 2, p.P, (int64_t)p.max_pages * p.P))
+          return launch_unit_t<T, HD, 2, SB, 4, true>(p, units, cluster, smem, s);
+      return warps == 4 ? launch_unit_t<T, HD, 2, SB, 4>(p, units, cluster, smem, s) : cudaErrorInvalidValue;
     case 4:
       if constexpr (sizeof(T) == 2)
         if (warps == 4) return launch_unit_t<T, HD, 4, SB, 4>(p, units, cluster, smem, s);

@@ -61,14 +61,13 @@ constexpr int attn_ctas_per_sm(int stage_bytes, int G) { return stage_bytes == 4
 constexpr int attn_part_rec(int G, int d) { return G * d + (2 * G + 1 + 3) / 4 * 4; }
 
 // Launches whose stage math runs on the tensor cores (attn_mma.cuh): bf16
-// with four or eight query heads per kv head, or two of 64 or 96.  Two heads of
-// 128 stay on the CUDA cores, which were faster there with the 8 warps per SM that
-// its stages leave room for (step of 8 layers, 4 ragged sequences up to 4096, 16/8
-// heads: 115 us, 127 on the tensor cores; of 64, 16 sequences of 2048, 12/6 heads:
-// 123 and 120; of 96, 6/3 heads, 16 layers: 185 and 173).  A stage of theirs is kAttnMmaPad bytes longer in shared
-// memory.
+// with four or eight query heads per kv head, or two of 96 (69 launches in 0.92 of
+// the time on the CUDA cores).  Two of 128 were faster on the CUDA cores, with the 8 warps
+// per SM that its stages leave room for (step of 8 layers, 4 ragged sequences up to 4096,
+// 16/8 heads: 115 us, 127 on the tensor cores).  Two of 64: see attn_unit_mma.  A stage of
+// theirs is kAttnMmaPad bytes longer in shared memory.
 constexpr bool attn_uses_mma(int dtype, int d, int G) {
-  return dtype == WM_DT_BF16 && (G >= 4 || (G == 2 && d <= 96));
+  return dtype == WM_DT_BF16 && (G >= 4 || (G == 2 && d == 96));
 }
 constexpr int kAttnMmaPad = 64;
 
@@ -81,6 +80,16 @@ cudaError_t launch_decode_attn(const AttnParams& p, int stage_bytes, int dtype, 
 // (sequence, kv head) unit, `units` = B * Hkv clusters.
 constexpr int kAttnUnitMaxCluster = 8;
 int attn_unit_warps_per_cta(int stage_bytes, int G);  // 0: unsupported
+// ... and of the unit split; its two query heads of 64 can run either way: V in two
+// copies per stage (pages of more than 16 slots) costs what the tensor cores gain, so
+// only where pages are that small or the units short.  (us, CUDA cores / tensor cores: six
+// sequences of 162, 16 kv heads 5.4 / 5.0; three of up to 3687, 8, pages of 16: 8.9 / 8.6;
+// nine of up to 4811, 4, pages of 64: 10.1 / 10.6; on stream-K 83 of up to 2776, 32: 218 /
+// 229, and 34 of 617, 12: 18.4 / 19.3.)
+constexpr bool attn_unit_either(int dtype, int d, int G) { return dtype == WM_DT_BF16 && d == 64 && G == 2; }
+constexpr bool attn_unit_mma(int dtype, int d, int G, int page, int64_t max_slots) {
+  return attn_uses_mma(dtype, d, G) || (attn_unit_either(dtype, d, G) && (page <= 16 || max_slots <= 2048));
+}
 size_t attn_unit_smem_bytes(int stage_bytes, int dtype, int d, int G, int warps);
 int attn_unit_max_clusters(int stage_bytes, int dtype, int d, int G, int warps, int cluster);
 cudaError_t launch_decode_attn_unit(const AttnParams& p, int stage_bytes, int dtype, int d, int G,
