@@ -397,7 +397,7 @@ cudaError_t launch_gemm_f32(const GemmArgs& a, int batch, cudaStream_t s) {
 //
 // Bound by memory: h in, the operand out (201 MB at 4096 tokens, L = k = 16, D =
 // 512).  There the scalar kernel before took 194 us, this one 59; at 32
-// tokens, L = 32, k = 16, D = 4096: 40 and 20 (cold caches).
+// tokens, L = 32, k = 16, D = 4096: 40 and 18 (cold caches).
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
       "{%8, %9}, {%0, %1, %2, %3};"

@@ -53,8 +53,8 @@
 // where the matrix products alone take 2048 and the 32768 exponentials 2048.
 // One launch at 32 heads of 128, two prompts of 8192 positions: 939 us before
 // (one item per CTA; every descriptor moved to uniform registers one by one,
-// 90 cycles per MMA; 16-byte row stores at the end), 738 us now; 6/3 heads of
-// 96, sixteen prompts of 2048: 126 and 78 us.
+// 90 cycles per MMA; 16-byte row stores at the end), 717 us now (655 replayed from a
+// graph); 6/3 heads of 96, sixteen prompts of 2048: 126 and 75.5 us.
 #include <limits.h>
 #include <math.h>
 
