@@ -487,13 +487,13 @@ __global__ void __launch_bounds__((COOP ? kCoopWarps : kTokenWarps) * 32, COOP ?
     }
   };
 
-  for (int mt = 0; mt * 16 < p.k; ++mt) {
+  for (int mt = blockIdx.y; mt * 16 < p.k; mt += gridDim.y) {
     uint4 hn[KB][4];
     if (KSR > 0)
 #pragma unroll
       for (int ks = 0; ks < KB; ++ks) load_h(c0, ks, hn[ks]);
     if (COOP) {
-      if (mt > 0) __syncthreads();
+      if (mt > (int)blockIdx.y) __syncthreads();
       // the layer pairs and channels there are; the rest of the operand is 0
       const int npair = (L + 1) / 2, nch = min(16, p.k - mt * 16);
       if (npair < KS * 8 || nch < 16) {
@@ -1043,8 +1043,14 @@ cudaError_t launch_bf16(const MixParams& p, cudaStream_t s) {
                                   : mix_mma_kernel<true, 0>);
     e = opt_in_smem(kern, smem, smem_set[3 * warps + v]);
     if (e != cudaSuccess) return e;
-    const int units = p.B * p.mix_parts;
-    e = launch_pdl(kern, dim3(warps ? (units + kTokenWarps - 1) / kTokenWarps : units),
+    const int units = p.B * p.mix_parts, groups = (p.k + 15) / 16;
+    // Few units: their groups of 16 channels, which share nothing but the reads of h, side
+    // by side, as far as two CTAs fit each SM (pools, us, one after another / so: 33 layers
+    // and channels, D = 512, 3 heads of 96, 16 tokens: 42.5 / 29.3; 28, D = 264, 8 tokens:
+    // 31.0 / 23.1; 128, D = 264, 2 tokens: 313 / 200; 100 tokens of 24, D = 1024: the same).
+    int side = warps ? 1 : 2 * p.sms / units;
+    side = side < 1 ? 1 : (side < groups ? side : groups);
+    e = launch_pdl(kern, dim3(warps ? (units + kTokenWarps - 1) / kTokenWarps : units, side),
                    dim3((warps ? kTokenWarps : kCoopWarps) * 32), smem, s, p, KS, csteps);
     if (e != cudaSuccess) return e;
   }
